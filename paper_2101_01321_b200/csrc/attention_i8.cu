@@ -218,7 +218,7 @@ attention_coarse_kernel(const __grid_constant__ CUtensorMap map_qk, const __grid
     load_phase[stage] ^= 1;
 
     // ---- S = Q K^T: K = 64 bytes = two MMA K-steps; N in chunks of at most 256 columns
-    if (ok && tid == 0) {
+    if (ok && warp == 0 && ptx::elect_one()) {
       ptx::tc_fence_after_sync();
       const uint64_t dq = ptx::make_kmajor_desc(ptx::smem_addr(sQ), 512, ptx::kSwizzle64);
       for (int n0 = 0; n0 < Lp; n0 += 256) {
@@ -256,7 +256,7 @@ attention_coarse_kernel(const __grid_constant__ CUtensorMap map_qk, const __grid
     if (!ok) break;
 
     // ---- ctx = P V: K = Lp in steps of 32, accumulator in columns 0..63 (scores are dead)
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
       ptx::tc_fence_after_sync();
       const uint32_t idesc = ptx::make_idesc_i8(128, kHeadDim, false, true);   // u8 x s8
       for (int kk = 0; kk < Lp / 32; ++kk) {
@@ -469,7 +469,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
   uint32_t kv_phase = 0, mma_phase = 0;
   int qbuf = 0;
   bool ok = true;
-  if (tid == 0 && (int)blockIdx.x < total) {
+  if (warp == 0 && (int)blockIdx.x < total && ptx::elect_one()) {
     load_q(blockIdx.x, 0, 0);
     load_k(blockIdx.x);
     load_v(blockIdx.x);
@@ -518,7 +518,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       q_phase[qbuf] ^= 1;
 
       // ---- S = Q K^T: K = 64 bytes = two MMA K-steps; N in chunks of at most 256 columns
-      if (ok && tid == 0) {
+      if (ok && warp == 0 && ptx::elect_one()) {
         ptx::tc_fence_after_sync();
         if constexpr (QT) {
           // MN-major operands: [64 dims][128 tokens] tiles, 128-byte swizzle; eight dims form a 1 KB group,
@@ -555,7 +555,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_mma, mma_phase));
       mma_phase ^= 1;
       // K is no longer read once the last tile's scores exist: fetch the next pair's K behind the softmax
-      if (ok && tid == 0 && last_tile && next < total) {
+      if (ok && warp == 0 && last_tile && next < total && ptx::elect_one()) {
         load_k(next);
         if (a.q_bufs == 1) load_q(next, 0, 0);      // single tile per pair: Q is as dead as K by now
       }
@@ -675,7 +675,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       if (!ok) break;
 
       // ---- ctx = P V: K = Lp in steps of 32, accumulator in columns 0..63 (scores are dead)
-      if (tid == 0) {
+      if (warp == 0 && ptx::elect_one()) {
         ptx::tc_fence_after_sync();
         // B = V as loaded ([key][head dim], head dim contiguous): the MN-major operand form (bit 16)
         const uint32_t idesc = ptx::make_idesc_i8(128, kHeadDim, false, true) | (QT ? 0u : (1u << 16));   // u8 x s8
@@ -697,7 +697,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       }
       ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_mma, mma_phase));
       mma_phase ^= 1;
-      if (ok && tid == 0 && last_tile && next < total) load_v(next);   // V was read by the MMAs that just completed
+      if (ok && warp == 0 && last_tile && next < total && ptx::elect_one()) load_v(next);   // V was read by the MMAs that just completed
 
       // ---- epilogue: the 64 context values of a row in two halves, taken by column groups 0 and 1
       // (by group 0 alone when there is only one)

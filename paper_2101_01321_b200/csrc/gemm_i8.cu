@@ -203,7 +203,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       if constexpr (C::kTable) {
         // the table may have been written by the kernel before this one: fetched after the dependency wait
         ptx::mbar_arrive_expect_tx(bar_table, kGeluTableBytes);
@@ -237,7 +237,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (PAIR: leader CTA only)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::make_idesc_i8(kTileChannels, TOK, true, true);
       uint32_t stage = 0, phase = 0;
       uint32_t acc = 0, acc_phase = 0;

@@ -170,7 +170,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t stage = 0, phase = 0;
       for (uint32_t it = 0; unit_of(it) < n_units && ok; ++it) {
         const int t0 = (int)tile_of(it) * kTok;
@@ -196,7 +196,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (PAIR: the pair's leader only)
-    if (lane == 0 && half == 0) {
+    if (half == 0 && ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::make_idesc_i8(PAIR ? 2 * kTok : kTok, kCh, true, true) | (XT ? (1u << 15) : 0u);
       const uint16_t pair_mask = (uint16_t)(3u << leader);
       uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;

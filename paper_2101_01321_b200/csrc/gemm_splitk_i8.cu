@@ -132,7 +132,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t stage = 0, phase = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!ptx::mbar_wait(bar_empty + 8 * stage, phase ^ 1)) { ok = false; break; }
@@ -146,7 +146,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && has_k) {
+    if (has_k && ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::make_idesc_i8(kCh, kTok, true, true);
       uint32_t stage = 0, phase = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
