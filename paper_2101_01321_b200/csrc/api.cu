@@ -510,6 +510,28 @@ static int ensure_workspace(ibert_ctx* ctx, size_t need) {
   return IBERT_OK;
 }
 
+// projection + residual + LayerNorm: the small-problem cluster kernel while the problem is one wave of it, the
+// large-tile cluster kernel once its tiles keep half of the SMs busy, in between two kernels over an int16
+// tensor at `mid` (room for T H of them)
+enum LnPath { LN_SMALL, LN_LARGE, LN_TWO };
+static LnPath linear_ln_path(const ibert_ctx* ctx, int64_t T, int H, int K, const GemmEpilogue& e, const LnConsts& ln) {
+  if (ctx->fusion_mode == 0 && ctx->splitk_mode == 0 && gemm_ln_small_supported(ctx, T, H, K, e, ln)) return LN_SMALL;
+  return gemm_ln_profitable(ctx, T, H) && gemm_ln_supported(H, K, e, ln) ? LN_LARGE : LN_TWO;
+}
+static int linear_ln(ibert_ctx* ctx, LnPath path, const int8_t* x, const int8_t* w, int64_t T, int H, int K,
+                     GemmEpilogue e, const int8_t* res, const LnConsts& ln, const int32_t* d_b_i,
+                     const int64_t* d_B_i, int16_t* mid, int8_t* out, bool x_transposed = false) {
+  if (path != LN_TWO) {
+    ProfileScope ps(ctx, K > 2048 ? IBERT_K_GEMM_LN_WIDE : IBERT_K_GEMM_LN);
+    return path == LN_SMALL ? launch_gemm_ln_small_i8(ctx, x, w, T, H, K, e, res, ln, d_b_i, d_B_i, out)
+                            : launch_gemm_ln_i8(ctx, x, w, T, H, K, e, res, ln, d_b_i, d_B_i, out, x_transposed);
+  }
+  e.kind = EPI_Q16H;               // int16 between the two kernels (value-identical, half the bytes)
+  { ProfileScope ps(ctx, gemm_class(EPI_Q16, K)); if (int rc = launch_gemm_i8(ctx, x, w, T, H, K, e, mid)) return rc; }
+  ProfileScope ps(ctx, IBERT_K_LAYERNORM);
+  return launch_layernorm_i16(ctx, mid, res, T, ln, d_b_i, d_B_i, out);
+}
+
 int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const int8_t* w, const double* S_w,
                               const int32_t* bias, int64_t M, int N, int K, double S_mid,
                               const int8_t* res, double S_res, const double* gamma, const double* beta,
@@ -550,19 +572,10 @@ int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const
   if ((rc = cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &d_Bi))) return rc;
   epi.d_b = (const int32_t*)d_b;
   epi.d_c = (const int32_t*)d_c;
-  if (gemm_ln_profitable(ctx, M, N) && gemm_ln_supported(N, K, epi, k)) {
-    ProfileScope ps(ctx, K > 2048 ? IBERT_K_GEMM_LN_WIDE : IBERT_K_GEMM_LN);
-    rc = launch_gemm_ln_i8(ctx, x, w, M, N, K, epi, res, k, (const int32_t*)d_bi, (const int64_t*)d_Bi, out);
-  } else {
-    // the Q16 tensor between the two kernels is held as int16 (value-identical, half the bytes)
-    if ((rc = ensure_workspace(ctx, (size_t)M * N * 2 + 256))) return rc;
-    int16_t* mid = static_cast<int16_t*>(ctx->ws);
-    epi.kind = EPI_Q16H;
-    { ProfileScope ps(ctx, gemm_class(EPI_Q16, K)); rc = launch_gemm_i8(ctx, x, w, M, N, K, epi, mid); }
-    if (rc) return rc;
-    ProfileScope ps(ctx, IBERT_K_LAYERNORM);
-    rc = launch_layernorm_i16(ctx, mid, res, M, k, (const int32_t*)d_bi, (const int64_t*)d_Bi, out);
-  }
+  const LnPath path = linear_ln_path(ctx, M, N, K, epi, k);
+  if (path == LN_TWO && (rc = ensure_workspace(ctx, (size_t)M * N * 2 + 256))) return rc;
+  rc = linear_ln(ctx, path, x, w, M, N, K, epi, res, k, (const int32_t*)d_bi, (const int64_t*)d_Bi,
+                 static_cast<int16_t*>(ctx->ws), out);
   if (rc == IBERT_OK && S_ret) *S_ret = S_out;
   return rc;
   });
@@ -812,11 +825,13 @@ static int encoder_layer_common(ibert_ctx* ctx, const ibert_layer* ly, const int
 
   GemmEpilogue e{};
   int rc;
+  e.w_static = true;
   e.kind = EPI_INT8; e.d_b = ly->b_qkv; e.d_c = ly->c_qkv; e.d_bias = ly->bias_qkv; e.fast = ly->fast_qkv;
   // Q | K | V between the two kernels: transposed ([3H][T]) where both sides take it -- a thread of the GEMM
   // holds one channel of 32 tokens, which are contiguous bytes of that layout
   const bool qkv_t = ctx->qkv_layout_mode != 1 && !cu_seqlens && ly->fast_qkv == 1 &&
-                     attention_takes_transposed(B, L, ly->attn);
+                     attention_takes_transposed(B, L, ly->attn) &&
+                     !(ctx->qkv_layout_mode == 0 && ctx->splitk_mode == 0 && gemm_small_takes(ctx, T, 3 * H, H));
   e.out_transposed = qkv_t;
   { ProfileScope ps(ctx, IBERT_K_GEMM_QKV); rc = launch_gemm_i8(ctx, x, ly->w_qkv, T, 3 * H, H, e, qkv); }
   e.out_transposed = false;
@@ -825,29 +840,20 @@ static int encoder_layer_common(ibert_ctx* ctx, const ibert_layer* ly, const int
   if (rc) return rc;
   // output projection + residual + LayerNorm: one kernel when shapes and constants allow it
   e.kind = EPI_Q16; e.d_b = ly->b_o; e.d_c = ly->c_o; e.d_bias = ly->bias_o; e.fast = ly->fast_o;
-  // the cluster kernel pays off once its 128-token tiles keep at least half of the SMs busy; below
-  // that the two kernels, which spread a small problem over more CTAs, are faster
-  const bool fuse = gemm_ln_profitable(ctx, T, H);
-  if (fuse && gemm_ln_supported(H, H, e, ly->ln1)) {
-    ProfileScope ps(ctx, IBERT_K_GEMM_LN);
-    rc = launch_gemm_ln_i8(ctx, cx, ly->w_o, T, H, H, e, x, ly->ln1, ly->ln1_b, ly->ln1_B, h1);
-  } else {
-    e.kind = EPI_Q16H;
-    { ProfileScope ps(ctx, IBERT_K_GEMM_Q16); rc = launch_gemm_i8(ctx, cx, ly->w_o, T, H, H, e, r); }
-    if (rc) return rc;
-    { ProfileScope ps(ctx, IBERT_K_LAYERNORM); rc = launch_layernorm_i16(ctx, r, x, T, ly->ln1, ly->ln1_b, ly->ln1_B, h1); }
-  }
-  if (rc) return rc;
+  if ((rc = linear_ln(ctx, linear_ln_path(ctx, T, H, H, e, ly->ln1), cx, ly->w_o, T, H, H, e, x, ly->ln1, ly->ln1_b,
+                      ly->ln1_B, r, h1)))
+    return rc;
   GemmEpilogue e2{};
+  e2.w_static = true;
   e2.kind = EPI_Q16; e2.d_b = ly->b_f2; e2.d_c = ly->c_f2; e2.d_bias = ly->bias_f2; e2.fast = ly->fast_f2;
-  const bool fuse2 = fuse && gemm_ln_supported(H, F, e2, ly->ln2);
+  const LnPath path2 = linear_ln_path(ctx, T, H, F, e2, ly->ln2);
   // the FFN1 result between its GEMM and the cluster kernel: transposed ([F][T]) where both sides take it
   // (the table epilogue of a CTA-pair sized problem on one side, the fused kernel on the other)
   // (a tensor that no longer fits L2 comes back from HBM, where the fused kernel's channel-major tiles --
   // 128 rows of 128 bytes, T bytes apart -- read slower than token-major ones: T = 32768, F = 4096, 128 MB,
   // loses 1.5 % of the step)
   const bool g_pays = T >= 4096 && (int64_t)T * F <= ctx->l2_bytes / 2;
-  const bool g_t = fuse2 && ctx->qkv_layout_mode != 1 && (g_pays || ctx->qkv_layout_mode == 2) && ly->gelu_table &&
+  const bool g_t = path2 == LN_LARGE && ctx->qkv_layout_mode != 1 && (g_pays || ctx->qkv_layout_mode == 2) && ly->gelu_table &&
                    ctx->gelu_table_mode == 0 && ly->fast_f1 != 0 && ly->gelu.fast != 0 &&
                    gemm_gelu_takes_transposed(ctx, T, F);
   e.kind = EPI_GELU; e.d_b = ly->b_f1; e.d_c = ly->c_f1; e.d_bias = ly->bias_f1; e.gelu = ly->gelu; e.fast = ly->fast_f1; e.gelu_table = ly->gelu_table;
@@ -855,16 +861,7 @@ static int encoder_layer_common(ibert_ctx* ctx, const ibert_layer* ly, const int
   { ProfileScope ps(ctx, IBERT_K_GEMM_GELU); rc = launch_gemm_i8(ctx, h1, ly->w_f1, T, F, H, e, g); }
   e.out_transposed = false;
   if (rc) return rc;
-  e.kind = EPI_Q16; e.d_b = ly->b_f2; e.d_c = ly->c_f2; e.d_bias = ly->bias_f2; e.fast = ly->fast_f2;
-  if (fuse2) {
-    ProfileScope ps(ctx, F > 2048 ? IBERT_K_GEMM_LN_WIDE : IBERT_K_GEMM_LN);
-    return launch_gemm_ln_i8(ctx, g, ly->w_f2, T, H, F, e, h1, ly->ln2, ly->ln2_b, ly->ln2_B, out, g_t);
-  }
-  e.kind = EPI_Q16H;
-  { ProfileScope ps(ctx, IBERT_K_GEMM_Q16_WIDE); rc = launch_gemm_i8(ctx, g, ly->w_f2, T, H, F, e, r); }
-  if (rc) return rc;
-  { ProfileScope ps(ctx, IBERT_K_LAYERNORM); rc = launch_layernorm_i16(ctx, r, h1, T, ly->ln2, ly->ln2_b, ly->ln2_B, out); }
-  return rc;
+  return linear_ln(ctx, path2, g, ly->w_f2, T, H, F, e2, h1, ly->ln2, ly->ln2_b, ly->ln2_B, r, out, g_t);
 }
 
 int ibert_encoder_layer(ibert_ctx* ctx, const ibert_layer* ly, const int8_t* x, int B, int L,
@@ -1132,6 +1129,17 @@ int ibert_selftest_exp_division(double S, int32_t* q_ln2_out) {
     const uint64_t wide = (uint64_t)(uint32_t)(d << k.div_pre) * (uint64_t)k.div_m;
     const uint32_t z = (uint32_t)(wide >> 32) >> k.div_post;
     if (z != d / k.q_ln2) return IBERT_ERR_VALUE_RANGE;
+  }
+  if (k.fold_m != 0) {               // quotient and post-shift in one multiply-high: the exponential itself, every d < 2^21
+    for (uint32_t d = 0; d < (1u << 21); ++d) {
+      const uint32_t dp = d >> k.s_in, z = dp / k.q_ln2;
+      const int32_t t = k.q_b - (int32_t)(dp - z * k.q_ln2);
+      const uint32_t n = z + (uint32_t)k.s_out, want = n > 31 ? 0u : (uint32_t)(t * t + k.q_c) >> n;
+      const uint32_t D = dp + (uint32_t)k.s_out * k.q_ln2 + (uint32_t)k.fold_add;
+      const uint32_t nf = (uint32_t)(((uint64_t)D * (uint64_t)k.fold_m) >> 32);
+      const int32_t tf = (int32_t)(nf * k.q_ln2) + (k.q_b + k.fold_add - (int32_t)D);
+      if ((nf > 31 ? 0u : (uint32_t)(tf * tf + k.q_c) >> nf) != want) return IBERT_ERR_VALUE_RANGE;
+    }
   }
   if (k.wide_post >= 0) {            // the unclamped form used on attention scores: every d < 2^21
     for (uint32_t d = 0; d < (1u << 21); ++d) {

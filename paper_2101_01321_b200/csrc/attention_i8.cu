@@ -18,7 +18,6 @@ namespace ibert {
 namespace {
 
 constexpr int kAttnThreads = 128;   // thread t owns query row t (= TMEM lane t)
-constexpr int kHeadDim = 64;
 
 struct CoarseArgs {
   int B, L, H, heads;
@@ -31,13 +30,6 @@ struct CoarseArgs {
   int8_t* out;
   int32_t* status;
 };
-
-// byte offset of element (row, col) in a K-major operand tile made of 128-byte-wide K blocks
-// with the 128-byte swizzle: 16-byte chunk c of row r sits at chunk c ^ (r & 7).
-__device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t col, uint32_t rows_per_block) {
-  const uint32_t kb = col >> 7, cc = (col >> 4) & 7, by = col & 15;
-  return kb * (rows_per_block * 128u) + row * 128u + (((cc ^ (row & 7u)) << 4) | by);
-}
 
 // i-softmax (Algorithm 3) of one score row held in TMEM lane `t_row`, columns [0, L):
 // pass 1 row maximum, pass 2 i-exp + int32 row sum (exponentials written back over the scores),

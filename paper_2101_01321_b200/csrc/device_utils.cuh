@@ -125,6 +125,27 @@ __device__ __forceinline__ int32_t ihgelu_to_int8(int32_t q, const GeluConsts& k
   return requant_add((q * r + 128) >> 8, k.b, half, k.c, 127);
 }
 
+// One output value of a linear layer from one complete accumulator, by epilogue kind.  FAST: multipliers in
+// upper-word form; `padd` = bias * b + rounding constant for the generic form; `gelu_rnd` = 2^s_f - 1.
+template <int KIND, bool FAST>
+__device__ __forceinline__ int32_t epilogue_value(int32_t a, int32_t bias, int32_t pb, int32_t pc, int64_t padd,
+                                                  const GeluConsts& gk, int64_t gelu_half, int32_t gelu_rnd) {
+  if constexpr (KIND == EPI_RAW) return a + bias;
+  else if constexpr (KIND == EPI_Q16 || KIND == EPI_Q16H) {
+    if constexpr (FAST) return clamp_sym(requant_upper(a + bias, pb), 32767);
+    else return requant_add(a, pb, padd, pc, 32767);
+  } else if constexpr (KIND == EPI_INT8) {
+    if constexpr (FAST) return clamp_sym(requant_upper(a + bias, pb), 127);
+    else return requant_add(a, pb, padd, pc, 127);
+  } else if constexpr (KIND == EPI_HGELU) {
+    if constexpr (FAST) return clamp_sym(ihgelu_upper(requant_upper(a + bias, pb), gk), 127);
+    else return ihgelu_to_int8(requant_add(a, pb, padd, pc, 32767), gk, gelu_half);
+  } else {
+    if constexpr (FAST) return clamp_sym(igelu_magnitude_upper(requant_upper(a + bias, pb), gk, gelu_rnd), 127);
+    else return igelu_q16_to_int8(requant_add(a, pb, padd, pc, 32767), gk, gelu_half);
+  }
+}
+
 __device__ __forceinline__ uint32_t shr_clamped(uint32_t v, uint32_t n) {
   uint32_t r;
   asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));   // shift counts above 31 give 0
@@ -161,14 +182,62 @@ __device__ __forceinline__ uint32_t iexp_dist_pow2(uint32_t dk, int32_t q_b, int
   const int32_t t = q_b - (int32_t)(dk & mask);                          // q_b - r
   return shr_clamped((uint32_t)(t * t + q_c), dk >> k);
 }
+// The same when quotient and post-shift come from one multiply-high (ExpConsts::fold_m): `D` = pre-shifted
+// distance + s_out q_ln2 + fold_add, `w` = q_b + fold_add - D.
+__device__ __forceinline__ uint32_t iexp_folded(uint32_t D, int32_t w, uint32_t fold_m, uint32_t q_ln2, int32_t q_c) {
+  const uint32_t n = __umulhi(D, fold_m);                                // floor(d / q_ln2) + s_out
+  const int32_t t = (int32_t)(n * q_ln2) + w;                            // q_b - r
+  return shr_clamped((uint32_t)(t * t + q_c), n);
+}
 __host__ __device__ __forceinline__ int exp_div_mode(const ExpConsts& k) {
   return k.div_pre != 0 ? 2 : (k.div_post != 0 ? 1 : 0);
 }
 
+// floor(sqrt(floor(ss / C))), i.e. the largest s with s*s*C <= ss -- the value Algorithm 4
+// returns for n = floor(ss / C).  A 64-bit integer division costs on the order of a hundred
+// instructions here, so instead of iterating x <- (x + n/x)/2 the warp finds the same integer by
+// a radix-32 search: in each of five rounds the 32 lanes test 32 candidates with one multiply
+// each.  Needs s < 2^25 and ss < 2^61 / C.
+__device__ __forceinline__ uint32_t warp_isqrt_of_quotient(uint64_t ss, uint32_t C, int lane) {
+  uint32_t base = 0;
+  // ss / C < 2^bits bounds the result below 2^ceil(bits / 2): rounds above that cannot set a digit
+  const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));
+  const int top = 5 * ((min(max((bits + 1) >> 1, 1), 25) + 4) / 5 - 1);
+  for (int shift = top; shift >= 0; shift -= 5) {
+    const uint32_t cand = base + ((uint32_t)lane << shift);
+    const uint64_t sq = (uint64_t)cand * (uint64_t)cand;
+    const bool le = sq * (uint64_t)C <= ss;                       // true for a prefix of the lanes
+    const uint32_t cnt = __popc(__ballot_sync(0xffffffffu, le));  // >= 1: lane 0 tests `base` itself
+    base += (cnt - 1u) << shift;
+  }
+  return base;
+}
+
+// byte offset of element (row, col) in a K-major operand tile made of 128-byte-wide K blocks
+// with the 128-byte swizzle: 16-byte chunk c of row r sits at chunk c ^ (r & 7).
+__device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t col, uint32_t rows_per_block) {
+  const uint32_t kb = col >> 7, cc = (col >> 4) & 7, by = col & 15;
+  return kb * (rows_per_block * 128u) + row * 128u + (((cc ^ (row & 7u)) << 4) | by);
+}
+
+// Reciprocal of a normalised 32-bit integer by Newton-Raphson iteration (r <- r (2 - y r), the usual linear
+// start 48/17 - 32/17 y, relative error 1/17 squared by every step): for y in [2^31, 2^32) the result is
+// floor(2^63 / y) or one less (saturated to 32 bits at y = 2^31).  Two steps in 32-bit fixed point (Q30), the
+// last one on the exact 64-bit remainder.
+__device__ __forceinline__ uint32_t reciprocal_q31(uint32_t y) {
+  uint32_t r = 0xB4B4B4B4u - __umulhi(0x78787878u, y);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) r = __umulhi(r, 0x80000000u - __umulhi(y, r)) << 2;
+  const int64_t rem = (int64_t)((uint64_t(1) << 62) - (uint64_t)y * (uint64_t)r);     // below 2^46
+  return 2u * r + (uint32_t)(__mulhi((int32_t)(rem >> 15), (int32_t)r) >> 14);
+}
+
 // Per-row divisor for p = floor(e * p_max / sum) with e < 2^21 and e <= sum < 2^31:
-// with l = bit length of sum, K = 21 + l and m = ceil(p_max 2^K / sum) (< 2^30),
-// floor(e m / 2^K) is exact: the excess e (m sum - p_max 2^K) / (sum 2^K) stays below 2^-l < 1/sum.
-// Evaluated as umulhi(e << pre, m) >> post with post - pre = K - 32.
+// with l = bit length of sum, K = 23 + l and any integer m with 0 <= m sum - p_max 2^K < 4 sum,
+// floor(e m / 2^K) is exact: the excess e (m sum - p_max 2^K) / (sum 2^K) stays below
+// 2^(21 + 2 - K) = 2^-l < 1/sum.  p_max 2^K / sum = p_max 2^55 / y for the normalised sum y, so
+// m = floor(p_max R / 256) + 3 from the reciprocal above lies 0.3 to 3 too high (a 64-bit division costs four
+// times the instructions).  Evaluated as umulhi(e << pre, m) >> post with post - pre = K - 32.
 struct RowDivisor {
   uint32_t m;
   int pre, post;
@@ -176,10 +245,8 @@ struct RowDivisor {
 
 __device__ __forceinline__ RowDivisor make_row_divisor(uint32_t sum, uint32_t p_max) {
   RowDivisor r;
-  const int l = 32 - __clz(sum);
-  const int K = 21 + l;
-  const uint64_t num = ((uint64_t)p_max << K) + (uint64_t)(sum - 1u);
-  r.m = (uint32_t)(num / (uint64_t)sum);
+  const int lz = __clz(sum), K = 23 + 32 - lz;
+  r.m = __umulhi(reciprocal_q31(sum << lz), p_max << 24) + 3u;
   r.pre = K < 32 ? 32 - K : 0;
   r.post = K < 32 ? 0 : K - 32;
   return r;
@@ -188,7 +255,7 @@ __device__ __forceinline__ RowDivisor make_row_divisor(uint32_t sum, uint32_t p_
 __device__ __forceinline__ uint32_t softmax_quotient(uint32_t e, const RowDivisor& r) {
   return __umulhi(e << r.pre, r.m) >> r.post;
 }
-// the common case pre == 0 (row sum >= 2^10)
+// the common case pre == 0 (row sum >= 2^8)
 __device__ __forceinline__ uint32_t softmax_quotient_nopre(uint32_t e, const RowDivisor& r) {
   return __umulhi(e, r.m) >> r.post;
 }

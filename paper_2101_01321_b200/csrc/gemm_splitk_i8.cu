@@ -58,26 +58,6 @@ __device__ __forceinline__ int32_t ld_cluster_s32(uint32_t cluster_addr) {
   return v;
 }
 
-// one output value from one complete accumulator
-template <int KIND, bool FAST>
-__device__ __forceinline__ int32_t epilogue_value(int32_t a, int32_t bias, int32_t pb, int32_t pc, int64_t padd,
-                                                  const GeluConsts& gk, int64_t gelu_half, int32_t gelu_rnd) {
-  if constexpr (KIND == EPI_RAW) return a + bias;
-  else if constexpr (KIND == EPI_Q16 || KIND == EPI_Q16H) {
-    if constexpr (FAST) return clamp_sym(requant_upper(a + bias, pb), 32767);
-    else return requant_add(a, pb, padd, pc, 32767);
-  } else if constexpr (KIND == EPI_INT8) {
-    if constexpr (FAST) return clamp_sym(requant_upper(a + bias, pb), 127);
-    else return requant_add(a, pb, padd, pc, 127);
-  } else if constexpr (KIND == EPI_HGELU) {
-    if constexpr (FAST) return clamp_sym(ihgelu_upper(requant_upper(a + bias, pb), gk), 127);
-    else return ihgelu_to_int8(requant_add(a, pb, padd, pc, 32767), gk, gelu_half);
-  } else {
-    if constexpr (FAST) return clamp_sym(igelu_magnitude_upper(requant_upper(a + bias, pb), gk, gelu_rnd), 127);
-    else return igelu_q16_to_int8(requant_add(a, pb, padd, pc, 32767), gk, gelu_half);
-  }
-}
-
 template <int KIND, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,

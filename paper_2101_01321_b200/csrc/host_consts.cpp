@@ -107,6 +107,22 @@ int make_exp_consts(double S, int p_max, ExpConsts* k) {
   k->q_c = (int32_t)q_c;
   k->s_out = bl > 21 ? bl - 21 : 0;
   k->p_max = (uint32_t)p_max;
+  // Quotient and post-shift in one multiply-high: n = floor(D' / q) = floor(d' / q) + s_out for D' = d' + s_out q.
+  // Rounded up, m = ceil(2^32 / q) with m q = 2^32 + e0 gives n = umulhi(D', m) exactly while D' e0 < 2^32;
+  // rounded down, m = floor(2^32 / q) with m q = 2^32 - e1 gives n = umulhi(D' + 1, m) exactly while
+  // 0 < (D' + 1) e1 <= 2^32 (e0 + e1 = q, so one of them is at most q / 2).  Exactness is needed up to
+  // D' = bl q: from there on the count is at least bl > log2 of the polynomial, so e = 0; the count is off by
+  // at most one there (D' < 2^22), which moves the remainder by at most 16 past [0, q) and the polynomial
+  // below 2^(bl + 1) with the count at least bl + 1 when it rounds up.  Needs q_b well above 16: q >= 16.
+  k->fold_m = 0;
+  k->fold_add = 0;
+  if (k->q_ln2 >= 16) {
+    const uint64_t q = k->q_ln2, d_top = (uint64_t)bl * q;
+    const uint64_t up = ((uint64_t(1) << 32) + q - 1) / q, down = (uint64_t(1) << 32) / q;
+    const uint64_t e0 = up * q - (uint64_t(1) << 32), e1 = (uint64_t(1) << 32) - down * q;
+    if (d_top * e0 < (uint64_t(1) << 32)) k->fold_m = (uint32_t)up;
+    else if ((d_top + 1) * e1 <= (uint64_t(1) << 32)) { k->fold_m = (uint32_t)down; k->fold_add = 1; }
+  }
   k->pow2_k = -1;
   if (s_in == 0 && (k->q_ln2 & (k->q_ln2 - 1)) == 0) {
     int lg = 0;

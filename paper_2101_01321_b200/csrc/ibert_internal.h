@@ -35,6 +35,12 @@ struct ExpConsts {
   // k when q_ln2 = 2^k and s_in = 0 (score scale exactly ln2 / 2^k): quotient and remainder of the
   // distance are then a shift and a mask; -1 otherwise
   int32_t pow2_k;
+  // the quotient and the post-shift in one multiply-high (attention scores): with the distance d' offset to
+  // D = d' + s_out q_ln2 + fold_add,  umulhi(D, fold_m) = floor(d' / q_ln2) + s_out -- the whole shift count of
+  // Algorithm 3 -- wherever e is not zero, and a count that still shifts everything out beyond.  fold_m = 0:
+  // not available (q_ln2 < 16, and a few q_ln2 above 16645)
+  uint32_t fold_m;
+  int32_t fold_add;
 };
 
 // i-GELU (Algorithm 2) followed by requantization to int8
@@ -182,6 +188,9 @@ struct GemmEpilogue {
   // A thread of the GEMM owns one channel and 32 tokens, so its results are contiguous bytes of the
   // transposed tensor and leave without a transposing store; the attention kernel reads that layout.
   bool out_transposed = false;
+  // the weights and constants belong to a layer (complete before the call): a kernel may read them before the
+  // work in front of it on the stream has finished
+  bool w_static = false;
 };
 
 // Upper-word form of a column set: true if for every n, c[n] >= 1 and b[n] << (32 - c[n]) fits
@@ -201,6 +210,16 @@ int launch_gemm_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, 
 int gemm_splitk_width(const ibert_ctx* ctx, int64_t M, int N, int K);
 int launch_gemm_splitk_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int N, int K,
                           const GemmEpilogue& epi, void* out, int split);
+
+// One-wave kernels for small token counts (128 channels x 16..128 tokens per CTA; with LayerNorm a cluster of
+// H / 128 CTAs per 16..64 tokens).  The two predicates tell whether the problem is one wave or less.
+bool gemm_small_takes(const ibert_ctx* ctx, int64_t M, int N, int K);
+int launch_gemm_small_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int N, int K,
+                         const GemmEpilogue& epi, void* out);
+bool gemm_ln_small_supported(const ibert_ctx* ctx, int64_t M, int H, int K, const GemmEpilogue& epi, const LnConsts& ln);
+int launch_gemm_ln_small_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int H, int K,
+                            const GemmEpilogue& epi, const int8_t* res, const LnConsts& ln, const int32_t* d_b_i,
+                            const int64_t* d_B_i, int8_t* out);
 
 // Launch with programmatic stream serialization (the kernel must call grid_dep_wait() before its
 // first global-memory access) and an optional cluster width.
@@ -228,6 +247,8 @@ inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
   return IBERT_OK;
 }
 
+constexpr int kHeadDim = 64;
+
 struct AttnConsts {
   ExpConsts e;
   int32_t b, c;            // dyadic((1/p_max) * S_v / S_ctx)
@@ -249,6 +270,10 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
 int launch_attention(ibert_ctx* ctx, const int8_t* qkv, int B, int L, int H, int heads,
                      const AttnConsts& k, const int32_t* lens, int8_t* out, const int32_t* cu_seqlens = nullptr,
                      int64_t total_rows = 0, bool qkv_t = false);
+// Few (batch, head) pairs: one CTA per 32, 64 or 128 queries of a pair (launch_attention dispatches to it)
+bool attention_small_takes(const ibert_ctx* ctx, int B, int L, int heads, const AttnConsts& k);
+int launch_attention_small(ibert_ctx* ctx, const int8_t* qkv, int B, int L, int H, int heads, const AttnConsts& k,
+                           const int32_t* lens, int8_t* out, const int32_t* cu_seqlens, int64_t total_rows);
 // true when launch_attention can read the transposed tensor qkv^T [3H][B L] (qkv_t): padded batch, L a
 // multiple of 16, a score scale the main kernel takes
 bool attention_takes_transposed(int B, int L, const AttnConsts& k);

@@ -177,26 +177,6 @@ __global__ void __launch_bounds__(kThreads) softmax_kernel(const int32_t* __rest
 }
 
 // ----------------------------------------------------------------------------- i-LayerNorm
-// floor(sqrt(floor(ss / C))), i.e. the largest s with s*s*C <= ss -- the value Algorithm 4
-// returns for n = floor(ss / C).  A 64-bit integer division costs on the order of a hundred
-// instructions here, so instead of iterating x <- (x + n/x)/2 the warp finds the same integer by
-// a radix-32 search: in each of five rounds the 32 lanes test 32 candidates with one multiply
-// each.  Needs s < 2^25 and ss < 2^61 / C.
-__device__ __forceinline__ uint32_t warp_isqrt_of_quotient(uint64_t ss, uint32_t C, int lane) {
-  uint32_t base = 0;
-  // ss / C < 2^bits bounds the result below 2^ceil(bits / 2): rounds above that cannot set a digit
-  const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));
-  const int top = 5 * ((min(max((bits + 1) >> 1, 1), 25) + 4) / 5 - 1);
-  for (int shift = top; shift >= 0; shift -= 5) {
-    const uint32_t cand = base + ((uint32_t)lane << shift);
-    const uint64_t sq = (uint64_t)cand * (uint64_t)cand;
-    const bool le = sq * (uint64_t)C <= ss;                       // true for a prefix of the lanes
-    const uint32_t cnt = __popc(__ballot_sync(0xffffffffu, le));  // >= 1: lane 0 tests `base` itself
-    base += (cnt - 1u) << shift;
-  }
-  return base;
-}
-
 // Four consecutive Q16 values of a row, from an int32 or an int16 container (16 / 8 bytes)
 template <typename QT>
 __device__ __forceinline__ void load_q4(const QT* p, int32_t (&v)[4], bool streaming) {
@@ -597,7 +577,7 @@ __global__ void __launch_bounds__(kThreads, 4) softmax_short_kernel(const int32_
     for (int r = 0; r < R; ++r) {
       RowDivisor rd;
       rd.m = __shfl_sync(0xffffffffu, my_m, r);
-      const int K = 21 + 32 - __clz(sums[r]);
+      const int K = 23 + 32 - __clz(sums[r]);
       rd.pre = K < 32 ? 32 - K : 0;
       rd.post = K < 32 ? 0 : K - 32;
       uint32_t p[4];
