@@ -758,6 +758,8 @@ int launch_attention(ibert_ctx* ctx, const int8_t* qkv, int B, int L, int H, int
   if (B == 0) return IBERT_OK;
   if (qkv_t && (cu_seqlens || !attention_takes_transposed(B, L, k))) return IBERT_ERR_ARG;
   if (cu_seqlens && k.e.wide_post < 0) return IBERT_ERR_SCALE_RANGE;   // packed batches: main kernel only
+  if (!qkv_t && attention_small_takes(ctx, B, L, heads, k))
+    return launch_attention_small(ctx, qkv, B, L, H, heads, k, lens, out, cu_seqlens, total_rows);
   const int Lp = (L + 31) & ~31, n_slabs = (L + 127) / 128;
   uint32_t cols = 64;
   while ((int)cols < Lp) cols <<= 1;

@@ -56,3 +56,28 @@ def test_linear_layernorm(M, N, K, constant_rows):
     ctx().check()
     mid = oracle.linear(x, S_x, w, S_w, bias, 1, S_mid)
     assert_same(host(out), oracle.layernorm(mid, S_mid, res, S_res, gamma, beta, S_out)[0], "linear + LayerNorm")
+
+
+# four, two and one copies of the queries; 8, 16 and 32 columns per thread; lengths around multiples of 32; the
+# first pair count past the range; score scales with and without a pre-shift, and an exact ln2 / 2^k
+@pytest.mark.parametrize("B,L,heads", [(1, 1, 1), (1, 31, 2), (2, 33, 3), (1, 128, 12), (3, 129, 2), (2, 256, 4),
+                                       (1, 257, 2), (1, 512, 16), (8, 77, 12), (12, 100, 12), (24, 128, 12), (25, 128, 12)])
+@pytest.mark.parametrize("S_qk", [0.02, 0.004, float(np.sqrt(8.0 * np.log(2.0) / 2.0 ** 14))])
+def test_attention(B, L, heads, S_qk):
+    H = heads * 64
+    rng = np.random.default_rng(B * 1000 + L)
+    qkv = np.clip(np.rint(rng.standard_normal((B * L, 3 * H)) * 40), -127, 127).astype(np.int8)
+    c = ctx()
+    out, _ = c.ibert_attention_i8(dev(qkv), B, L, H, heads, S_qk, S_qk, 0.02, 0.006, 255)
+    assert_same(host(out), oracle.attention(qkv, B, L, H, heads, S_qk, S_qk, 0.02, 0.006, 255), "attention")
+    lens = rng.integers(0, L + 1, B).astype(np.int32)
+    lens[0] = L if B > 1 else max(L - 1, 0)
+    want = oracle.attention(qkv, B, L, H, heads, S_qk, S_qk, 0.02, 0.006, 127, lens=lens)
+    out, _ = c.ibert_attention_masked_i8(dev(qkv), B, L, H, heads, dev(lens), S_qk, S_qk, 0.02, 0.006, 127)
+    assert_same(host(out), want, "masked attention")
+    rows = np.concatenate([np.arange(b * L, b * L + n) for b, n in enumerate(lens)]).astype(int)
+    if rows.size:
+        cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        out, _ = c.ibert_attention_packed_i8(dev(np.ascontiguousarray(qkv[rows])), dev(cu), L, H, heads, S_qk, S_qk, 0.02, 0.006, 127)
+        assert_same(host(out), want[rows], "packed attention")
+    c.check()
