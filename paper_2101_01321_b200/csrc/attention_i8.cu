@@ -334,6 +334,7 @@ struct AttnArgs {
   int Lp, n_slabs, groups;
   int q_bufs;        // 2 when a pair has several query tiles (next tile's Q prefetched), else 1
   uint32_t tmem_cols;
+  int32_t int_min;   // INT32_MIN, as a run-time value (see add_alu)
   AttnConsts k;
   // padded batches: [B] valid keys per sequence, or nullptr: all L.  Packed batches (the PACKED
   // instantiation of the kernel): [B + 1] first rows of the sequences in a [total tokens, 3H] tensor
@@ -563,14 +564,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
           uint32_t v[kW];
           ptx::tmem_ld(t_row + c0, v);
           ptx::tmem_wait_ld();
-          if (c0 + kW <= n) {
-#pragma unroll
-            for (int i = 0; i < kW; i += 2) mx = __vimax3_s32(mx, (int32_t)v[i], (int32_t)v[i + 1]);
-          } else {
+          if (c0 + kW > n) {
 #pragma unroll
             for (int i = 0; i < kW; ++i)
-              if (c0 + i < n) mx = max(mx, (int32_t)v[i]);
+              if (c0 + i >= n) v[i] = (uint32_t)INT32_MIN;
           }
+#pragma unroll
+          for (int i = 0; i < kW; i += 2) mx = __vimax3_s32(mx, (int32_t)v[i], (int32_t)v[i + 1]);
         }
         s_max[grp * 128 + row] = mx;
       }
@@ -579,50 +579,44 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       uint32_t sum = 0;
       if (ok && live) {
         for (int g = 0; g < G; ++g) mx = max(mx, s_max[g * 128 + row]);
-        if (a.k.e.pow2_k >= 0) {
-          // score scale exactly ln2 / 2^k: quotient and remainder by shift and mask
-          const uint32_t k2 = (uint32_t)a.k.e.pow2_k, mask = (1u << k2) - 1u;
-          const uint32_t mxk = (uint32_t)mx + ((uint32_t)a.k.e.s_out << k2);
-          const int32_t q_b = a.k.e.q_b, q_c = a.k.e.q_c;
+        // one loop per form of the exponential: exp_of turns a score into its exponential.  Bound by the
+        // multiply-add pipe: a multiply-high takes it four clocks, a multiply-add two.  Quotient and post-shift
+        // from one multiply-high, one of the two additions on the ALU pipe and bytes packed by permutes make a
+        // score 11.7 instructions over the three passes instead of 14.7 (probe: 18.7 instead of 21.1 clocks per
+        // warp and scheduler); B = 64, L = 512, 16 heads 262 -> 246 us, B = 128, L = 128, 12 heads 33.1 -> 31.0
+        auto pass2 = [&](auto exp_of) {
           for (int c0 = c_begin; c0 < c_end; c0 += kW) {
             uint32_t v[kW];
             ptx::tmem_ld(t_row + c0, v);
             ptx::tmem_wait_ld();
-            if (c0 + kW <= n) {
 #pragma unroll
-              for (int i = 0; i < kW; ++i) {
-                v[i] = iexp_dist_pow2(mxk - v[i], q_b, q_c, k2, mask);
-                sum += v[i];
-              }
-            } else {
+            for (int i = 0; i < kW; ++i) v[i] = exp_of(v[i]);
+            if (c0 + kW > n) {
 #pragma unroll
-              for (int i = 0; i < kW; ++i) {
-                v[i] = (c0 + i < n) ? iexp_dist_pow2(mxk - v[i], q_b, q_c, k2, mask) : 0u;
-                sum += v[i];
-              }
+              for (int i = 0; i < kW; ++i)
+                if (c0 + i >= n) v[i] = 0u;
             }
+#pragma unroll
+            for (int i = 0; i < kW; i += 2) sum = sum + v[i] + v[i + 1];
             ptx::tmem_st(t_row + c0, v);
+          }
+        };
+        const ExpConsts& ek = a.k.e;
+        if (ek.fold_m != 0) {
+          const uint32_t off = (uint32_t)ek.s_out * ek.q_ln2 + (uint32_t)ek.fold_add;
+          const int32_t qb = ek.q_b + ek.fold_add;
+          if (ek.s_in == 0) {
+            const uint32_t mxk = (uint32_t)mx + off;
+            const int32_t wk = qb - (int32_t)mxk;
+            pass2([&](uint32_t v) { return iexp_folded(mxk - v, add_alu((int32_t)v, wk, a.int_min), ek.fold_m, ek.q_ln2, ek.q_c); });
+          } else {
+            pass2([&](uint32_t v) {
+              const uint32_t D = (((uint32_t)mx - v) >> ek.s_in) + off;
+              return iexp_folded(D, qb - (int32_t)D, ek.fold_m, ek.q_ln2, ek.q_c);
+            });
           }
         } else {
-          for (int c0 = c_begin; c0 < c_end; c0 += kW) {
-            uint32_t v[kW];
-            ptx::tmem_ld(t_row + c0, v);
-            ptx::tmem_wait_ld();
-            if (c0 + kW <= n) {
-#pragma unroll
-              for (int i = 0; i < kW; ++i) {
-                v[i] = iexp_dist_wide((uint32_t)mx - v[i], a.k.e);
-                sum += v[i];
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < kW; ++i) {
-                v[i] = (c0 + i < n) ? iexp_dist_wide((uint32_t)mx - v[i], a.k.e) : 0u;
-                sum += v[i];
-              }
-            }
-            ptx::tmem_st(t_row + c0, v);
-          }
+          pass2([&](uint32_t v) { return iexp_dist_wide((uint32_t)mx - v, ek); });
         }
         ptx::tmem_wait_st();
         s_sum[grp * 128 + row] = sum;
@@ -633,31 +627,27 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
         sum = 0;
         for (int g = 0; g < G; ++g) sum += s_sum[g * 128 + row];
         const RowDivisor rd = make_row_divisor(max(sum, 1u), a.k.e.p_max);   // sum = 0 only without valid keys
-        const bool nopre = __all_sync(0xffffffffu, rd.pre == 0);
-        for (int c0 = c_begin; c0 < c_end; c0 += kW) {
-          uint32_t v[kW];
-          ptx::tmem_ld(t_row + c0, v);
-          ptx::tmem_wait_ld();
+        auto pass3 = [&](auto quotient) {
+          for (int c0 = c_begin; c0 < c_end; c0 += kW) {
+            uint32_t v[kW];
+            ptx::tmem_ld(t_row + c0, v);
+            ptx::tmem_wait_ld();
 #pragma unroll
-          for (int h = 0; h < kW / 16; ++h) {
-            uint32_t w[4];
+            for (int h = 0; h < kW / 16; ++h) {
+              uint32_t w[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int j = h * 16 + i * 4;
-              uint32_t p0, p1, p2, p3;
-              if (nopre) {
-                p0 = softmax_quotient_nopre(v[j], rd); p1 = softmax_quotient_nopre(v[j + 1], rd);
-                p2 = softmax_quotient_nopre(v[j + 2], rd); p3 = softmax_quotient_nopre(v[j + 3], rd);
-              } else {
-                p0 = softmax_quotient(v[j], rd); p1 = softmax_quotient(v[j + 1], rd);
-                p2 = softmax_quotient(v[j + 2], rd); p3 = softmax_quotient(v[j + 3], rd);
+              for (int i = 0; i < 4; ++i) {
+                const int j = h * 16 + i * 4;
+                w[i] = __byte_perm(__byte_perm(quotient(v[j]), quotient(v[j + 1]), 0x0040),
+                                   __byte_perm(quotient(v[j + 2]), quotient(v[j + 3]), 0x0040), 0x5410);
               }
-              w[i] = ((p3 * 256u + p2) * 256u + p1) * 256u + p0;
+              *reinterpret_cast<uint4*>(sP + sw128_offset((uint32_t)row, (uint32_t)(c0 + h * 16), 128)) =
+                  make_uint4(w[0], w[1], w[2], w[3]);
             }
-            *reinterpret_cast<uint4*>(sP + sw128_offset((uint32_t)row, (uint32_t)(c0 + h * 16), 128)) =
-                make_uint4(w[0], w[1], w[2], w[3]);
           }
-        }
+        };
+        if (__all_sync(0xffffffffu, rd.pre == 0)) pass3([&](uint32_t e) { return softmax_quotient_nopre(e, rd); });
+        else pass3([&](uint32_t e) { return softmax_quotient(e, rd); });
         ptx::fence_proxy_async_smem();
       }
       // V of this pair (requested while the previous pair's epilogue ran) is needed from here on
@@ -794,7 +784,7 @@ int launch_attention(ibert_ctx* ctx, const int8_t* qkv, int B, int L, int H, int
       a.groups = std::min(std::max(n_slabs, g), std::max(Lp / 32, n_slabs));
     }
     a.q_bufs = n_slabs > 1 ? 2 : 1;
-    a.tmem_cols = cols; a.k = k; a.lens = cu_seqlens ? cu_seqlens : lens; a.out = out; a.status = ctx->d_status;
+    a.tmem_cols = cols; a.int_min = INT32_MIN; a.k = k; a.lens = cu_seqlens ? cu_seqlens : lens; a.out = out; a.status = ctx->d_status;
     const int smem = a.q_bufs * slab + 2 * n_slabs * slab + n_slabs * 128 * 128 + 2 * 4 * 128 * 4 + 64 + 1024 +
                      (cu_seqlens ? 2 * kMaxSorted : 0);      // (packed: the sequence order)
     // resident CTAs per SM: bounded by the register file (128 G threads of at most 128 registers),

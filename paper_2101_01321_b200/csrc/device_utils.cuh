@@ -176,12 +176,10 @@ __device__ __forceinline__ uint32_t iexp_dist_wide(uint32_t d, const ExpConsts& 
   const uint32_t poly = (uint32_t)(t * t + k.q_c);
   return shr_clamped(poly, z + (uint32_t)k.s_out);
 }
-// i-exp when q_ln2 = 2^k (and no pre-shift): z and r are a shift and a mask of the distance.
-// `dk` = distance + s_out 2^k, so that dk >> k = z + s_out is the final shift count directly.
-__device__ __forceinline__ uint32_t iexp_dist_pow2(uint32_t dk, int32_t q_b, int32_t q_c, uint32_t k, uint32_t mask) {
-  const int32_t t = q_b - (int32_t)(dk & mask);                          // q_b - r
-  return shr_clamped((uint32_t)(t * t + q_c), dk >> k);
-}
+// a + b on the ALU pipe (add-and-maximum against INT32_MIN, passed as a run-time value so that the compiler cannot
+// fold it): left to itself the compiler puts additions on the multiply-add pipe, which the multiply-highs of
+// i-softmax keep busy for four clocks each
+__device__ __forceinline__ int32_t add_alu(int32_t a, int32_t b, int32_t int_min) { return __viaddmax_s32(a, b, int_min); }
 // The same when quotient and post-shift come from one multiply-high (ExpConsts::fold_m): `D` = pre-shifted
 // distance + s_out q_ln2 + fold_add, `w` = q_b + fold_add - D.
 __device__ __forceinline__ uint32_t iexp_folded(uint32_t D, int32_t w, uint32_t fold_m, uint32_t q_ln2, int32_t q_c) {

@@ -123,12 +123,6 @@ int make_exp_consts(double S, int p_max, ExpConsts* k) {
     if (d_top * e0 < (uint64_t(1) << 32)) k->fold_m = (uint32_t)up;
     else if ((d_top + 1) * e1 <= (uint64_t(1) << 32)) { k->fold_m = (uint32_t)down; k->fold_add = 1; }
   }
-  k->pow2_k = -1;
-  if (s_in == 0 && (k->q_ln2 & (k->q_ln2 - 1)) == 0) {
-    int lg = 0;
-    while ((1u << lg) < k->q_ln2) ++lg;
-    k->pow2_k = lg;
-  }
   return IBERT_OK;
 }
 

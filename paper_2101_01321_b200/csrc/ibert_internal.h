@@ -32,9 +32,6 @@ struct ExpConsts {
   // floor(d / q_ln2) = umulhi(d, wide_m) >> wide_post for every d < 2^21, no clamp to d_max needed
   uint32_t wide_m;
   int32_t wide_post;
-  // k when q_ln2 = 2^k and s_in = 0 (score scale exactly ln2 / 2^k): quotient and remainder of the
-  // distance are then a shift and a mask; -1 otherwise
-  int32_t pow2_k;
   // the quotient and the post-shift in one multiply-high (attention scores): with the distance d' offset to
   // D = d' + s_out q_ln2 + fold_add,  umulhi(D, fold_m) = floor(d' / q_ln2) + s_out -- the whole shift count of
   // Algorithm 3 -- wherever e is not zero, and a count that still shifts everything out beyond.  fold_m = 0:
