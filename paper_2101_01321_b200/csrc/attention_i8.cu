@@ -502,12 +502,15 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       if (!ok) break;
       next = s_next[iter & 1];
     }
-    ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_k, kv_phase));
+    // The operand barriers are waited on by warp 0 alone, which issues the MMAs: it also requests the next operands as
+    // soon as the MMAs are done, so a warp that looked late could find the barrier two phases on and never see its
+    // own.  (The others meet it at the MMA barrier, whose phases are separated by barriers of the whole CTA.)
+    if (warp == 0) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_k, kv_phase));
     kv_phase ^= 1;
 
     for (int qt = 0; qt < q_tiles; ++qt) {
       const bool last_tile = qt == q_tiles - 1;
-      if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_q0 + 8 * qbuf, q_phase[qbuf]));
+      if (ok && warp == 0) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_q0 + 8 * qbuf, q_phase[qbuf]));
       q_phase[qbuf] ^= 1;
 
       // ---- S = Q K^T: K = 64 bytes = two MMA K-steps; N in chunks of at most 256 columns
@@ -651,7 +654,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
         ptx::fence_proxy_async_smem();
       }
       // V of this pair (requested while the previous pair's epilogue ran) is needed from here on
-      if (qt == 0 && ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_v, kv_phase ^ 1));
+      if (qt == 0 && ok && warp == 0) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_v, kv_phase ^ 1));
       ptx::tc_fence_before_sync();
       ok = __syncthreads_and(ok);             // P complete; every row's exponentials have been consumed
       if (!ok) break;
