@@ -191,6 +191,20 @@ __host__ __device__ __forceinline__ int exp_div_mode(const ExpConsts& k) {
   return k.div_pre != 0 ? 2 : (k.div_post != 0 ? 1 : 0);
 }
 
+// floor(sqrt(floor(ss / C))) = the largest s with s^2 C <= ss, one thread per value, bit by bit.
+// ss / C < 2^(bits(ss) - floor(log2 C)) bounds the highest bit that can be set, so the loop runs
+// about half the bit length of the variance.  Needs s < 2^24 and C < 2^12 (then s^2 C < 2^60).
+__device__ __forceinline__ uint32_t isqrt_of_quotient(uint64_t ss, uint32_t C) {
+  const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));   // ss / C < 2^bits
+  uint32_t s = 0;
+  for (int bit = min(max((bits + 1) >> 1, 1), 24) - 1; bit >= 0; --bit) {
+    const uint32_t cand = s | (1u << bit);
+    const uint64_t sq = (uint64_t)cand * (uint64_t)cand;
+    if (sq * (uint64_t)C <= ss) s = cand;
+  }
+  return s;
+}
+
 // floor(sqrt(floor(ss / C))), i.e. the largest s with s*s*C <= ss -- the value Algorithm 4
 // returns for n = floor(ss / C).  A 64-bit integer division costs on the order of a hundred
 // instructions here, so instead of iterating x <- (x + n/x)/2 the warp finds the same integer by

@@ -67,20 +67,6 @@ struct GemmLnArgs {
   int32_t* status;
 };
 
-// floor(sqrt(floor(ss / C))) = the largest s with s^2 C <= ss, one thread per value, bit by bit.
-// ss / C < 2^(bits(ss) - floor(log2 C)) bounds the highest bit that can be set, so the loop runs
-// about half the bit length of the variance.  Needs s < 2^24 and C < 2^12 (then s^2 C < 2^60).
-__device__ __forceinline__ uint32_t isqrt_of_quotient(uint64_t ss, uint32_t C) {
-  const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));   // ss / C < 2^bits
-  uint32_t s = 0;
-  for (int bit = min(max((bits + 1) >> 1, 1), 24) - 1; bit >= 0; --bit) {
-    const uint32_t cand = s | (1u << bit);
-    const uint64_t sq = (uint64_t)cand * (uint64_t)cand;
-    if (sq * (uint64_t)C <= ss) s = cand;
-  }
-  return s;
-}
-
 // PAIR: two CTAs (same 256 channels, adjacent 128-token tiles) share every MMA through
 // tcgen05.mma.cta_group::2 -- each loads its own token rows and half of the weight rows, which cuts
 // the bytes an SM pulls from L2 per MMA by a third (L2 bandwidth bounds the K = 3072 main loop).

@@ -369,33 +369,63 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     return;
   }
 
-  // pass 3: mean, I-Sqrt of the variance, normalize, affine + requantize, store
-  const int32_t bb[4] = {bv.x, bv.y, bv.z, bv.w};
-  const int64_t BB[4] = {B01.x, B01.y, B23.x, B23.y};
+  // pass 3: mean and I-Sqrt of the variance (sum (v - mu)^2 = sum v^2 - 2 mu sum v + C mu^2 in integers).  One token
+  // per warp: the warp together, a round of the root's search tests 32 candidates -- the shortest chain.  More
+  // tokens: a thread per token, because the warp form repeats some 200 instructions for every token and CTA
+  // (95 instructions per element at 48 tokens); encoder layer Large B = 7, L = 128 43.0 -> 40.4 us, Base B = 8,
+  // L = 77 30.1 -> 29.7.
   const int C = a.N;
-#pragma unroll
-  for (int j = 0; j < TPW; ++j) {
-    const int t = warp * TPW + j;
+  auto mean_of = [&](int32_t sum) { return (int32_t)(__umulhi((uint32_t)(sum + (C << 18)), a.c_magic) >> a.c_shift) - (1 << 18); };
+  // {mu, floor(2^31 / sigma), shift}; sigma <= 1: 2^30 and one shift less
+  auto params_of = [](int32_t mu, uint32_t sigma) {
+    return make_int4(mu, sigma > 1u ? (int32_t)(0x80000000u / sigma) : (1 << 30), sigma > 1u ? 15 : 14, 0);
+  };
+  int4 one = make_int4(0, 0, 0, 0);
+  if constexpr (TPW == 1) {
     uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
     if (lane < cl)
       asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(p0), "=r"(p1), "=r"(p2), "=r"(p3)
-                   : "r"(s_part + (uint32_t)((lane * a.nt + t) * 16)));
+                   : "r"(s_part + (uint32_t)((lane * a.nt + warp) * 16)));
     const int32_t sum = __reduce_add_sync(0xffffffffu, (int32_t)p0);
     // (at most eight records with low words below 2^30: their 16-bit halves reduce as 32-bit sums)
     const uint64_t sumsq = (uint64_t)__reduce_add_sync(0xffffffffu, p1 & 0xffffu) +
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p1 >> 16) << 16) +
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p2) << 25);
-    const int32_t mu = (int32_t)(__umulhi((uint32_t)(sum + (C << 18)), a.c_magic) >> a.c_shift) - (1 << 18);   // floor(sum / C)
-    const uint64_t ss = sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum));
-    const uint32_t sigma = warp_isqrt_of_quotient(ss, (uint32_t)C, lane);
-    // floor(2^31 / sigma); sigma <= 1: 2^30 and one shift less
-    const int32_t rho = sigma > 1u ? (int32_t)(0x80000000u / sigma) : (1 << 30);
-    const uint32_t nsh = sigma > 1u ? 15u : 14u;
+    const int32_t mu = mean_of(sum);
+    one = params_of(mu, warp_isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, lane));
+  } else {
+    if ((int)threadIdx.x < a.nt) {
+      int32_t sum = 0;
+      uint64_t sumsq = 0;
+#pragma unroll 2
+      for (int r = 0; r < cl; ++r) {
+        uint32_t p0, p1, p2, p3;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(p0), "=r"(p1), "=r"(p2), "=r"(p3)
+                     : "r"(s_part + (uint32_t)((r * a.nt + (int)threadIdx.x) * 16)));
+        sum += (int32_t)p0;
+        sumsq += (uint64_t)p1 + ((uint64_t)p2 << 25);
+      }
+      const int32_t mu = mean_of(sum);
+      const int4 pr = params_of(mu, isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C));
+      // (the token's own records are consumed: the first one's place takes the result)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(s_part + threadIdx.x * 16), "r"(pr.x), "r"(pr.y), "r"(pr.z), "r"(0) : "memory");
+    }
+    __syncthreads();
+  }
+  // pass 4: normalize, affine + requantize, store
+  const int32_t bb[4] = {bv.x, bv.y, bv.z, bv.w};
+  const int64_t BB[4] = {B01.x, B01.y, B23.x, B23.y};
+#pragma unroll
+  for (int j = 0; j < TPW; ++j) {
+    const int t = warp * TPW + j;
+    int4 pr = one;
+    if constexpr (TPW > 1)
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pr.x), "=r"(pr.y), "=r"(pr.z), "=r"(pr.w) : "r"(s_part + (uint32_t)(t * 16)));
     int32_t o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int64_t pr = (int64_t)(v[j][i] - mu) * (int64_t)rho;
-      const int32_t nrm = (int32_t)__funnelshift_r((uint32_t)pr, (uint32_t)(pr >> 32), nsh) << ln.out_sh;
+      const int64_t x = (int64_t)(v[j][i] - pr.x) * (int64_t)pr.y;
+      const int32_t nrm = (int32_t)__funnelshift_r((uint32_t)x, (uint32_t)(x >> 32), (uint32_t)pr.z) << ln.out_sh;
       o[i] = max(requant_upper_add(nrm, bb[i], BB[i]), -127);
     }
     if (t0 + t < a.T)
@@ -490,6 +520,9 @@ SmallArgs small_args(ibert_ctx* ctx, int64_t M, int N, int K, int nt, int extra_
   a.T = (int)M; a.N = N; a.K = K; a.nt = nt;
   const int stage = kWBytes + nt * kBK, k_blocks = (K + kBK - 1) / kBK;
   a.stages = std::min({k_blocks, kMaxStages, (kSmemLimit - kBarBytes - 1024 - extra_smem) / stage});
+  // a stage that is filled again must stay with one issuer: the other could reach it before its first filling and
+  // take the barrier's initial phase for the second one
+  if (a.stages < k_blocks) a.stages -= a.stages % kIssuers;
   a.w_static = epi.w_static ? 1 : 0;
   a.tmem_cols = tmem_columns(kIssuers * nt);
   a.b = epi.d_b; a.c = epi.d_c; a.bias = epi.d_bias; a.gelu = epi.gelu; a.out = out; a.status = ctx->d_status;
