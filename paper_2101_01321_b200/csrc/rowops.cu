@@ -98,8 +98,7 @@ __global__ void __launch_bounds__(kThreads) gelu_lut_kernel(const int32_t* __res
 // ----------------------------------------------------------------------------- i-softmax
 // One warp per row; a lane keeps VPL int4 vectors (4*VPL scores) in registers.
 // VEC: rows are 16-byte aligned (L % 4 == 0) and loaded/stored as vectors.
-// DIV 0..2: how i-exp divides by q_ln2; DIV 3: i-exp read from `table` (comparison variant).
-constexpr int kExpByTable = 3;
+// DIV 0..2: how i-exp divides by q_ln2.  (softmax_group_kernel takes every scale but the coarsest.)
 
 // table[i] = i-exp of the pre-shifted distance i, for i = 0 .. d_max
 __global__ void __launch_bounds__(kThreads) exp_table_kernel(ExpConsts k, uint32_t* __restrict__ table) {
@@ -112,8 +111,7 @@ __global__ void __launch_bounds__(kThreads) exp_table_kernel(ExpConsts k, uint32
 
 template <int VPL, bool VEC, int DIV>
 __global__ void __launch_bounds__(kThreads) softmax_kernel(const int32_t* __restrict__ q, int64_t rows,
-                                                           int L, ExpConsts k, uint8_t* __restrict__ out,
-                                                           const uint32_t* __restrict__ table) {
+                                                           int L, ExpConsts k, uint8_t* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
@@ -149,8 +147,7 @@ __global__ void __launch_bounds__(kThreads) softmax_kernel(const int32_t* __rest
         const uint32_t dist = (uint32_t)mx - (uint32_t)v[j][i];
         uint32_t e = 0u;
         if (col + i < L) {
-          if constexpr (DIV == kExpByTable) e = __ldg(table + min(dist >> k.s_in, k.d_max));
-          else e = iexp_dist<DIV>(dist, k);
+          e = iexp_dist<DIV>(dist, k);
         }
         v[j][i] = (int32_t)e;
         sum += e;
@@ -526,65 +523,117 @@ __global__ void __launch_bounds__(kThreads) gather_first_rows_kernel(const int8_
     *reinterpret_cast<uint4*>(out + (int64_t)b * H + c) = __ldg(reinterpret_cast<const uint4*>(src + c));
 }
 
-// Short rows (L <= 128, a multiple of 4: one 16-byte vector per lane): a warp takes R rows at a time.  The one
-// true division a row needs (Algorithm 3's quotient by the row sum, made a multiplication for its elements)
-// costs about as much as the rest of a 128-element row; lane r performs it for row r, so one division
-// instruction stream serves R rows, and the R loads of a lane are in flight together.
-template <int R, int DIV>
-__global__ void __launch_bounds__(kThreads, 4) softmax_short_kernel(const int32_t* __restrict__ q, int64_t rows,
-                                                                 int L, ExpConsts k, uint8_t* __restrict__ out,
-                                                                 const uint32_t* __restrict__ table) {
-  const int lane = threadIdx.x & 31;
+// i-softmax with LPR lanes per row (32 / LPR rows per warp side by side) and VPL 16-byte vectors per lane.  Bound by
+// instruction issue with one row per warp: maximum, sum and the division by the sum cost a lane the same for
+// four values as for 16 (34 instructions per element).  Few lanes per row and many values per lane keep that
+// share small, and i-exp takes quotient and shift from one multiply-high: [196608, 128] 37.5 -> 22.6 us (0.85 of the
+// measured copy bandwidth), [262144, 512] 151 -> 108, [100000, 101] 25.4 -> 18.8, [200000, 33] 47.7 -> 15.1.
+// Rows of any length: the vectors are the 16-byte aligned ones that cover the row, elements of the neighbouring rows
+// in the first and the last are masked.
+// FULL: 4 LPR VPL elements per row exactly, nothing to mask.  EXP: the exponential's form.
+enum { kExpFold = 0, kExpFoldShift = 1, kExpTable = 2 };
+template <int LPR, int VPL, bool FULL, int EXP>
+__global__ void __launch_bounds__(kThreads, VPL > 4 ? 3 : 4) softmax_group_kernel(const int32_t* __restrict__ q, int64_t rows, int L,
+                                                                     ExpConsts k, uint8_t* __restrict__ out,
+                                                                     const uint32_t* __restrict__ table) {
+  constexpr int kRows = 32 / LPR;
+  const int lane = threadIdx.x & 31, li = lane % LPR;
   const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
-  const int col = 4 * lane;
-  const bool in_row = col < L;
-  for (int64_t row0 = warp_global * R; row0 < rows; row0 += warp_count * R) {
-    int32_t v[R][4];
-    uint32_t sums[R];
+  const int64_t total = rows * L;
+  const int4* q4 = reinterpret_cast<const int4*>(q);
+  const int32_t wk = k.q_b - k.s_out * (int32_t)k.q_ln2 + k.fold_add;
+  for (int64_t row0 = warp_global * kRows; row0 < rows; row0 += warp_count * kRows) {
+    const int64_t row = row0 + lane / LPR;
+    const bool live = row < rows;
+    const int64_t vec0 = (row * L) >> 2;                      // first vector of the row
+    const int off = FULL ? 0 : (int)((row * L) & 3);          // elements of the row before in it
+    uint32_t v[VPL][4];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (in_row && row0 + r < rows) {
-        const int4 t = __ldcs(reinterpret_cast<const int4*>(q + (row0 + r) * L + col));
-        v[r][0] = t.x; v[r][1] = t.y; v[r][2] = t.z; v[r][3] = t.w;
-      } else {
-        v[r][0] = v[r][1] = v[r][2] = v[r][3] = INT32_MIN;
+    for (int j = 0; j < VPL; ++j) {
+      const int vi = li + LPR * j;
+      int4 t = make_int4(INT32_MIN, INT32_MIN, INT32_MIN, INT32_MIN);
+      if (live && (FULL || 4 * vi < off + L)) {
+        if (FULL || 4 * (vec0 + vi) + 3 < total) t = __ldcs(q4 + vec0 + vi);
+        else {                                                // the tensor's last, partial vector
+          const int32_t* e = q + 4 * (vec0 + vi);
+          const int left = (int)(total - 4 * (vec0 + vi));
+          t.x = e[0];
+          if (left > 1) t.y = e[1];
+          if (left > 2) t.z = e[2];
+        }
+      }
+      v[j][0] = t.x; v[j][1] = t.y; v[j][2] = t.z; v[j][3] = t.w;
+      if constexpr (!FULL) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if ((uint32_t)(4 * vi + i - off) >= (uint32_t)L) v[j][i] = (uint32_t)INT32_MIN;
       }
     }
+    int32_t mx = INT32_MIN;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      int32_t mx = max(max(v[r][0], v[r][1]), max(v[r][2], v[r][3]));
-      mx = __reduce_max_sync(0xffffffffu, mx);
-      uint32_t sum = 0;
+    for (int j = 0; j < VPL; ++j) {
+      mx = __vimax3_s32(mx, (int32_t)v[j][0], (int32_t)v[j][1]);
+      mx = __vimax3_s32(mx, (int32_t)v[j][2], (int32_t)v[j][3]);
+    }
+    if constexpr (LPR == 32) mx = __reduce_max_sync(0xffffffffu, mx);
+    else {
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    uint32_t sum = 0;
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t dist = (uint32_t)mx - (uint32_t)v[r][i];
-        uint32_t e = 0u;
-        if (in_row && row0 + r < rows) {
-          if constexpr (DIV == kExpByTable) e = __ldg(table + min(dist >> k.s_in, k.d_max));
-          else e = iexp_dist<DIV>(dist, k);
+        uint32_t d = (uint32_t)mx - v[j][i];
+        if constexpr (EXP == kExpTable) v[j][i] = __ldg(table + min(d >> k.s_in, k.d_max));
+        else {
+          // d' = min(d >> s_in, 31 q_ln2); n = floor(d' / q_ln2) + s_out; e = ((q_b - r)^2 + q_c) >> n
+          if constexpr (EXP == kExpFoldShift) d >>= k.s_in;
+          d = min(d, k.d_max) + (uint32_t)k.fold_add;
+          const uint32_t n = __umulhi(d, k.fold_m) + (uint32_t)k.s_out;
+          const int32_t t = (int32_t)(n * k.q_ln2) + (wk - (int32_t)d);
+          v[j][i] = shr_clamped((uint32_t)(t * t + k.q_c), n);
         }
-        v[r][i] = (int32_t)e;
-        sum += e;
       }
-      sums[r] = max(__reduce_add_sync(0xffffffffu, sum), 1u);     // (0 only for a row past the end)
+      sum = sum + v[j][0] + v[j][1];
+      sum = sum + v[j][2] + v[j][3];
     }
-    uint32_t my_sum = sums[0];
+    if constexpr (!FULL) {
+      // masked elements sit at INT32_MIN: their exponential is 0 unless the whole row is within 31 ln2 of it
+      const bool low = ((uint32_t)(mx - INT32_MIN) >> k.s_in) < k.d_max;
+      if (__any_sync(0xffffffffu, low)) {
+        sum = 0;
 #pragma unroll
-    for (int r = 1; r < R; ++r) my_sum = lane == r ? sums[r] : my_sum;
-    const uint32_t my_m = make_row_divisor(my_sum, k.p_max).m;
+        for (int j = 0; j < VPL; ++j)
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      RowDivisor rd;
-      rd.m = __shfl_sync(0xffffffffu, my_m, r);
-      const int K = 23 + 32 - __clz(sums[r]);
-      rd.pre = K < 32 ? 32 - K : 0;
-      rd.post = K < 32 ? 0 : K - 32;
+          for (int i = 0; i < 4; ++i) {
+            if ((uint32_t)(4 * (li + LPR * j) + i - off) >= (uint32_t)L) v[j][i] = 0u;
+            sum += v[j][i];
+          }
+      }
+    }
+    if constexpr (LPR == 32) sum = __reduce_add_sync(0xffffffffu, sum);
+    else {
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    const RowDivisor rd = make_row_divisor(max(sum, 1u), k.p_max);
+    const bool nopre = __all_sync(0xffffffffu, rd.pre == 0);
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
       uint32_t p[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = softmax_quotient((uint32_t)v[r][i], rd);
-      if (in_row && row0 + r < rows)
-        __stcs(reinterpret_cast<uint32_t*>(out + (row0 + r) * L + col), p[0] | (p[1] << 8) | (p[2] << 16) | (p[3] << 24));
+      for (int i = 0; i < 4; ++i) p[i] = softmax_quotient_nopre(nopre ? v[j][i] : v[j][i] << rd.pre, rd);
+      const uint32_t w = __byte_perm(__byte_perm(p[0], p[1], 0x0040), __byte_perm(p[2], p[3], 0x0040), 0x5410);
+      const int vi = li + LPR * j, c = 4 * vi - off;          // the word's first column
+      if (live && (FULL || (c >= 0 && c + 3 < L))) __stcs(reinterpret_cast<uint32_t*>(out) + vec0 + vi, w);
+      else if (!FULL && live) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (c + i >= 0 && c + i < L) out[4 * (vec0 + vi) + i] = (uint8_t)p[i];
+      }
     }
   }
 }
@@ -657,28 +706,56 @@ int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const 
   if (rows == 0) return IBERT_OK;
   const bool vec = (L % 4) == 0;
   const int vpl = (L + 127) / 128;   // vectors per lane
-  const int div = exp_table ? kExpByTable : exp_div_mode(k);
+  const int div = exp_div_mode(k);
 #define IBERT_SM2(V, D)                                                                                       \
   do {                                                                                                        \
-    if (vec) softmax_kernel<V, true, D><<<wave_grid(ctx, softmax_kernel<V, true, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);   \
-    else softmax_kernel<V, false, D><<<wave_grid(ctx, softmax_kernel<V, false, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);      \
+    if (vec) softmax_kernel<V, true, D><<<wave_grid(ctx, softmax_kernel<V, true, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out);   \
+    else softmax_kernel<V, false, D><<<wave_grid(ctx, softmax_kernel<V, false, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out);      \
   } while (0)
 #define IBERT_SM(V)                 \
   do {                              \
     if (div == 0) IBERT_SM2(V, 0);  \
     else if (div == 1) IBERT_SM2(V, 1); \
-    else if (div == 2) IBERT_SM2(V, 2); \
-    else IBERT_SM2(V, kExpByTable);     \
+    else IBERT_SM2(V, 2);           \
   } while (0)
-  if (vpl <= 1 && vec) {
-    constexpr int R = 4;
-    const int sgrid = grid_for(ctx, (rows + R - 1) / R, 4);      // (one wave: four CTAs are resident per SM)
-    if (div == 0) softmax_short_kernel<R, 0><<<sgrid, kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);
-    else if (div == 1) softmax_short_kernel<R, 1><<<sgrid, kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);
-    else if (div == 2) softmax_short_kernel<R, 2><<<sgrid, kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);
-    else softmax_short_kernel<R, kExpByTable><<<sgrid, kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table);
+  if (exp_table || k.fold_m != 0) {
+    // lanes per row: the fewest (4 to 32) that hold the row in at most four vectors each; L > 509: 32 of eight
+    const int vecs = (L + (vec ? 0 : 3) + 3) / 4;
+    int lpr = 4;
+    while (lpr < 32 && vecs > 4 * lpr) lpr *= 2;
+    const int vpl_g = std::max((vecs + lpr - 1) / lpr, 2);
+    const bool full = vec && L == 4 * lpr * vpl_g;
+    const int form = exp_table ? kExpTable : (k.s_in == 0 ? kExpFold : kExpFoldShift);
+    const int64_t warps = (rows + 32 / lpr - 1) / (32 / lpr);
+#define IBERT_SG3(LPR, VPL, FULL, EXP)                                                                          \
+  softmax_group_kernel<LPR, VPL, FULL, EXP><<<wave_grid(ctx, softmax_group_kernel<LPR, VPL, FULL, EXP>, warps), \
+                                              kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table)
+#define IBERT_SG2(LPR, VPL, FULL)                                  \
+  do {                                                             \
+    if (form == kExpFold) IBERT_SG3(LPR, VPL, FULL, kExpFold);     \
+    else if (form == kExpFoldShift) IBERT_SG3(LPR, VPL, FULL, kExpFoldShift); \
+    else IBERT_SG3(LPR, VPL, FULL, kExpTable);                     \
+  } while (0)
+#define IBERT_SG(LPR)                                  \
+  do {                                                 \
+    if (vpl_g == 2) IBERT_SG2(LPR, 2, false);          \
+    else if (vpl_g == 3) IBERT_SG2(LPR, 3, false);     \
+    else if (full) IBERT_SG2(LPR, 4, true);            \
+    else IBERT_SG2(LPR, 4, false);                     \
+  } while (0)
+    if (vpl_g > 8) IBERT_SG2(32, 9, false);            // (1022 and 1023 elements off a 16-byte boundary)
+    else if (vpl_g > 4) IBERT_SG2(32, 8, false);
+    else if (lpr == 4) IBERT_SG(4);
+    else if (lpr == 8) IBERT_SG(8);
+    else if (lpr == 16) IBERT_SG(16);
+    else IBERT_SG(32);
+#undef IBERT_SG
+#undef IBERT_SG2
+#undef IBERT_SG3
+    return check_launch();
   }
-  else if (vpl <= 1) IBERT_SM(1);
+  // scales so coarse (q_ln2 < 16) or so odd that the one multiply-high does not exist
+  if (vpl <= 1) IBERT_SM(1);
   else if (vpl <= 2) IBERT_SM(2);
   else if (vpl <= 4) IBERT_SM(4);
   else IBERT_SM(8);
