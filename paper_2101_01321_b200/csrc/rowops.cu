@@ -18,6 +18,8 @@ constexpr int kThreads = 256;
 // after vector j-1 so that every load and store instruction of a warp is contiguous.
 __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restrict__ q, int64_t n,
                                                         GeluConsts k, int8_t* __restrict__ out) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
   const int64_t half = rounding_half(k.c);
   const int64_t n_vec = n >> 2;
   const int32_t rnd_f = (1 << k.s_f) - 1;
@@ -540,6 +542,8 @@ __global__ void __launch_bounds__(kThreads, VPL > 4 ? 3 : 4) softmax_group_kerne
   const int lane = threadIdx.x & 31, li = lane % LPR;
   const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
   const int64_t total = rows * L;
   const int4* q4 = reinterpret_cast<const int4*>(q);
   const int32_t wk = k.q_b - k.s_out * (int32_t)k.q_ln2 + k.fold_add;
@@ -692,8 +696,7 @@ int launch_gelu_lut(ibert_ctx* ctx, const int32_t* q, int64_t n, const int8_t* t
 int launch_gelu(ibert_ctx* ctx, const int32_t* q, int64_t n, const GeluConsts& k, int8_t* out) {
   if (n == 0) return IBERT_OK;
   const int64_t warps = ((n >> 2) + 127) / 128 + 1;
-  gelu_kernel<<<wave_grid(ctx, gelu_kernel, warps), kThreads, 0, ctx->stream>>>(q, n, k, out);
-  return check_launch();
+  return launch_pdl(gelu_kernel, dim3(wave_grid(ctx, gelu_kernel, warps)), dim3(kThreads), 0, ctx->stream, 1, q, n, k, out);
 }
 
 int launch_exp_table(ibert_ctx* ctx, const ExpConsts& k, uint32_t* table) {
@@ -728,8 +731,9 @@ int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const 
     const int form = exp_table ? kExpTable : (k.s_in == 0 ? kExpFold : kExpFoldShift);
     const int64_t warps = (rows + 32 / lpr - 1) / (32 / lpr);
 #define IBERT_SG3(LPR, VPL, FULL, EXP)                                                                          \
-  softmax_group_kernel<LPR, VPL, FULL, EXP><<<wave_grid(ctx, softmax_group_kernel<LPR, VPL, FULL, EXP>, warps), \
-                                              kThreads, 0, ctx->stream>>>(q, rows, L, k, out, exp_table)
+  return launch_pdl(softmax_group_kernel<LPR, VPL, FULL, EXP>,                                                  \
+                    dim3(wave_grid(ctx, softmax_group_kernel<LPR, VPL, FULL, EXP>, warps)), dim3(kThreads), 0,   \
+                    ctx->stream, 1, q, rows, L, k, out, exp_table)
 #define IBERT_SG2(LPR, VPL, FULL)                                  \
   do {                                                             \
     if (form == kExpFold) IBERT_SG3(LPR, VPL, FULL, kExpFold);     \
@@ -749,10 +753,10 @@ int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const 
     else if (lpr == 8) IBERT_SG(8);
     else if (lpr == 16) IBERT_SG(16);
     else IBERT_SG(32);
+    return IBERT_ERR_ARG;
 #undef IBERT_SG
 #undef IBERT_SG2
 #undef IBERT_SG3
-    return check_launch();
   }
   // scales so coarse (q_ln2 < 16) or so odd that the one multiply-high does not exist
   if (vpl <= 1) IBERT_SM(1);
