@@ -145,7 +145,7 @@ def ibert_layernorm_i_static(q: torch.Tensor, S: float, r: torch.Tensor | None, 
     rows = q.numel() // Cn if Cn else 0
     g, b = _host(gamma, np.float64), _host(beta, np.float64)
     if out is None:
-        out = torch.empty(q.shape, dtype=torch.int8, device=q.device)
+        out = q.new_empty(q.shape, dtype=torch.int8)
     S_ret = C.c_double()
     sp = None if stream is None else stream.cuda_stream
     _chk(lib().ibert_layernorm_i_static(sp, _dev(q, torch.int32), S, _dev(r, torch.int8), S_r or 0.0,
@@ -221,7 +221,7 @@ class Context:
     # ------------------------------------------------------------------ simple ops
     def ibert_gelu_i(self, q: torch.Tensor, S: float, S_out: float, out: torch.Tensor | None = None):
         if out is None:
-            out = torch.empty(q.shape, dtype=torch.int8, device=q.device)
+            out = q.new_empty(q.shape, dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_gelu_i(self.h, _dev(q, torch.int32), S, q.numel(), S_out, _dev(out, torch.int8),
                                 C.byref(S_ret)), "ibert_gelu_i")
@@ -230,7 +230,7 @@ class Context:
     def ibert_gelu_lut_i(self, q: torch.Tensor, S: float, S_out: float, out: torch.Tensor | None = None):
         """i-GELU through a look-up table built from the integer kernel (comparison only)."""
         if out is None:
-            out = torch.empty(q.shape, dtype=torch.int8, device=q.device)
+            out = q.new_empty(q.shape, dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_gelu_lut_i(self.h, _dev(q, torch.int32), S, q.numel(), S_out, _dev(out, torch.int8),
                                     C.byref(S_ret)), "ibert_gelu_lut_i")
@@ -239,7 +239,7 @@ class Context:
     def ibert_hgelu_i(self, q: torch.Tensor, S: float, S_out: float, out: torch.Tensor | None = None):
         """Integer h-GELU (Eq. 6), the paper's comparison function."""
         if out is None:
-            out = torch.empty(q.shape, dtype=torch.int8, device=q.device)
+            out = q.new_empty(q.shape, dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_hgelu_i(self.h, _dev(q, torch.int32), S, q.numel(), S_out, _dev(out, torch.int8),
                                  C.byref(S_ret)), "ibert_hgelu_i")
@@ -250,7 +250,7 @@ class Context:
         L = q.shape[-1]
         rows = q.numel() // L if L else 0
         if out is None:
-            out = torch.empty(q.shape, dtype=torch.uint8, device=q.device)
+            out = q.new_empty(q.shape, dtype=torch.uint8)
         S_ret = C.c_double()
         _chk(getattr(lib(), _entry)(self.h, _dev(q, torch.int32), S, rows, L, p_max, _dev(out, torch.uint8),
                                     C.byref(S_ret)), _entry)
@@ -267,7 +267,7 @@ class Context:
         g, b = _host(gamma, np.float64), _host(beta, np.float64)
         assert g.size == Cn and b.size == Cn
         if out is None:
-            out = torch.empty(q.shape, dtype=torch.int8, device=q.device)
+            out = q.new_empty(q.shape, dtype=torch.int8)
         S_ret = C.c_double()
         if q.dtype == torch.int16:           # Q16 values in an int16 container
             _chk(lib().ibert_layernorm_i16(self.h, _dev(q, torch.int16), S, _dev(r, torch.int8), S_r or 0.0,
@@ -288,8 +288,7 @@ class Context:
         sw = _host(S_w, np.float64)
         assert sw.size == N
         if out is None:
-            out = torch.empty(x.shape[:-1] + (N,), device=x.device,
-                              dtype={0: torch.int8, 3: torch.int16}.get(out_kind, torch.int32))
+            out = x.new_empty(x.shape[:-1] + (N,), dtype={0: torch.int8, 3: torch.int16}.get(out_kind, torch.int32))
         S_ret = np.zeros(N if out_kind == 2 else 1, dtype=np.float64)
         _chk(lib().ibert_linear_i8(self.h, _dev(x, torch.int8), S_x, _dev(w, torch.int8), sw.ctypes.data,
                                    _dev(bias, torch.int32), M, N, K, out_kind, S_out, out.data_ptr(),
@@ -303,7 +302,7 @@ class Context:
         N = w.shape[0]
         sw = _host(S_w, np.float64)
         if out is None:
-            out = torch.empty(x.shape[:-1] + (N,), dtype=torch.int8, device=x.device)
+            out = x.new_empty(x.shape[:-1] + (N,), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_linear_hgelu_i8(self.h, _dev(x, torch.int8), S_x, _dev(w, torch.int8), sw.ctypes.data,
                                          _dev(bias, torch.int32), M, N, K, S_mid, S_out, _dev(out, torch.int8),
@@ -322,7 +321,7 @@ class Context:
         g, b = _host(gamma, np.float64), _host(beta, np.float64)
         assert sw.size == N and g.size == N and b.size == N
         if out is None:
-            out = torch.empty(x.shape[:-1] + (N,), dtype=torch.int8, device=x.device)
+            out = x.new_empty(x.shape[:-1] + (N,), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_linear_layernorm_i8(self.h, _dev(x, torch.int8), S_x, _dev(w, torch.int8), sw.ctypes.data,
                                              _dev(bias, torch.int32), M, N, K, S_mid, _dev(res, torch.int8), S_res,
@@ -337,7 +336,7 @@ class Context:
         N = w.shape[0]
         sw = _host(S_w, np.float64)
         if out is None:
-            out = torch.empty(x.shape[:-1] + (N,), dtype=torch.int8, device=x.device)
+            out = x.new_empty(x.shape[:-1] + (N,), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_linear_gelu_i8(self.h, _dev(x, torch.int8), S_x, _dev(w, torch.int8), sw.ctypes.data,
                                         _dev(bias, torch.int32), M, N, K, S_mid, S_out, _dev(out, torch.int8),
@@ -348,7 +347,7 @@ class Context:
                            S_v: float, S_ctx: float, p_max: int = 255, out: torch.Tensor | None = None):
         assert qkv.numel() == B * L * 3 * H
         if out is None:
-            out = torch.empty((B * L, H), dtype=torch.int8, device=qkv.device)
+            out = qkv.new_empty((B * L, H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_attention_i8(self.h, _dev(qkv, torch.int8), B, L, H, heads, S_q, S_k, S_v, S_ctx, p_max,
                                       _dev(out, torch.int8), C.byref(S_ret)), "ibert_attention_i8")
@@ -360,7 +359,7 @@ class Context:
         """Attention with a key-padding mask; ``lens``: device int32 [B], valid keys per sequence."""
         assert qkv.numel() == B * L * 3 * H and lens.numel() == B
         if out is None:
-            out = torch.empty((B * L, H), dtype=torch.int8, device=qkv.device)
+            out = qkv.new_empty((B * L, H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_attention_masked_i8(self.h, _dev(qkv, torch.int8), B, L, H, heads, _dev(lens, torch.int32),
                                              S_q, S_k, S_v, S_ctx, p_max, _dev(out, torch.int8), C.byref(S_ret)),
@@ -406,7 +405,7 @@ class Context:
         B = cu_seqlens.numel() - 1
         total = qkv.numel() // (3 * H)
         if out is None:
-            out = torch.empty((total, H), dtype=torch.int8, device=qkv.device)
+            out = qkv.new_empty((total, H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_attention_packed_i8(self.h, _dev(qkv, torch.int8), _dev(cu_seqlens, torch.int32), B, max_len,
                                              total, H, heads, S_q, S_k, S_v, S_ctx, p_max, _dev(out, torch.int8),
@@ -419,7 +418,7 @@ class Context:
         B = cu_seqlens.numel() - 1
         total = x.numel() // layer.H
         if out is None:
-            out = torch.empty((total, layer.H), dtype=torch.int8, device=x.device)
+            out = x.new_empty((total, layer.H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_encoder_layer_packed(self.h, layer.h, _dev(x, torch.int8), _dev(cu_seqlens, torch.int32), B,
                                               max_len, total, _dev(out, torch.int8), C.byref(S_ret)),
@@ -462,7 +461,7 @@ class Context:
     def ibert_encoder_layer(self, layer: "Layer", x: torch.Tensor, B: int, L: int,
                             out: torch.Tensor | None = None):
         if out is None:
-            out = torch.empty((B * L, layer.H), dtype=torch.int8, device=x.device)
+            out = x.new_empty((B * L, layer.H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_encoder_layer(self.h, layer.h, _dev(x, torch.int8), B, L, _dev(out, torch.int8),
                                        C.byref(S_ret)), "ibert_encoder_layer")
@@ -473,7 +472,7 @@ class Context:
         """The encoder layer on padded sequences; ``lens``: device int32 [B], valid keys per sequence."""
         assert lens.numel() == B
         if out is None:
-            out = torch.empty((B * L, layer.H), dtype=torch.int8, device=x.device)
+            out = x.new_empty((B * L, layer.H), dtype=torch.int8)
         S_ret = C.c_double()
         _chk(lib().ibert_encoder_layer_masked(self.h, layer.h, _dev(x, torch.int8), B, L, _dev(lens, torch.int32),
                                               _dev(out, torch.int8), C.byref(S_ret)), "ibert_encoder_layer_masked")

@@ -465,8 +465,9 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
   if (int rc = trim_tables(ctx)) return rc;
   if (kind != EPI_RAW) {
     const double S_acc_to = (kind == EPI_GELU || kind == EPI_HGELU) ? S_mid : S_out;
-    std::vector<int32_t> b, c;
-    int rc = make_linear_tables(S_x, S_w, N, nullptr, S_acc_to, &b, &c);
+    std::vector<int32_t> b, c, upper;
+    bool fits = false;
+    int rc = make_linear_tables(S_x, S_w, N, nullptr, S_acc_to, &b, &c, &upper, &fits);
     if (rc) return rc;
     // The epilogue runs in ONE form: the upper-word form needs the per-channel multipliers AND (for
     // the GELU kinds) the final multiplier to fit it.  The per-channel table is converted only then --
@@ -477,7 +478,8 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
       if (rc) return rc;
       upper_ok = epi.gelu.fast != 0;
     }
-    epi.fast = (upper_ok && to_upper_word_form(&b, c)) ? 1 : 0;
+    epi.fast = (upper_ok && fits) ? 1 : 0;
+    if (epi.fast) b.swap(upper);
     // i-GELU by table (the tile shapes with room for it use it)
     if (kind == EPI_GELU && epi.fast && ctx->gelu_table_mode == 0)
       if ((rc = cached_gelu_table(ctx, epi.gelu, &epi.gelu_table))) return rc;
@@ -561,10 +563,12 @@ int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const
   GemmEpilogue epi{};
   epi.kind = EPI_Q16;
   epi.d_bias = bias;
-  std::vector<int32_t> b, c;
-  int rc = make_linear_tables(S_x, S_w, N, nullptr, S_mid, &b, &c);
+  std::vector<int32_t> b, c, upper;
+  bool fits = false;
+  int rc = make_linear_tables(S_x, S_w, N, nullptr, S_mid, &b, &c, &upper, &fits);
   if (rc) return rc;
-  epi.fast = to_upper_word_form(&b, c) ? 1 : 0;
+  epi.fast = fits ? 1 : 0;
+  if (fits) b.swap(upper);
   LnConsts k{};
   k.C = N;
   k.has_res = 1;
@@ -722,10 +726,12 @@ int ibert_layer_create(ibert_ctx* ctx, const ibert_layer_desc* d, ibert_layer** 
   auto lin = [&](double S_in, const double* S_w, int N, const double* so_cols, double so, int32_t** db, int32_t** dc,
                  int* fast, bool upper_ok = true, int64_t max_acc = 0) {
     if (rc != IBERT_OK) return;
-    std::vector<int32_t> b, c;
-    rc = make_linear_tables(S_in, S_w, N, so_cols, so, &b, &c);
+    std::vector<int32_t> b, c, upper;
+    bool fits = false;
+    rc = make_linear_tables(S_in, S_w, N, so_cols, so, &b, &c, &upper, &fits);
     if (rc != IBERT_OK) return;
-    *fast = (upper_ok && to_upper_word_form(&b, c)) ? 1 : 0;
+    *fast = (upper_ok && fits) ? 1 : 0;
+    if (*fast) b.swap(upper);
     if (!*fast && upper_ok && max_acc > 0 && to_upper_word_wide(&b, &c, max_acc)) *fast = 2;
     up(b.data(), b.size() * sizeof(int32_t), (void**)db);
     up(c.data(), c.size() * sizeof(int32_t), (void**)dc);

@@ -13,6 +13,13 @@
 
 #include "ibert_internal.h"
 
+// array loops in an AVX2 version beside the baseline one, chosen when the library is loaded
+#if defined(__x86_64__) && defined(__GNUC__) && !defined(__clang__)
+#define IBERT_HOST_SIMD __attribute__((target_clones("avx2", "default"), optimize("O3")))
+#else
+#define IBERT_HOST_SIMD
+#endif
+
 namespace ibert {
 
 namespace {
@@ -248,6 +255,10 @@ bool to_upper_word_wide(std::vector<int32_t>* b, std::vector<int32_t>* c, int64_
   return true;
 }
 
+IBERT_HOST_SIMD static void scaled_addends(const double* beta, double S_out, double two_c, int n, double* x) {
+  for (int i = 0; i < n; ++i) x[i] = (beta[i] / S_out) * two_c + 0.5;
+}
+
 // LayerNorm affine + requantization folded into one dyadic step per channel: the
 // normalized value n ~ y_hat * 2^16, out = (n * b_i + B_i) >> c with a shared c.
 int make_ln_tables(const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
@@ -266,9 +277,11 @@ int make_ln_tables(const double* gamma, const double* beta, int C, double S_out,
   B_i->resize(C);
   const int64_t half = c > 0 ? (int64_t(1) << (c - 1)) : 0;
   const double two_c = std::ldexp(1.0, c);  // (multiplying by a power of two is exact)
+  std::vector<double> addend(C);
+  scaled_addends(beta, S_out, two_c, C, addend.data());
   for (int i = 0; i < C; ++i) {
     const int64_t mag = (int64_t)((std::fabs(gamma[i]) * m0) * two_c + 0.5);     // positive: truncation is floor
-    const double x = (beta[i] / S_out) * two_c + 0.5;
+    const double x = addend[i];
     if (std::fabs(x) > 4.0e18) return IBERT_ERR_SCALE_RANGE;
     const int64_t t = (int64_t)x;
     (*b_i)[i] = (int32_t)(gamma[i] < 0.0 ? -mag : mag);
@@ -327,30 +340,73 @@ int make_ln_residual(double S_r, double S, LnConsts* k) {
   return IBERT_OK;
 }
 
+// dyadic_bits over an array of up to kTableStep values in loops without branches (the compiler vectorizes them): b, c
+// and b 2^(32-c); false if a value is outside its range.  `fits` is cleared when a pair may have no upper-word
+// form (c < 1 or |b| 2^(32-c) beyond 31 bits).
+constexpr int kTableStep = 256;
+IBERT_HOST_SIMD static bool dyadic_array(const double* m, int n, int32_t* b, int32_t* c, int32_t* upper, bool* fits) {
+  uint64_t u[kTableStep], mult[kTableStep], shift[kTableStep], up[kTableStep];
+  std::memcpy(u, m, sizeof(double) * (size_t)n);
+  uint64_t bad = 0, wide = 0;
+  for (int i = 0; i < n; ++i) {
+    const uint64_t e = (u[i] >> 52) & 0x7ff;
+    const uint64_t sh = e < 1022 ? 31 : 1053 - e;             // min(31, 31 - frexp's exponent)
+    const uint64_t r = (1075 - e - sh) & 63;                  // 22 .. 52
+    const uint64_t f = (u[i] & ((uint64_t(1) << 52) - 1)) | (uint64_t(1) << 52);
+    const uint64_t v = ((f >> (r - 1)) + 1) >> 1;             // (f + 2^(r-1)) >> r
+    const uint64_t over = (v >> 31) & 1;                      // rounded up to 2^31
+    mult[i] = v >> over;
+    shift[i] = sh - over;
+    up[i] = mult[i] << ((32 - shift[i]) & 63);
+  }
+  for (int i = 0; i < n; ++i) {
+    const uint64_t e = (u[i] >> 52) & 0x7ff;
+    bad |= (e - (1023 - 31)) >> 63 | ((1023 + 30) - e) >> 63 | shift[i] >> 63;
+    wide |= up[i] >> 31 | (shift[i] - 1) >> 63;
+  }
+  for (int i = 0; i < n; ++i) {
+    const uint64_t neg = uint64_t(0) - (u[i] >> 63);
+    b[i] = (int32_t)(uint32_t)((mult[i] ^ neg) - neg);
+    c[i] = (int32_t)(uint32_t)shift[i];
+    upper[i] = (int32_t)(uint32_t)((up[i] ^ neg) - neg);
+  }
+  if (wide) *fits = false;
+  return bad == 0;
+}
+IBERT_HOST_SIMD static bool scale_quotients(double S_x, const double* S_w, const double* S_cols, double S_out, int n, double* m) {
+  int bad = 0;
+  for (int i = 0; i < n; ++i) bad |= (int)!(S_w[i] > 0.0) | (int)!(S_w[i] <= DBL_MAX);
+  if (S_cols) {
+    for (int i = 0; i < n; ++i) bad |= (int)!(S_cols[i] > 0.0) | (int)!(S_cols[i] <= DBL_MAX);
+    for (int i = 0; i < n; ++i) m[i] = (S_x * S_w[i]) / S_cols[i];
+  } else {
+    for (int i = 0; i < n; ++i) m[i] = (S_x * S_w[i]) / S_out;
+  }
+  return bad == 0;
+}
+
+// b, c and -- when every pair has one (*fits) -- the upper-word form `upper`
 int make_linear_tables(double S_x, const double* S_w, int N, const double* S_out_cols, double S_out,
-                       std::vector<int32_t>* b, std::vector<int32_t>* c) {
+                       std::vector<int32_t>* b, std::vector<int32_t>* c, std::vector<int32_t>* upper, bool* fits) {
   if (!good_scale(S_x)) return IBERT_ERR_SCALE_RANGE;
   if (!S_out_cols && !good_scale(S_out)) return IBERT_ERR_SCALE_RANGE;
   b->resize(N);
   c->resize(N);
-  // (single-operator calls derive these on every call: 3072 channels 30 us with frexp, ldexp and floor per channel,
-  // 12 us with the divisions in a loop of their own and the pairs from the bits)
-  constexpr int kStep = 256;
-  double m[kStep];
-  for (int n0 = 0; n0 < N; n0 += kStep) {
-    const int len = std::min(kStep, N - n0);
-    bool good = true;
-    for (int i = 0; i < len; ++i) good = good && S_w[n0 + i] > 0.0 && S_w[n0 + i] <= DBL_MAX;
-    if (S_out_cols)
-      for (int i = 0; i < len; ++i) good = good && good_scale(S_out_cols[n0 + i]);
-    if (!good) return IBERT_ERR_SCALE_RANGE;
-    if (S_out_cols)
-      for (int i = 0; i < len; ++i) m[i] = (S_x * S_w[n0 + i]) / S_out_cols[n0 + i];
-    else
-      for (int i = 0; i < len; ++i) m[i] = (S_x * S_w[n0 + i]) / S_out;
+  upper->resize(N);
+  *fits = true;
+  // (single-operator calls derive these on every call: 3072 channels 30 us with frexp, ldexp and floor per channel)
+  double m[kTableStep];
+  for (int n0 = 0; n0 < N; n0 += kTableStep) {
+    const int len = std::min(kTableStep, N - n0);
+    if (!scale_quotients(S_x, S_w + n0, S_out_cols ? S_out_cols + n0 : nullptr, S_out, len, m)) return IBERT_ERR_SCALE_RANGE;
+    if (dyadic_array(m, len, b->data() + n0, c->data() + n0, upper->data() + n0, fits)) continue;
+    *fits = false;                                            // multipliers outside [2^-31, 2^31): one by one
     for (int i = 0; i < len; ++i)
-      if (!dyadic_bits(m[i], &(*b)[n0 + i], &(*c)[n0 + i]))
-        if (const int rc = dyadic_general(m[i], &(*b)[n0 + i], &(*c)[n0 + i])) return rc;
+      if (const int rc = dyadic(m[i], &(*b)[n0 + i], &(*c)[n0 + i])) return rc;
+  }
+  if (!*fits) {                                               // (an out-of-range block may fit all the same)
+    *upper = *b;
+    *fits = to_upper_word_form(upper, *c);
   }
   return IBERT_OK;
 }

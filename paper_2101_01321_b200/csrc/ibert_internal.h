@@ -85,8 +85,9 @@ int make_ln_tables(const double* gamma, const double* beta, int C, double S_out,
                    std::vector<int32_t>* b_i, std::vector<int64_t>* B_i);
 int make_ln_residual(double S_r, double S, LnConsts* k);
 // per-output-channel dyadic multipliers of a linear layer; S_out_cols (N entries) or S_out
+// (b, c); `upper`: the upper-word form, when every column has one (*fits)
 int make_linear_tables(double S_x, const double* S_w, int N, const double* S_out_cols, double S_out,
-                       std::vector<int32_t>* b, std::vector<int32_t>* c);
+                       std::vector<int32_t>* b, std::vector<int32_t>* c, std::vector<int32_t>* upper, bool* fits);
 
 // ---------------------------------------------------------------------------------------
 // Context
