@@ -37,15 +37,15 @@ __device__ __forceinline__ int32_t requant_upper_wide(int32_t v, int32_t r, int3
   return v * w + (int32_t)(t >> 32) + (int32_t)((uint32_t)t >> 31);
 }
 
-// (v * b2 + add) >> 32 for a general 64-bit addend, the carry of the lower words propagated by hand
+// (v * b2 + add) >> 32 for a general 64-bit addend: two multiply-adds with a carry between them (a wide multiply and
+// two additions cost 4.5 instructions instead of 2)
 __device__ __forceinline__ int32_t requant_upper_add(int32_t v, int32_t b2, int64_t add) {
-  const int64_t t = (int64_t)v * (int64_t)b2;
   int32_t hi;
-  asm("{\n\t.reg .u32 s;\n\t"
-      "add.cc.u32 s, %1, %3;\n\t"
-      "addc.s32 %0, %2, %4;\n\t}"
+  asm("{\n\t.reg .u32 lo;\n\t"
+      "mad.lo.cc.u32 lo, %1, %2, %3;\n\t"
+      "madc.hi.s32 %0, %1, %2, %4;\n\t}"
       : "=r"(hi)
-      : "r"((uint32_t)t), "r"((int32_t)(t >> 32)), "r"((uint32_t)add), "r"((int32_t)(add >> 32)));
+      : "r"(v), "r"(b2), "r"((uint32_t)add), "r"((int32_t)(add >> 32)));
   return hi;
 }
 
@@ -191,6 +191,22 @@ __host__ __device__ __forceinline__ int exp_div_mode(const ExpConsts& k) {
   return k.div_pre != 0 ? 2 : (k.div_post != 0 ? 1 : 0);
 }
 
+// i-LayerNorm's normalization of one token: n = floor((v - mu) rho / 2^15) with rho = floor(2^31 / sigma) (sigma <= 1:
+// 2^30 and 2^14) as ONE multiply-high, (v 2^a - mu 2^a) times rho 2^s with a + s = 17 (18).  s is as large as rho
+// allows, at least floor(log2 sigma) - 1; |v - mu| <= (sigma + 1) sqrt(C) then keeps (v - mu) 2^a below 2^25 for
+// C < 2048, so neither factor overflows (v 2^a and mu 2^a alone may: their difference is right modulo 2^32).
+struct LnNorm {
+  int32_t scale, shift, rho;       // 2^a, mu 2^a, rho 2^s
+};
+__device__ __forceinline__ LnNorm ln_norm(int32_t mu, uint32_t sigma) {
+  const uint32_t rho = sigma > 1u ? 0x80000000u / sigma : 1u << 30;
+  const int total = sigma > 1u ? 17 : 18, s = min(__clz((int)rho) - 1, total), a = total - s;
+  return {1 << a, (int32_t)((uint32_t)mu << a), (int32_t)(rho << s)};
+}
+__device__ __forceinline__ int32_t ln_normalize(int32_t v, const LnNorm& n) {
+  return __mulhi((int32_t)((uint32_t)v * (uint32_t)n.scale - (uint32_t)n.shift), n.rho);
+}
+
 // floor(sqrt(floor(ss / C))) = the largest s with s^2 C <= ss, one thread per value, bit by bit.
 // ss / C < 2^(bits(ss) - floor(log2 C)) bounds the highest bit that can be set, so the loop runs
 // about half the bit length of the variance.  Needs s < 2^24 and C < 2^12 (then s^2 C < 2^60).
@@ -207,20 +223,25 @@ __device__ __forceinline__ uint32_t isqrt_of_quotient(uint64_t ss, uint32_t C) {
 
 // floor(sqrt(floor(ss / C))), i.e. the largest s with s*s*C <= ss -- the value Algorithm 4
 // returns for n = floor(ss / C).  A 64-bit integer division costs on the order of a hundred
-// instructions here, so instead of iterating x <- (x + n/x)/2 the warp finds the same integer by
-// a radix-32 search: in each of five rounds the 32 lanes test 32 candidates with one multiply
-// each.  Needs s < 2^25 and ss < 2^61 / C.
+// instructions here, so instead of iterating x <- (x + n/x)/2 a group of GROUP lanes (32 or 16; ss is the group's) finds
+// the same integer by a radix-GROUP search: in each round its lanes test GROUP candidates with one multiply each.
+// Needs s < 2^25 and ss < 2^61 / C.
+template <int GROUP = 32>
 __device__ __forceinline__ uint32_t warp_isqrt_of_quotient(uint64_t ss, uint32_t C, int lane) {
+  constexpr int kDigit = GROUP == 32 ? 5 : 4;
+  const int li = lane & (GROUP - 1);
   uint32_t base = 0;
   // ss / C < 2^bits bounds the result below 2^ceil(bits / 2): rounds above that cannot set a digit
   const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));
-  const int top = 5 * ((min(max((bits + 1) >> 1, 1), 25) + 4) / 5 - 1);
-  for (int shift = top; shift >= 0; shift -= 5) {
-    const uint32_t cand = base + ((uint32_t)lane << shift);
+  int need = min(max((bits + 1) >> 1, 1), 25);
+  if constexpr (GROUP != 32) need = __reduce_max_sync(0xffffffffu, need);
+  for (int shift = kDigit * ((need + kDigit - 1) / kDigit - 1); shift >= 0; shift -= kDigit) {
+    const uint32_t cand = base + ((uint32_t)li << shift);
     const uint64_t sq = (uint64_t)cand * (uint64_t)cand;
     const bool le = sq * (uint64_t)C <= ss;                       // true for a prefix of the lanes
-    const uint32_t cnt = __popc(__ballot_sync(0xffffffffu, le));  // >= 1: lane 0 tests `base` itself
-    base += (cnt - 1u) << shift;
+    uint32_t votes = __ballot_sync(0xffffffffu, le);
+    if constexpr (GROUP == 16) votes = (votes >> (lane & 16)) & 0xffffu;
+    base += (uint32_t)(__popc(votes) - 1) << shift;               // (lane 0 tests `base` itself: at least one vote)
   }
   return base;
 }

@@ -51,7 +51,7 @@ constexpr int kLnOff = kCbOff + kCh * 8;         // int4 {b_i, 0, B_i lo, B_i hi
 constexpr int kStatBytes = kTok * 12;
 constexpr int kLocOff = kLnOff + kCh * 16;       // [3]: this CTA's partial sums, by tile index mod 3
 constexpr int kGatOff = kLocOff + 3 * kStatBytes;   // [2][kMaxCta]: every CTA's partial sums, by tile parity
-constexpr int kParOff = kGatOff + 2 * kMaxCta * kStatBytes;   // [2][128] int4 {mu, floor(2^31 / sigma), shift, -}
+constexpr int kParOff = kGatOff + 2 * kMaxCta * kStatBytes;   // [2][128] int4: the token's LnNorm
 constexpr int kBarOff = kParOff + 2 * kTok * 16;
 constexpr int kAlloc = kBarOff + 512 + 1024;     // + slack to align the base to 1024 bytes
 static_assert(kAlloc <= 227 * 1024, "shared memory budget");
@@ -311,7 +311,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         const int i = par * kTok + tk;
         if (ok) ok = ptx::mbar_wait_cluster(bar_stats + 8 * par, phase);
         ok = __all_sync(0xffffffffu, ok);
-        int32_t mu = 0, rho = 1 << 30, nsh = 14;
+        LnNorm norm = ln_norm(0, 1u);
         if (ok) {
           int32_t sum = 0;
           uint64_t sumsq = 0;
@@ -327,13 +327,12 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             reinterpret_cast<unsigned long long*>(old)[tk] = 0;
             reinterpret_cast<int32_t*>(old + kTok * 8)[tk] = 0;
           }
-          mu = sum / C;                                // floor(sum / C)
+          int32_t mu = sum / C;                        // floor(sum / C)
           if (sum - mu * C < 0) mu -= 1;
           const int64_t ss = (int64_t)sumsq - 2 * (int64_t)mu * (int64_t)sum + (int64_t)C * (int64_t)mu * (int64_t)mu;
-          const uint32_t sigma = isqrt_of_quotient((uint64_t)ss, (uint32_t)C);
-          if (sigma > 1u) { rho = (int32_t)(0x80000000u / sigma); nsh = 15; }   // floor(2^31 / sigma); sigma <= 1: 2^30, one shift less
+          norm = ln_norm(mu, isqrt_of_quotient((uint64_t)ss, (uint32_t)C));
         }
-        s_par[i] = make_int4(mu, rho, nsh, 0);
+        s_par[i] = make_int4(norm.scale, norm.shift, norm.rho, 0);
       }
     };
     // pass B of tile `it`: normalize, affine + requantize to int8, store; frees the accumulator stage
@@ -342,8 +341,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       const int t0 = (int)tile_of(it) * kTok;
       if (ok) {
         const int4 mr = s_par[par * kTok + tok];
-        const int32_t mu = mr.x, rho = mr.y;
-        const uint32_t nsh = (uint32_t)mr.z;
+        const LnNorm norm{mr.x, mr.y, mr.z};
 #pragma unroll 1
         for (int ci = 0; ci < 2; ++ci) {
           const int col = part * 64 + ci * 32;
@@ -360,10 +358,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int4 lc = s_ln[col + i + j];
-              const int32_t y = (int32_t)v[i + j] - mu;
-              const int64_t pr = (int64_t)y * (int64_t)rho;
-              // floor(pr / 2^nsh) fits 32 bits: the low word of the 64-bit shift is a funnel shift
-              const int32_t nrm = (int32_t)__funnelshift_r((uint32_t)pr, (uint32_t)(pr >> 32), nsh) << ln.out_sh;
+              const int32_t nrm = ln_normalize((int32_t)v[i + j], norm) << ln.out_sh;
               const int64_t Bv = (int64_t)(((uint64_t)(uint32_t)lc.w << 32) | (uint32_t)lc.z);
               o[j] = max(requant_upper_add(nrm, lc.x, Bv), -127);
             }

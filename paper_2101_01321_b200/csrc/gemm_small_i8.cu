@@ -376,11 +376,7 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   // L = 77 30.1 -> 29.7.
   const int C = a.N;
   auto mean_of = [&](int32_t sum) { return (int32_t)(__umulhi((uint32_t)(sum + (C << 18)), a.c_magic) >> a.c_shift) - (1 << 18); };
-  // {mu, floor(2^31 / sigma), shift}; sigma <= 1: 2^30 and one shift less
-  auto params_of = [](int32_t mu, uint32_t sigma) {
-    return make_int4(mu, sigma > 1u ? (int32_t)(0x80000000u / sigma) : (1 << 30), sigma > 1u ? 15 : 14, 0);
-  };
-  int4 one = make_int4(0, 0, 0, 0);
+  LnNorm one{};
   if constexpr (TPW == 1) {
     uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
     if (lane < cl)
@@ -392,7 +388,7 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p1 >> 16) << 16) +
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p2) << 25);
     const int32_t mu = mean_of(sum);
-    one = params_of(mu, warp_isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, lane));
+    one = ln_norm(mu, warp_isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, lane));
   } else {
     if ((int)threadIdx.x < a.nt) {
       int32_t sum = 0;
@@ -406,9 +402,9 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
         sumsq += (uint64_t)p1 + ((uint64_t)p2 << 25);
       }
       const int32_t mu = mean_of(sum);
-      const int4 pr = params_of(mu, isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C));
+      const LnNorm pr = ln_norm(mu, isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C));
       // (the token's own records are consumed: the first one's place takes the result)
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(s_part + threadIdx.x * 16), "r"(pr.x), "r"(pr.y), "r"(pr.z), "r"(0) : "memory");
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(s_part + threadIdx.x * 16), "r"(pr.scale), "r"(pr.shift), "r"(pr.rho), "r"(0) : "memory");
     }
     __syncthreads();
   }
@@ -418,15 +414,14 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
 #pragma unroll
   for (int j = 0; j < TPW; ++j) {
     const int t = warp * TPW + j;
-    int4 pr = one;
+    LnNorm pr = one;
+    int32_t unused;
     if constexpr (TPW > 1)
-      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pr.x), "=r"(pr.y), "=r"(pr.z), "=r"(pr.w) : "r"(s_part + (uint32_t)(t * 16)));
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(pr.scale), "=r"(pr.shift), "=r"(pr.rho), "=r"(unused) : "r"(s_part + (uint32_t)(t * 16)));
     int32_t o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int64_t x = (int64_t)(v[j][i] - pr.x) * (int64_t)pr.y;
-      const int32_t nrm = (int32_t)__funnelshift_r((uint32_t)x, (uint32_t)(x >> 32), (uint32_t)pr.z) << ln.out_sh;
-      o[i] = max(requant_upper_add(nrm, bb[i], BB[i]), -127);
+      o[i] = max(requant_upper_add(ln_normalize(v[j][i], pr) << ln.out_sh, bb[i], BB[i]), -127);
     }
     if (t0 + t < a.T)
       *reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(a.out) + (int64_t)(t0 + t) * a.N + ch) = pack4_sat_s8(o[0], o[1], o[2], o[3]);

@@ -311,27 +311,30 @@ __global__ void __launch_bounds__(kThreads, ln_min_blocks(VPL)) layernorm_kernel
   }
 }
 
-// Same row computation, fed by bulk async copies: every warp streams its rows (Q16 row and int8
-// residual row) through a private ring of DEPTH shared-memory slots, so the loads of the next
-// rows are in flight while the current row is reduced -- the row loop no longer waits on HBM.
-// Requires C % 16 == 0 (16-byte aligned rows), upper-word constants, and a residual.
+// Same row computation, fed by bulk async copies: every warp streams its rows (Q16 rows and int8 residual rows)
+// through a private ring of DEPTH shared-memory slots of R rows, so the loads of the next rows are in flight while
+// the current ones are reduced.  Requires C % 16 == 0 (16-byte aligned rows), upper-word constants, and a residual.
+// R = 2: a warp finishes two adjacent rows together -- half-warps share what is scalar per row (mean, square root,
+// divisions: some 150 instructions), both rows use a constant once it is loaded, and the second row hides the
+// latency of the first one's reductions.  One row per warp was bound by instruction issue (31 per element):
+// [16384, 768] 19.5 -> 17.5 us with int32, 19.1 -> 16.5 with int16 input, [32768, 1024] 44.1 -> 37.0, [16384, 256] 12.7 -> 8.1.
 // FULL: C == 128 VPL, no lane ever runs past the row.
-template <int VPL, int DEPTH, typename QT, bool FULL>
-__global__ void __launch_bounds__(kThreads, DEPTH == 2 ? 3 : 2) layernorm_pipe_kernel(const QT* __restrict__ q,
-                                                                     const int8_t* __restrict__ r, int64_t rows,
-                                                                     LnConsts k, const int32_t* __restrict__ b_i,
-                                                                     const int64_t* __restrict__ B_i,
-                                                                     int8_t* __restrict__ out, int32_t* status) {
+template <int VPL, int R, int DEPTH, typename QT, bool FULL>
+__global__ void __launch_bounds__(kThreads, VPL * R > 12 ? 2 : 3)
+layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, int64_t rows, LnConsts k,
+                      const int32_t* __restrict__ b_i, const int64_t* __restrict__ B_i, int8_t* __restrict__ out,
+                      int32_t* status) {
   extern __shared__ __align__(128) uint8_t ln_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int C = k.C;
   const uint32_t q_bytes = (uint32_t)C * (uint32_t)sizeof(QT), r_bytes = (uint32_t)C;
-  const uint32_t slot_bytes = q_bytes + r_bytes;                 // multiple of 16
+  const uint32_t slot_bytes = R * (q_bytes + r_bytes);           // multiple of 16: R Q16 rows, then R residual rows
   uint8_t* ring = ln_smem + (size_t)warp * DEPTH * slot_bytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(ln_smem + (size_t)(kThreads / 32) * DEPTH * slot_bytes) + warp * DEPTH;
   // the per-channel tables, copied once per CTA: every row reads all of them
   int64_t* s_B = reinterpret_cast<int64_t*>(ln_smem + (size_t)(kThreads / 32) * DEPTH * slot_bytes + (kThreads / 32) * DEPTH * 8);
   int32_t* s_b = reinterpret_cast<int32_t*>(s_B + C);
+  const int64_t groups = (rows + R - 1) / R;
   const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
   for (int i = threadIdx.x; i < C; i += kThreads) {        // constants, not outputs of the previous kernel
@@ -342,26 +345,28 @@ __global__ void __launch_bounds__(kThreads, DEPTH == 2 ? 3 : 2) layernorm_pipe_k
 
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();              // the kernel that produced q (and r) has completed
-  auto issue = [&](int64_t row, int slot) {
+  auto issue = [&](int64_t group, int slot) {
     const uint32_t bar = ptx::smem_addr(bars + slot);
     const uint32_t dst = ptx::smem_addr(ring + (size_t)slot * slot_bytes);
-    ptx::mbar_arrive_expect_tx(bar, slot_bytes);
-    ptx::bulk_load_1d(dst, q + row * C, q_bytes, bar);
-    ptx::bulk_load_1d(dst + q_bytes, r + row * C, r_bytes, bar);
+    const int64_t row = group * R;
+    const uint32_t n = (uint32_t)min((int64_t)R, rows - row);
+    ptx::mbar_arrive_expect_tx(bar, n * (q_bytes + r_bytes));
+    ptx::bulk_load_1d(dst, q + row * C, n * q_bytes, bar);
+    ptx::bulk_load_1d(dst + R * q_bytes, r + row * C, n * r_bytes, bar);
   };
   if (lane == 0) {
     for (int s = 0; s < DEPTH; ++s) ptx::mbar_init(ptx::smem_addr(bars + s), 1);
     ptx::fence_mbar_init();
     for (int s = 0; s < DEPTH; ++s) {
-      const int64_t row = warp_global + (int64_t)s * warp_count;
-      if (row < rows) issue(row, s);
+      const int64_t group = warp_global + (int64_t)s * warp_count;
+      if (group < groups) issue(group, s);
     }
   }
   __syncwarp();
 
   int slot = 0;
   uint32_t phase = 0;
-  for (int64_t row = warp_global; row < rows; row += warp_count) {
+  for (int64_t group = warp_global; group < groups; group += warp_count) {
     const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_addr(bars + slot), phase));
     if (!ok) {
       if (lane == 0) atomicCAS(status, 0, IBERT_ERR_TIMEOUT);
@@ -371,56 +376,66 @@ __global__ void __launch_bounds__(kThreads, DEPTH == 2 ? 3 : 2) layernorm_pipe_k
         int s2 = slot + j;
         uint32_t ph2 = phase;
         if (s2 >= DEPTH) { s2 -= DEPTH; ph2 ^= 1; }
-        if (row + (int64_t)j * warp_count < rows) ptx::mbar_wait(ptx::smem_addr(bars + s2), ph2);
+        if (group + (int64_t)j * warp_count < groups) ptx::mbar_wait(ptx::smem_addr(bars + s2), ph2);
       }
       break;
     }
     const uint8_t* sq = ring + (size_t)slot * slot_bytes;
-    int32_t v[VPL][4];
-    uint32_t rw[VPL];
+    int32_t v[R][VPL][4];
+    uint32_t rw[R][VPL];
 #pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-      const int col = 4 * (j * 32 + lane);
-      if (FULL || col < C) {
-        load_q4(reinterpret_cast<const QT*>(sq) + col, v[j], false);
-        rw[j] = *reinterpret_cast<const uint32_t*>(sq + q_bytes + col);
-      } else {
-        v[j][0] = v[j][1] = v[j][2] = v[j][3] = 0;
-        rw[j] = 0;
+    for (int h = 0; h < R; ++h)
+#pragma unroll
+      for (int j = 0; j < VPL; ++j) {
+        const int col = 4 * (j * 32 + lane);
+        if (FULL || col < C) {
+          load_q4(reinterpret_cast<const QT*>(sq + h * q_bytes) + col, v[h][j], false);
+          rw[h][j] = *reinterpret_cast<const uint32_t*>(sq + R * q_bytes + h * r_bytes + col);
+        } else {
+          v[h][j][0] = v[h][j][1] = v[h][j][2] = v[h][j][3] = 0;
+          rw[h][j] = 0;
+        }
       }
-    }
     __syncwarp();                                    // every lane has its copy: the slot can be refilled
     if (lane == 0) {
-      const int64_t next = row + (int64_t)DEPTH * warp_count;
-      if (next < rows) issue(next, slot);
+      const int64_t next = group + (int64_t)DEPTH * warp_count;
+      if (next < groups) issue(next, slot);
     }
     if (++slot == DEPTH) { slot = 0; phase ^= 1; }
 
-    // one pass over the row: sum v and sum v^2 (columns past C hold zeros); the centred sum of squares
+    // one pass over a row: sum v and sum v^2 (columns past C hold zeros); the centred sum of squares
     // follows exactly in integers: sum (v - mu)^2 = sum v^2 - 2 mu sum v + C mu^2
     int32_t sum = 0;
     uint64_t s2 = 0;
 #pragma unroll
-    for (int j = 0; j < VPL; ++j)
+    for (int h = 0; h < R; ++h) {
+      int32_t t = 0;
+      uint64_t t2 = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        v[j][i] += (sext_byte(rw[j], i) * k.res_nb + k.res_nhalf) >> k.res_nc;   // the residual, rescaled (narrow form)
-        sum += v[j][i];
-        s2 += (uint64_t)((int64_t)v[j][i] * (int64_t)v[j][i]);
-      }
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    // a lane's share is below 2^50 (|v| <= 2^21, at most 64 values): two 25-bit halves reduce as 32-bit sums
-    s2 = (uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)s2 & 0x1ffffffu) +
-         ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(s2 >> 25)) << 25);
+      for (int j = 0; j < VPL; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          v[h][j][i] += (sext_byte(rw[h][j], i) * k.res_nb + k.res_nhalf) >> k.res_nc;   // the residual, rescaled (narrow form)
+          t += v[h][j][i];
+          t2 += (uint64_t)((int64_t)v[h][j][i] * (int64_t)v[h][j][i]);
+        }
+      t = __reduce_add_sync(0xffffffffu, t);
+      // a lane's share is below 2^50 (|v| <= 2^21, at most 64 values): two 25-bit halves reduce as 32-bit sums
+      t2 = (uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)t2 & 0x1ffffffu) +
+           ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(t2 >> 25)) << 25);
+      if (h == 0 || lane >= 16) { sum = t; s2 = t2; }            // (two rows: the upper half-warp takes the second)
+    }
     int32_t mu = sum / C;                            // mu = floor(sum / C)
     if (sum - mu * C < 0) mu -= 1;
     const uint64_t ss = (uint64_t)((int64_t)s2 - 2 * (int64_t)mu * (int64_t)sum + (int64_t)C * (int64_t)mu * (int64_t)mu);
-    uint32_t sigma = warp_isqrt_of_quotient(ss, (uint32_t)C, lane);   // I-Sqrt(floor(ss / C))
-    sigma = sigma < 1u ? 1u : sigma;
-    // floor(2^31 / sigma) as a positive int32 multiplier: for sigma = 1 use 2^30 and shift one less
-    const int32_t rho = sigma == 1u ? (1 << 30) : (int32_t)(0x80000000u / sigma);
-    const int nsh = sigma == 1u ? 14 : 15;
-    int8_t* orow = out + row * C;
+    const LnNorm own = ln_norm(mu, warp_isqrt_of_quotient<32 / R>(ss, (uint32_t)C, lane));   // I-Sqrt(floor(ss / C))
+    LnNorm norm[R];
+#pragma unroll
+    for (int h = 0; h < R; ++h)
+      norm[h] = R == 1 ? own : LnNorm{__shfl_sync(0xffffffffu, own.scale, 16 * h), __shfl_sync(0xffffffffu, own.shift, 16 * h),
+                                      __shfl_sync(0xffffffffu, own.rho, 16 * h)};
+    int8_t* orow = out + group * R * C;
+    const bool second = R == 1 || group * R + 1 < rows;
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
       const int col = 4 * (j * 32 + lane);
@@ -430,15 +445,14 @@ __global__ void __launch_bounds__(kThreads, DEPTH == 2 ? 3 : 2) layernorm_pipe_k
         const longlong2 B23 = *reinterpret_cast<const longlong2*>(s_B + col + 2);
         const int32_t bv[4] = {bb.x, bb.y, bb.z, bb.w};
         const int64_t Bv[4] = {B01.x, B01.y, B23.x, B23.y};
-        int32_t o[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int64_t pr = (int64_t)(v[j][i] - mu) * (int64_t)rho;
-          // floor(pr / 2^nsh) fits 32 bits: the low word of the 64-bit shift is a funnel shift
-          const int32_t nrm = (int32_t)__funnelshift_r((uint32_t)pr, (uint32_t)(pr >> 32), (uint32_t)nsh) << k.out_sh;
-          o[i] = max(requant_upper_add(nrm, bv[i], Bv[i]), -127);
+        for (int h = 0; h < R; ++h) {
+          int32_t o[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            o[i] = max(requant_upper_add(ln_normalize(v[h][j][i], norm[h]) << k.out_sh, bv[i], Bv[i]), -127);
+          if (h == 0 || second) __stcs(reinterpret_cast<uint32_t*>(orow + (size_t)h * C + col), pack4_sat_s8(o[0], o[1], o[2], o[3]));
         }
-        __stcs(reinterpret_cast<uint32_t*>(orow + col), pack4_sat_s8(o[0], o[1], o[2], o[3]));
       }
     }
   }
@@ -776,39 +790,44 @@ static int launch_layernorm_t(ibert_ctx* ctx, const QT* q, const int8_t* r, int6
   const int vpl = (k.C + 127) / 128;
   const bool fast = vec && k.out_fast && (!k.has_res || k.res_fast);
   if (fast && k.has_res && k.res_narrow && k.C % 16 == 0 && k.C <= 1024) {
-    // streaming variant: per-warp ring of row slots filled by bulk async copies
-    const int depth = 2;
-    const size_t smem = (size_t)(kThreads / 32) * depth * (size_t)k.C * (sizeof(QT) + 1) + (kThreads / 32) * depth * 8 +
+    // streaming variant: per-warp ring of row slots filled by bulk async copies.  Two rows per warp once every warp of
+    // the resident wave has work that way; below, one row per warp keeps more warps busy
+    // (one-row slots are double-buffered, two-row slots single: the registers are the second buffer)
+    const size_t smem = (size_t)(kThreads / 32) * 2 * (size_t)k.C * (sizeof(QT) + 1) + (kThreads / 32) * 2 * 8 +
                         (size_t)k.C * 12;                  // rows in flight, barriers, the two tables
-    // one wave of resident CTAs: three per SM by registers, fewer when the row slots take more shared memory
-    // (C = 1024 with int32 input: two -- a grid of three per SM ran as a wave and a half)
-    const int per_sm = (int)std::min<size_t>(3, (size_t)(227 * 1024) / (smem + 1024));
-    const int pgrid = (int)std::min<int64_t>((rows + 7) / 8, (int64_t)ctx->num_sms * std::max(per_sm, 1));
-#define IBERT_LNP2(V, D, F)                                                                                 \
+    const bool two = rows >= (int64_t)ctx->num_sms * 3 * (kThreads / 32);
+    // one wave of resident CTAs: by registers three per SM (two for two rows of more than 768 channels), fewer when
+    // the row slots take more shared memory (C = 1024 with int32 input: two)
+    const int by_regs = two && k.C > 768 ? 2 : 3;
+    const int per_sm = (int)std::min<size_t>(by_regs, (size_t)(227 * 1024) / (smem + 1024));
+    const int64_t groups = two ? (rows + 1) / 2 : rows;
+    const int pgrid = (int)std::min<int64_t>((groups + 7) / 8, (int64_t)ctx->num_sms * std::max(per_sm, 1));
+#define IBERT_LNP3(V, R, F)                                                                                 \
   do {                                                                                                      \
     static bool attr_dev[kMaxDevices] = {false};                                                            \
     bool& attr = attr_dev[ctx->device % kMaxDevices];                                                       \
     if (!attr) {                                                                                            \
-      if (cudaFuncSetAttribute(layernorm_pipe_kernel<V, D, QT, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+      if (cudaFuncSetAttribute(layernorm_pipe_kernel<V, R, 3 - R, QT, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                100 * 1024) != cudaSuccess) return IBERT_ERR_CUDA;                           \
       attr = true;                                                                                          \
     }                                                                                                       \
-    if (int rc_ = launch_pdl(layernorm_pipe_kernel<V, D, QT, F>, dim3(pgrid), dim3(kThreads), smem, ctx->stream, 1, q, r, \
-                             rows, k, d_b, d_B, out, ctx->d_status))                                        \
-      return rc_;                                                                                           \
+    return launch_pdl(layernorm_pipe_kernel<V, R, 3 - R, QT, F>, dim3(pgrid), dim3(kThreads), smem, ctx->stream, 1, q, r, \
+                      rows, k, d_b, d_B, out, ctx->d_status);                                               \
   } while (0)
-#define IBERT_LNP(V, D)                       \
+#define IBERT_LNP(V)                          \
   do {                                        \
-    if (k.C == 128 * V) IBERT_LNP2(V, D, true); \
-    else IBERT_LNP2(V, D, false);             \
+    const bool full = k.C == 128 * V;         \
+    if (two && full) IBERT_LNP3(V, 2, true);  \
+    if (two) IBERT_LNP3(V, 2, false);         \
+    if (full) IBERT_LNP3(V, 1, true);         \
+    IBERT_LNP3(V, 1, false);                  \
   } while (0)
-    if (k.C <= 256) IBERT_LNP(2, 2);
-    else if (k.C <= 512) IBERT_LNP(4, 2);
-    else if (k.C <= 768) IBERT_LNP(6, 2);
-    else IBERT_LNP(8, 2);
+    if (k.C <= 256) IBERT_LNP(2);
+    if (k.C <= 512) IBERT_LNP(4);
+    if (k.C <= 768) IBERT_LNP(6);
+    IBERT_LNP(8);
 #undef IBERT_LNP
-#undef IBERT_LNP2
-    return check_launch();
+#undef IBERT_LNP3
   }
 #define IBERT_LN(V)                                                                                              \
   do {                                                                                                           \
