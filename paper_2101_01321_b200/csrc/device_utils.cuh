@@ -105,10 +105,14 @@ __device__ __forceinline__ int32_t igelu_q16_upper(int32_t q, const GeluConsts& 
 //   q <  0:  g = q ((-t^2) >> s_f) = q (-ceil(t^2 / 2^s_f))   = a ((t^2 + 2^s_f - 1) >> s_f)
 // so one select of the addend replaces the two-sided clamp, the negation and the select of f.
 // `rnd_f` = 2^s_f - 1.  The result still needs both clamps to +-127.
+// Written for the ALU pipe, which binds it: the clip and its offset are one add-and-minimum, the addend is selected by
+// a multiply-add with the sign (SHIFT = false: s_in is known to be 0).
+template <bool SHIFT = true>
 __device__ __forceinline__ int32_t igelu_magnitude_upper(int32_t x, const GeluConsts& k, int32_t rnd_f) {
   const int32_t a = (int32_t)min((uint32_t)abs(x), 32767u);    // unsigned: |INT32_MIN| stays 2^31
-  const int32_t t = min(a >> k.s_in, k.nq_b) - k.nq_b;
-  const int32_t f = (t * t + (x >= 0 ? 2 * k.q_c : rnd_f)) >> k.s_f;
+  const int32_t t = __viaddmin_s32(SHIFT ? a >> k.s_in : a, -k.nq_b, 0);
+  const int32_t add = (x >> 31) * (2 * k.q_c - rnd_f) + 2 * k.q_c;         // x >= 0: 2 q_c, else rnd_f
+  const int32_t f = (t * t + add) >> k.s_f;
   const int32_t g2 = (a * f + 128) >> 8;
   return requant_upper(g2, k.b2);
 }

@@ -16,6 +16,11 @@ constexpr int kThreads = 256;
 // ----------------------------------------------------------------------------- i-GELU
 // Each thread converts 4 int4 vectors (16 values); vector j of a thread sits 32 vectors
 // after vector j-1 so that every load and store instruction of a warp is contiguous.
+// FORM: kGeluAny takes every constant set; the others are the upper-word form of i-GELU without / with the pre-shift
+// of the erf argument and without / with a lower clamp (GeluConsts::low_free).  Bound by the ALU pipe in the general
+// form (12 of 20 instructions per element), close to HBM without the shift and the clamp: 2^24 elements 16.7 -> 14.5 us.
+enum { kGeluAny = 0, kGeluPlain = 1, kGeluShift = 2, kGeluClamp = 3, kGeluShiftClamp = 4 };
+template <int FORM>
 __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restrict__ q, int64_t n,
                                                         GeluConsts k, int8_t* __restrict__ out) {
   ptx::grid_dep_launch();
@@ -28,6 +33,15 @@ __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restric
   const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
   const int4* q4 = reinterpret_cast<const int4*>(q);
   uint32_t* o4 = reinterpret_cast<uint32_t*>(out);
+  auto gelu = [&](int32_t x) {
+    if constexpr (FORM != kGeluAny) {
+      const int32_t r = igelu_magnitude_upper<FORM == kGeluShift || FORM == kGeluShiftClamp>(x, k, rnd_f);
+      return FORM == kGeluClamp || FORM == kGeluShiftClamp ? max(r, -127) : r;
+    } else {
+      if (k.hard) return k.fast ? max(ihgelu_upper(x, k), -127) : ihgelu_to_int8(clamp_sym(x, 32767), k, half);
+      return k.fast ? max(igelu_magnitude_upper(x, k, rnd_f), -127) : igelu_q16_to_int8(clamp_sym(x, 32767), k, half);
+    }
+  };
   for (int64_t base = warp_global * 128; base < n_vec; base += warp_count * 128) {
     int4 v[4];
 #pragma unroll
@@ -38,34 +52,13 @@ __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restric
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int64_t idx = base + j * 32 + lane;
-      if (idx < n_vec) {
-        int32_t a, b, c, d;
-        if (k.hard) {
-          a = k.fast ? max(ihgelu_upper(v[j].x, k), -127) : ihgelu_to_int8(clamp_sym(v[j].x, 32767), k, half);
-          b = k.fast ? max(ihgelu_upper(v[j].y, k), -127) : ihgelu_to_int8(clamp_sym(v[j].y, 32767), k, half);
-          c = k.fast ? max(ihgelu_upper(v[j].z, k), -127) : ihgelu_to_int8(clamp_sym(v[j].z, 32767), k, half);
-          d = k.fast ? max(ihgelu_upper(v[j].w, k), -127) : ihgelu_to_int8(clamp_sym(v[j].w, 32767), k, half);
-        } else if (k.fast) {
-          a = max(igelu_magnitude_upper(v[j].x, k, rnd_f), -127);
-          b = max(igelu_magnitude_upper(v[j].y, k, rnd_f), -127);
-          c = max(igelu_magnitude_upper(v[j].z, k, rnd_f), -127);
-          d = max(igelu_magnitude_upper(v[j].w, k, rnd_f), -127);
-        } else {
-          a = igelu_q16_to_int8(clamp_sym(v[j].x, 32767), k, half);
-          b = igelu_q16_to_int8(clamp_sym(v[j].y, 32767), k, half);
-          c = igelu_q16_to_int8(clamp_sym(v[j].z, 32767), k, half);
-          d = igelu_q16_to_int8(clamp_sym(v[j].w, 32767), k, half);
-        }
-        __stcs(o4 + idx, pack4_sat_s8(a, b, c, d));
-      }
+      if (idx < n_vec) __stcs(o4 + idx, pack4_sat_s8(gelu(v[j].x), gelu(v[j].y), gelu(v[j].z), gelu(v[j].w)));
     }
   }
   // ragged tail (n not a multiple of 4)
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int64_t tail = n_vec << 2;
-  if (tid < n - tail)
-    out[tail + tid] = (int8_t)(k.hard ? ihgelu_to_int8(clamp_sym(q[tail + tid], 32767), k, half)
-                                      : igelu_q16_to_int8(clamp_sym(q[tail + tid], 32767), k, half));
+  if (tid < n - tail) out[tail + tid] = (int8_t)min(gelu(q[tail + tid]), 127);
 }
 
 // ----------------------------------------------------------------------------- table look-up GELU
@@ -710,7 +703,14 @@ int launch_gelu_lut(ibert_ctx* ctx, const int32_t* q, int64_t n, const int8_t* t
 int launch_gelu(ibert_ctx* ctx, const int32_t* q, int64_t n, const GeluConsts& k, int8_t* out) {
   if (n == 0) return IBERT_OK;
   const int64_t warps = ((n >> 2) + 127) / 128 + 1;
-  return launch_pdl(gelu_kernel, dim3(wave_grid(ctx, gelu_kernel, warps)), dim3(kThreads), 0, ctx->stream, 1, q, n, k, out);
+#define IBERT_GELU(F) \
+  return launch_pdl(gelu_kernel<F>, dim3(wave_grid(ctx, gelu_kernel<F>, warps)), dim3(kThreads), 0, ctx->stream, 1, q, n, k, out)
+  if (k.hard || !k.fast) IBERT_GELU(kGeluAny);
+  if (k.low_free && k.s_in == 0) IBERT_GELU(kGeluPlain);
+  if (k.low_free) IBERT_GELU(kGeluShift);
+  if (k.s_in == 0) IBERT_GELU(kGeluClamp);
+  IBERT_GELU(kGeluShiftClamp);
+#undef IBERT_GELU
 }
 
 int launch_exp_table(ibert_ctx* ctx, const ExpConsts& k, uint32_t* table) {
