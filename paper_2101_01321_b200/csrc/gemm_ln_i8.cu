@@ -4,7 +4,7 @@
 // kernel: the Q16 tensor never goes to HBM and two launches per layer disappear.
 //
 // LayerNorm needs statistics over all H channels of a token, so a thread-block CLUSTER of
-// H / 256 CTAs owns a 128-token tile: CTA r computes D[t, n] = X W^T for its 256 channels
+// H / 256 CTAs (H = 768 also: 4 CTAs of 192 channels, see choose_narrow) owns a 128-token tile: CTA r computes D[t, n] = X W^T for its 256 channels
 // (tcgen05.mma kind::i8, M = 128 tokens on the TMEM lanes, N = 256 channels on the columns).
 // With tokens on the lanes an epilogue thread owns ONE token, so the row sums are plain
 // per-thread accumulations; only 2 numbers per token cross the cluster (distributed shared
@@ -32,7 +32,7 @@ namespace ibert {
 namespace {
 
 constexpr int kTok = 128;           // tokens per tile = TMEM lanes = MMA M
-constexpr int kCh = 256;            // channels per CTA = MMA N = TMEM columns per accumulator stage
+constexpr int kCh = 256;            // channels per CTA at most = TMEM columns per accumulator stage
 constexpr int kBK = 128;            // K bytes per pipeline stage (one 128-byte swizzle span)
 constexpr int kMaxStages = 4;       // barrier slots; a kernel instance uses 3 (48 KB stages) or 4 (32 KB, CTA pairs)
 constexpr int kEpiWarps = 16;
@@ -73,7 +73,8 @@ struct GemmLnArgs {
 // XT: x is given transposed, x^T [K][T] (token index contiguous), as the FFN1 GEMM writes it without a
 // transposing store: a stage's token tile is then [128 K rows][128 tokens], an MN-major A operand
 // (instruction-descriptor bit 15; 1 KB from one group of eight K rows to the next).
-template <bool PAIR, bool XT = false>
+// CH: channels per CTA = MMA N, 256 or 192 (single CTAs only; see choose_narrow).
+template <bool PAIR, bool XT = false, int CH = kCh>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUtensorMap map_out,
@@ -88,8 +89,20 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   int4* s_par = reinterpret_cast<int4*>(smem + kParOff);
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + kBarOff);
   constexpr int kStages = PAIR ? 4 : 3;
-  constexpr int kWBytes = (PAIR ? kCh / 2 : kCh) * kBK;    // weight rows this CTA loads per K block
+  static_assert(CH == 256 || (!PAIR && CH == 192), "channels per CTA");
+  constexpr int kWBytes = (PAIR ? CH / 2 : CH) * kBK;    // weight rows this CTA loads per K block
   constexpr int kStageBytes = kXBytes + kWBytes;
+  // an epilogue warp's CH / 4 channels: staged kRowB of them at a time (residual and output), read kChunk
+  // at a time from TMEM.  48-byte rows keep the staging accesses free of bank conflicts.
+  constexpr int kWarpCh = CH / 4;
+  constexpr int kRowB = CH == 256 ? 32 : 48;
+  constexpr int kChunk = CH == 256 ? 32 : 16;
+  constexpr int kPieces = kWarpCh / kRowB, kPerPiece = kRowB / kChunk;
+  constexpr int kTile = 32 * kRowB;
+  // output staging: its own block, or (CH = 192) the space that the smaller operand stages leave
+  constexpr int kStageOut = CH == 256 ? kOutOff : kStages * kStageBytes;
+  static_assert(kTile * kEpiWarps <= (CH == 256 ? kOutBytes : kOperandBytes - kStageOut), "output staging");
+  static_assert(kPieces * kTile <= 2 * kOutTile, "residual buffers");
   // full[4], empty[4], acc_full[2], acc_empty[2], stats[2], TMEM base, res[16 warps][2], decision flags
   const uint32_t bar_full = ptx::smem_addr(s_bar);
   const uint32_t bar_empty = bar_full + 8 * kMaxStages;
@@ -102,9 +115,9 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();
-  const int n_slices = args.H / kCh;                       // CTAs that share a token tile
+  const int n_slices = args.H / CH;                        // CTAs that share a token tile
   const int cl = PAIR ? 2 * n_slices : n_slices;           // cluster width
-  const int slice = PAIR ? (int)(rank >> 1) : (int)rank;   // which 256 channels
+  const int slice = PAIR ? (int)(rank >> 1) : (int)rank;   // which channels
   const int half = PAIR ? (int)(rank & 1u) : 0;            // which of the pair's two token tiles
   const uint32_t leader = PAIR ? (rank & ~1u) : rank;      // the CTA of the pair that issues the MMAs
   const int cluster_id = (int)blockIdx.x / cl;
@@ -112,7 +125,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   const int64_t t_tiles = (args.T + kTok - 1) / kTok;
   const int64_t n_units = PAIR ? (t_tiles + 1) / 2 : t_tiles;   // tiles (pairs of tiles) a cluster steps through
   const int k_blocks = (args.K + kBK - 1) / kBK;
-  const int n0 = slice * kCh;                              // this CTA's first channel
+  const int n0 = slice * CH;                               // this CTA's first channel
   // unit / token tile of this CTA at step `it` of its cluster (a tile past T reads zeros, stores nothing)
   auto unit_of = [&](uint32_t it) { return (int64_t)cluster_id + (int64_t)it * num_clusters; };
   auto tile_of = [&](uint32_t it) { return PAIR ? 2 * unit_of(it) + half : unit_of(it); };
@@ -141,7 +154,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   // statistics start at zero; the per-channel constants are weights, not outputs of the previous
   // kernel, so they may be read before the grid dependency is resolved
   for (int i = threadIdx.x; i < 3 * kStatBytes / 4; i += kThreads) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
-  for (int i = threadIdx.x; i < kCh; i += kThreads) {
+  for (int i = threadIdx.x; i < CH; i += kThreads) {
     s_cb[i] = make_int2(__ldg(args.pb + n0 + i), args.bias ? __ldg(args.bias + n0 + i) : 0);
     const int64_t B = __ldg(args.B_i + n0 + i);
     s_ln[i] = make_int4(__ldg(args.b_i + n0 + i), 0, (int32_t)(uint32_t)B, (int32_t)(B >> 32));
@@ -169,7 +182,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             if (half == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * stage, 2 * kStageBytes);
             if constexpr (XT) ptx::tma_load_2d_pair(sx, &map_x, full_leader, t0, kb * kBK);
             else ptx::tma_load_2d_pair(sx, &map_x, full_leader, kb * kBK, t0);
-            ptx::tma_load_2d_pair(sx + kXBytes, &map_w, full_leader, kb * kBK, n0 + half * (kCh / 2));
+            ptx::tma_load_2d_pair(sx + kXBytes, &map_w, full_leader, kb * kBK, n0 + half * (CH / 2));
           } else {
             ptx::mbar_arrive_expect_tx(bar_full + 8 * stage, kStageBytes);
             if constexpr (XT) ptx::tma_load_2d(sx, &map_x, bar_full + 8 * stage, t0, kb * kBK);
@@ -183,7 +196,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (PAIR: the pair's leader only)
     if (half == 0 && ptx::elect_one()) {
-      constexpr uint32_t idesc = ptx::make_idesc_i8(PAIR ? 2 * kTok : kTok, kCh, true, true) | (XT ? (1u << 15) : 0u);
+      constexpr uint32_t idesc = ptx::make_idesc_i8(PAIR ? 2 * kTok : kTok, CH, true, true) | (XT ? (1u << 15) : 0u);
       const uint16_t pair_mask = (uint16_t)(3u << leader);
       uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
       for (uint32_t it = 0; unit_of(it) < n_units && ok; ++it) {
@@ -219,7 +232,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..17)
     // All 16 warps work on the same tile: warp w takes TMEM lane quadrant w & 3 (32 tokens) and
-    // channel quarter (w - 2) >> 2 (64 channels, two 32-column chunks).  Tiles are handled greedily:
+    // channel quarter (w - 2) >> 2 (64 channels in two 32-column chunks, 48 in three of 16).  Tiles are handled greedily:
     // when the next tile's accumulator is already complete, its pass A runs before this tile's
     // pass B, so the statistics exchange of one tile hides behind arithmetic of the other.
     const int ew = warp - 2;                           // 0..15
@@ -227,20 +240,20 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const int part = ew >> 2;
     const int tok = quad * 32 + lane;                  // this thread's token inside the tile
     const int e_tid = threadIdx.x - 64;                // 0..511
-    uint8_t* stage0 = smem + kOutOff + ew * kOutTile;
+    uint8_t* stage0 = smem + kStageOut + ew * kTile;
     const uint8_t* res0 = smem + kResOff + ew * 2 * kOutTile;
     const uint32_t my_res = bar_res + 16 * ew;
     const LnConsts ln = args.ln;
     const int C = ln.C;
     const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
 
-    // residual block of this warp for tile `it` (32 tokens x 64 channels) into its two private
-    // buffers; rows past T read as zero.  Called by lane 0 once both buffers have been consumed.
+    // residual block of this warp for tile `it` (32 tokens x kWarpCh channels) into its private
+    // buffers; rows past T read as zero.  Called by lane 0 once the buffers have been consumed.
     auto issue_res = [&](uint32_t it) {
       const int t0 = (int)tile_of(it) * kTok;
-      for (int b = 0; b < 2; ++b) {
-        ptx::mbar_arrive_expect_tx(my_res + 8 * b, kOutTile);
-        ptx::tma_load_2d(ptx::smem_addr(res0 + b * kOutTile), &map_res, my_res + 8 * b, n0 + part * 64 + b * 32,
+      for (int b = 0; b < kPieces; ++b) {
+        ptx::mbar_arrive_expect_tx(my_res + 8 * b, kTile);
+        ptx::tma_load_2d(ptx::smem_addr(res0 + b * kTile), &map_res, my_res + 8 * b, n0 + part * kWarpCh + b * kRowB,
                          t0 + quad * 32);
       }
     };
@@ -255,18 +268,23 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         int32_t s1 = 0;
         uint64_t s2 = 0;
 #pragma unroll 1
-        for (int ci = 0; ci < 2; ++ci) {
-          const int col = part * 64 + ci * 32;
-          uint32_t v[32];
-          ptx::tmem_ld32(t_lane + par * kCh + col, v);
-          const bool got = __all_sync(0xffffffffu, ptx::mbar_wait(my_res + 8 * ci, it & 1u));   // one fill per tile
-          const uint8_t* rsrc = res0 + ci * kOutTile + lane * 32;
-          const uint4 ra = *reinterpret_cast<const uint4*>(rsrc), rb = *reinterpret_cast<const uint4*>(rsrc + 16);
-          const uint32_t rw[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+        for (int ci = 0; ci < kPieces * kPerPiece; ++ci) {
+          const int col = part * kWarpCh + ci * kChunk;
+          const int piece = kPieces == 1 ? 0 : ci;
+          uint32_t v[kChunk];
+          ptx::tmem_ld(t_lane + par * kCh + col, v);
+          const bool got = __all_sync(0xffffffffu, ptx::mbar_wait(my_res + 8 * piece, it & 1u));   // one fill per tile
+          const uint8_t* rsrc = res0 + lane * kRowB + (kPieces == 1 ? ci * kChunk : ci * kTile);
+          uint32_t rw[kChunk / 4];
+#pragma unroll
+          for (int i = 0; i < kChunk / 16; ++i) {
+            const uint4 q = *reinterpret_cast<const uint4*>(rsrc + 16 * i);
+            rw[4 * i] = q.x; rw[4 * i + 1] = q.y; rw[4 * i + 2] = q.z; rw[4 * i + 3] = q.w;
+          }
           ptx::tmem_wait_ld();
           if (!got) ok = false;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
+          for (int i = 0; i < kChunk; ++i) {
             const int2 cb = s_cb[col + i];
             const int32_t q16 = clamp_sym(requant_upper((int32_t)v[i] + cb.y, cb.x), 32767);
             const int32_t rv = sext_byte(rw[i >> 2], i & 3);
@@ -275,7 +293,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             s1 += val;
             s2 += (uint64_t)((int64_t)val * (int64_t)val);
           }
-          ptx::tmem_st32(t_lane + par * kCh + col, v);
+          ptx::tmem_st(t_lane + par * kCh + col, v);
         }
         ptx::tmem_wait_st();
         uint8_t* loc = s_loc + (it % 3u) * kStatBytes;
@@ -283,7 +301,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         atomicAdd(reinterpret_cast<int32_t*>(loc + kTok * 8) + tok, s1);
       }
       ptx::fence_proxy_async_smem();
-      __syncwarp();                                    // both residual buffers are consumed
+      __syncwarp();                                    // the residual buffers are consumed
       if (lane == 0 && ok && unit_of(it + 1) < n_units) issue_res(it + 1);
     };
     // sends the CTA's partial sums of tile `it` to every CTA of the cluster: one bulk copy of the
@@ -343,17 +361,19 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         const int4 mr = s_par[par * kTok + tok];
         const LnNorm norm{mr.x, mr.y, mr.z};
 #pragma unroll 1
-        for (int ci = 0; ci < 2; ++ci) {
-          const int col = part * 64 + ci * 32;
-          uint32_t v[32];
-          ptx::tmem_ld32(t_lane + par * kCh + col, v);
+        for (int ci = 0; ci < kPieces * kPerPiece; ++ci) {
+          const int col = part * kWarpCh + ci * kChunk;
+          const bool first = kPieces > 1 || ci == 0, last = kPieces > 1 || ci == kPerPiece - 1;   // of a store's chunks
+          uint32_t v[kChunk];
+          ptx::tmem_ld(t_lane + par * kCh + col, v);
           ptx::tmem_wait_ld();
-          if (lane == 0) ptx::bulk_wait_read<0>();     // the previous store has read the staging tile
-          __syncwarp();
-          uint8_t* stage = stage0;
-          uint32_t w[8];
+          if (first) {
+            if (lane == 0) ptx::bulk_wait_read<0>();   // the previous store has read the staging tile
+            __syncwarp();
+          }
+          uint32_t w[kChunk / 4];
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
+          for (int i = 0; i < kChunk; i += 4) {
             int32_t o[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -364,13 +384,17 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             }
             w[i >> 2] = pack4_sat_s8(o[0], o[1], o[2], o[3]);
           }
-          *reinterpret_cast<uint4*>(stage + lane * 32) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(stage + lane * 32 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
-          ptx::fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            ptx::tma_store_2d(&map_out, ptx::smem_addr(stage), n0 + col, t0 + quad * 32);
-            ptx::bulk_commit();
+          uint8_t* row = stage0 + lane * kRowB + (kPieces == 1 ? ci * kChunk : 0);
+#pragma unroll
+          for (int i = 0; i < kChunk / 16; ++i)
+            *reinterpret_cast<uint4*>(row + 16 * i) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+          if (last) {
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              ptx::tma_store_2d(&map_out, ptx::smem_addr(stage0), n0 + col + kChunk - kRowB, t0 + quad * 32);
+              ptx::bulk_commit();
+            }
           }
         }
       }
@@ -440,6 +464,20 @@ bool gemm_ln_supported(int H, int K, const GemmEpilogue& epi, const LnConsts& ln
   return res_max < 200000.0;
 }
 
+// 192 instead of 256 channels per CTA (H = 768)?  A round of tiles is a quarter shorter, and 33 clusters of 4 use 132
+// SMs as 22 clusters of 6 do; taken when rounds x channels is smaller.  Without pairs an SM pulls 40 instead of 32 KB
+// per K block from L2: from the third round on, where main loops overlap epilogues, that bounds a long reduction.
+// us, 256-channel pairs / 192-channel CTAs, K = 768 and 3072:
+//   4096 tokens (1 round / 1)   13.8 / 12.3   19.1 / 17.5        9326 (2 / 3)    21.1 / 23.1   28.0 / 33.1
+//   5632 tokens (1 / 2)         14.4 / 16.9   20.0 / 23.2        12288 (3 / 3)   27.7 / 24.4   36.1 / 37.6
+//   8192 tokens (2 / 2)         20.2 / 18.2   27.0 / 25.5        16384 (3 / 4)   29.4 / 30.3   38.7 / 47.5
+static bool choose_narrow(int64_t units_wide, int resident_wide, int64_t units_narrow, int resident_narrow, bool long_k) {
+  if (resident_narrow <= 0) return false;
+  const int64_t wide = (units_wide + resident_wide - 1) / resident_wide;
+  const int64_t narrow = (units_narrow + resident_narrow - 1) / resident_narrow;
+  return 192 * narrow < 256 * wide && (narrow <= 2 || !long_k);
+}
+
 int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t T, int H, int K,
                       const GemmEpilogue& epi, const int8_t* res, const LnConsts& ln, const int32_t* d_b_i,
                       const int64_t* d_B_i, int8_t* out, bool x_transposed) {
@@ -461,19 +499,6 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
       if ((rc = encode_tensor_map(&mx, x, 2, tdims, tstr, tbox, 128))) return rc;
     }
   }
-  {
-    const uint64_t dims[2] = {(uint64_t)K, (uint64_t)H};
-    const uint64_t str[1] = {(uint64_t)K};
-    const uint32_t box[2] = {kBK, kCh};
-    if ((rc = encode_tensor_map(&mw, w, 2, dims, str, box, 128))) return rc;
-  }
-  {
-    const uint64_t dims[2] = {(uint64_t)H, (uint64_t)T};
-    const uint64_t str[1] = {(uint64_t)H};
-    const uint32_t obox[2] = {32, 32};
-    if ((rc = encode_tensor_map(&mr, res, 2, dims, str, obox, 0))) return rc;
-    if ((rc = encode_tensor_map(&mo, out, 2, dims, str, obox, 0))) return rc;
-  }
   GemmLnArgs a{};
   a.T = T; a.K = K; a.H = H;
   a.pb = epi.d_b; a.bias = epi.d_bias; a.b_i = d_b_i; a.B_i = d_B_i;
@@ -481,20 +506,20 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
   a.status = ctx->d_status;
   const int n_slices = H / kCh;
   const int64_t t_tiles = (T + kTok - 1) / kTok;
-  // CTA pairs (two token tiles per cluster step) when the cluster stays within 6 CTAs and there are
-  // tiles for both halves; resident clusters from the occupancy query, cached
-  static int max_clusters[kMaxDevices][2][9] = {{{0}}};
-  auto resident = [&](bool pair, int cl) {
-    int& slot = max_clusters[ctx->device % kMaxDevices][pair ? 1 : 0][cl];
+  // the kernel's instances: single CTAs, CTA pairs (two token tiles per cluster step), single CTAs of 192 channels
+  // (narrow); resident clusters of each from the occupancy query, cached
+  enum Shape { kSingle, kPair, kNarrow };
+  const auto instance = [](Shape sh, bool xt) {
+    if (sh == kPair) return xt ? gemm_ln_kernel<true, true> : gemm_ln_kernel<true>;
+    if (sh == kNarrow) return xt ? gemm_ln_kernel<false, true, 192> : gemm_ln_kernel<false, false, 192>;
+    return xt ? gemm_ln_kernel<false, true> : gemm_ln_kernel<false>;
+  };
+  const auto width = [&](Shape sh) { return sh == kPair ? 2 * n_slices : sh == kNarrow ? H / 192 : n_slices; };
+  static int max_clusters[kMaxDevices][3][2 * kMaxCta + 1] = {{{0}}};
+  const auto resident = [&](Shape sh) {
+    const int cl = width(sh);
+    int& slot = max_clusters[ctx->device % kMaxDevices][sh][cl];
     if (slot == 0) {
-      const void* fn = pair ? (const void*)gemm_ln_kernel<true> : (const void*)gemm_ln_kernel<false>;
-      const void* fnt = pair ? (const void*)gemm_ln_kernel<true, true> : (const void*)gemm_ln_kernel<false, true>;
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
-          cudaFuncSetAttribute(fnt, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess) {
-        cudaGetLastError();
-        slot = -1;
-        return slot;
-      }
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(cl * ctx->num_sms);
       cfg.blockDim = dim3(kThreads);
@@ -504,36 +529,40 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
       attr[0].val.clusterDim.x = cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr; cfg.numAttrs = 1;
       int n = 0;
-      const cudaError_t e = pair ? cudaOccupancyMaxActiveClusters(&n, gemm_ln_kernel<true>, &cfg)
-                                 : cudaOccupancyMaxActiveClusters(&n, gemm_ln_kernel<false>, &cfg);
-      if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
+      for (bool xt : {true, false})
+        if (cudaFuncSetAttribute(instance(sh, xt), cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, instance(sh, xt), &cfg) != cudaSuccess) {
+          cudaGetLastError();
+          n = 0;
+          break;
+        }
       slot = n >= 1 ? n : -1;
     }
     return slot;
   };
-  // (clusters of 8 fit only 16 times on the 148 SMs and measured slower than clusters of 4 single CTAs)
-  const bool want_pair = 2 * n_slices <= 6 && t_tiles >= 2;
-  if (want_pair && resident(true, 2 * n_slices) > 0) {
-    const int cl = 2 * n_slices;
-    CUtensorMap mw2;
+  // CTA pairs when the cluster stays within 6 CTAs and there are tiles for both halves (clusters of 8, H = 1024,
+  // fit only 15 times on the 148 SMs and measured slower than clusters of 4 single CTAs)
+  Shape shape = 2 * n_slices <= 6 && t_tiles >= 2 && resident(kPair) > 0 ? kPair : kSingle;
+  if (shape == kPair && H % 192 == 0 && choose_narrow((t_tiles + 1) / 2, resident(kPair), t_tiles, resident(kNarrow), K > H))
+    shape = kNarrow;
+  if (resident(shape) <= 0) return IBERT_ERR_CUDA;
+  const bool pair = shape == kPair, narrow = shape == kNarrow;
+  {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)H};
     const uint64_t str[1] = {(uint64_t)K};
-    const uint32_t box[2] = {kBK, kCh / 2};            // each CTA of a pair loads half of the weight rows
-    if ((rc = encode_tensor_map(&mw2, w, 2, dims, str, box, 128))) return rc;
-    const int clusters = (int)std::min<int64_t>((t_tiles + 1) / 2, resident(true, cl));
-    if (x_transposed)
-      return launch_pdl(gemm_ln_kernel<true, true>, dim3(clusters * cl), dim3(kThreads), (size_t)kAlloc, ctx->stream, cl,
-                        mx, mw2, mr, mo, a);
-    return launch_pdl(gemm_ln_kernel<true>, dim3(clusters * cl), dim3(kThreads), (size_t)kAlloc, ctx->stream, cl,
-                      mx, mw2, mr, mo, a);
+    const uint32_t box[2] = {kBK, (uint32_t)(narrow ? 192 : kCh) / (pair ? 2 : 1)};   // a pair shares the weight rows
+    if ((rc = encode_tensor_map(&mw, w, 2, dims, str, box, 128))) return rc;
   }
-  if (resident(false, n_slices) <= 0) return IBERT_ERR_CUDA;
-  const int clusters = (int)std::min<int64_t>(t_tiles, resident(false, n_slices));
-  if (x_transposed)
-    return launch_pdl(gemm_ln_kernel<false, true>, dim3(clusters * n_slices), dim3(kThreads), (size_t)kAlloc, ctx->stream,
-                      n_slices, mx, mw, mr, mo, a);
-  return launch_pdl(gemm_ln_kernel<false>, dim3(clusters * n_slices), dim3(kThreads), (size_t)kAlloc, ctx->stream,
-                    n_slices, mx, mw, mr, mo, a);
+  {
+    const uint64_t dims[2] = {(uint64_t)H, (uint64_t)T};
+    const uint64_t str[1] = {(uint64_t)H};
+    const uint32_t obox[2] = {narrow ? 48u : 32u, 32};
+    if ((rc = encode_tensor_map(&mr, res, 2, dims, str, obox, 0))) return rc;
+    if ((rc = encode_tensor_map(&mo, out, 2, dims, str, obox, 0))) return rc;
+  }
+  const int clusters = (int)std::min<int64_t>(pair ? (t_tiles + 1) / 2 : t_tiles, resident(shape));
+  return launch_pdl(instance(shape, x_transposed), dim3(clusters * width(shape)), dim3(kThreads), (size_t)kAlloc, ctx->stream,
+                    width(shape), mx, mw, mr, mo, a);
 }
 
 }  // namespace ibert

@@ -6,6 +6,7 @@ import pytest
 
 import oracle
 from gpu_util import assert_same, ctx, dev, host
+from paper_2101_01321_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -96,3 +97,28 @@ def test_linear_layernorm_equals_the_two_separate_calls():
     two, _ = c.ibert_layernorm_i(mid, S_mid, dev(res), S_res, gamma, beta, S_out)
     c.check()
     assert_same(host(fused), host(two), "fused vs separate")
+
+
+# 768 channels: 192 instead of 256 per CTA while that shortens the rounds of token tiles -- one full round, one tile
+# more (256 again), a second round that starts, one that is full, and the third (a short reduction only)
+@pytest.mark.parametrize("M,K", [(4224, 128), (4225, 128), (5633, 256), (8448, 144), (12161, 128), (12161, 896)])
+def test_linear_layernorm_rounds_of_narrow_tiles(M, K):
+    p = _problem(M, 768, K, M + K)
+    x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
+    ctx().ibert_set_fusion(1)
+    out, _ = ctx().ibert_linear_layernorm_i8(dev(x), S_x, dev(w), S_w, dev(bias), S_mid, dev(res), S_res,
+                                             gamma, beta, S_out)
+    ctx().check()
+    assert_same(host(out), _oracle(*p), f"linear+LN {M}x768x{K}")
+
+
+@pytest.mark.parametrize("B", [32, 64])
+def test_encoder_layer_rounds_of_narrow_tiles(B):
+    """FFN2 of 192 channels per CTA, its activations in the transposed layout."""
+    L, H, F = 128, 768, 256
+    x, params = synth.make_model(0, B, layers=1, H=H, heads=12, F=F, L=L)
+    layer = ctx().ibert_layer_create(params[0])
+    out, _ = ctx().ibert_encoder_layer(layer, dev(x), B, L)
+    ctx().check()
+    layer.close()
+    assert_same(host(out), oracle.encoder_layer(params[0], x, B, L).out, f"encoder layer {B}x{L}")
