@@ -504,8 +504,9 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
 }
 
 // true when T tokens give the fused GEMM + LayerNorm kernel (one cluster of H / 256 CTAs per
-// 128-token tile) enough tiles to occupy at least half of the SMs; measured crossover on config 2:
-// the two-kernel path wins up to T = 2048 (0.63 vs 0.76 ms at T = 128), the fused one from T = 4096
+// 128-token tile) enough tiles to occupy at least half of the SMs; below, the GEMM is one wave of small
+// tiles and a LayerNorm kernel after it costs less (H = 768, fused / two kernels, K = 768 and 3072:
+// 3072 tokens 11.8 / 10.0 and 16.6 / 15.7 us, 4096 tokens 12.3 / 13.7 and 17.5 / 19.3 us)
 static bool gemm_ln_profitable(const ibert_ctx* ctx, int64_t T, int H) {
   if (ctx->fusion_mode == 1) return true;
   if (ctx->fusion_mode == 2) return false;
@@ -526,12 +527,13 @@ static int ensure_workspace(ibert_ctx* ctx, size_t need) {
 }
 
 // projection + residual + LayerNorm: the small-problem cluster kernel while the problem is one wave of it, the
-// large-tile cluster kernel once its tiles keep half of the SMs busy, in between two kernels over an int16
-// tensor at `mid` (room for T H of them)
+// large-tile cluster kernel once its tiles keep half of the SMs busy, in between -- and where the GEMM alone needs
+// clearly fewer rounds of tiles than the clusters -- two kernels over an int16 tensor at `mid` (room for T H of them)
 enum LnPath { LN_SMALL, LN_LARGE, LN_TWO };
 static LnPath linear_ln_path(const ibert_ctx* ctx, int64_t T, int H, int K, const GemmEpilogue& e, const LnConsts& ln) {
   if (ctx->fusion_mode == 0 && ctx->splitk_mode == 0 && gemm_ln_small_supported(ctx, T, H, K, e, ln)) return LN_SMALL;
-  return gemm_ln_profitable(ctx, T, H) && gemm_ln_supported(H, K, e, ln) ? LN_LARGE : LN_TWO;
+  if (!gemm_ln_supported(H, K, e, ln) || !gemm_ln_profitable(ctx, T, H)) return LN_TWO;
+  return ctx->fusion_mode == 1 || gemm_ln_beats_two(ctx, T, H, K) ? LN_LARGE : LN_TWO;
 }
 static int linear_ln(ibert_ctx* ctx, LnPath path, const int8_t* x, const int8_t* w, int64_t T, int H, int K,
                      GemmEpilogue e, const int8_t* res, const LnConsts& ln, const int32_t* d_b_i,

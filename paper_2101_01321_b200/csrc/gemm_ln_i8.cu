@@ -4,7 +4,7 @@
 // kernel: the Q16 tensor never goes to HBM and two launches per layer disappear.
 //
 // LayerNorm needs statistics over all H channels of a token, so a thread-block CLUSTER of
-// H / 256 CTAs (H = 768 also: 4 CTAs of 192 channels, see choose_narrow) owns a 128-token tile: CTA r computes D[t, n] = X W^T for its 256 channels
+// H / 256 CTAs (H = 768 also: 4 CTAs of 192 channels, see choose_shape) owns a 128-token tile: CTA r computes D[t, n] = X W^T for its 256 channels
 // (tcgen05.mma kind::i8, M = 128 tokens on the TMEM lanes, N = 256 channels on the columns).
 // With tokens on the lanes an epilogue thread owns ONE token, so the row sums are plain
 // per-thread accumulations; only 2 numbers per token cross the cluster (distributed shared
@@ -73,7 +73,7 @@ struct GemmLnArgs {
 // XT: x is given transposed, x^T [K][T] (token index contiguous), as the FFN1 GEMM writes it without a
 // transposing store: a stage's token tile is then [128 K rows][128 tokens], an MN-major A operand
 // (instruction-descriptor bit 15; 1 KB from one group of eight K rows to the next).
-// CH: channels per CTA = MMA N, 256 or 192 (single CTAs only; see choose_narrow).
+// CH: channels per CTA = MMA N, 256 or 192 (single CTAs only; see choose_shape).
 template <bool PAIR, bool XT = false, int CH = kCh>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
@@ -464,6 +464,44 @@ bool gemm_ln_supported(int H, int K, const GemmEpilogue& epi, const LnConsts& ln
   return res_max < 200000.0;
 }
 
+// the kernel's instances: single CTAs, CTA pairs (two token tiles per cluster step), single CTAs of 192 channels
+enum Shape { kSingle, kPair, kNarrow };
+
+static auto instance(Shape sh, bool xt) {
+  if (sh == kPair) return xt ? gemm_ln_kernel<true, true> : gemm_ln_kernel<true>;
+  if (sh == kNarrow) return xt ? gemm_ln_kernel<false, true, 192> : gemm_ln_kernel<false, false, 192>;
+  return xt ? gemm_ln_kernel<false, true> : gemm_ln_kernel<false>;
+}
+
+static int cluster_width(Shape sh, int H) { return sh == kPair ? 2 * (H / kCh) : sh == kNarrow ? H / 192 : H / kCh; }
+
+// clusters that are resident at once, from the occupancy query, cached; <= 0: none
+static int resident_clusters(const ibert_ctx* ctx, Shape sh, int H) {
+  static int max_clusters[kMaxDevices][3][2 * kMaxCta + 1] = {{{0}}};
+  const int cl = cluster_width(sh, H);
+  int& slot = max_clusters[ctx->device % kMaxDevices][sh][cl];
+  if (slot == 0) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cl * ctx->num_sms);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kAlloc;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    for (bool xt : {true, false})
+      if (cudaFuncSetAttribute(instance(sh, xt), cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&n, instance(sh, xt), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+        break;
+      }
+    slot = n >= 1 ? n : -1;
+  }
+  return slot;
+}
+
 // 192 instead of 256 channels per CTA (H = 768)?  A round of tiles is a quarter shorter, and 33 clusters of 4 use 132
 // SMs as 22 clusters of 6 do; taken when rounds x channels is smaller.  Without pairs an SM pulls 40 instead of 32 KB
 // per K block from L2: from the third round on, where main loops overlap epilogues, that bounds a long reduction.
@@ -471,11 +509,40 @@ bool gemm_ln_supported(int H, int K, const GemmEpilogue& epi, const LnConsts& ln
 //   4096 tokens (1 round / 1)   13.8 / 12.3   19.1 / 17.5        9326 (2 / 3)    21.1 / 23.1   28.0 / 33.1
 //   5632 tokens (1 / 2)         14.4 / 16.9   20.0 / 23.2        12288 (3 / 3)   27.7 / 24.4   36.1 / 37.6
 //   8192 tokens (2 / 2)         20.2 / 18.2   27.0 / 25.5        16384 (3 / 4)   29.4 / 30.3   38.7 / 47.5
-static bool choose_narrow(int64_t units_wide, int resident_wide, int64_t units_narrow, int resident_narrow, bool long_k) {
-  if (resident_narrow <= 0) return false;
-  const int64_t wide = (units_wide + resident_wide - 1) / resident_wide;
-  const int64_t narrow = (units_narrow + resident_narrow - 1) / resident_narrow;
-  return 192 * narrow < 256 * wide && (narrow <= 2 || !long_k);
+struct ShapeChoice {
+  Shape shape;
+  int64_t rounds;       // of token tiles
+};
+static ShapeChoice choose_shape(const ibert_ctx* ctx, int64_t T, int H, int K) {
+  const int64_t t_tiles = (T + kTok - 1) / kTok;
+  const auto rounds = [&](Shape sh, int64_t units) { return (units + resident_clusters(ctx, sh, H) - 1) / resident_clusters(ctx, sh, H); };
+  // CTA pairs when the cluster stays within 6 CTAs and there are tiles for both halves (clusters of 8, H = 1024,
+  // fit only 15 times on the 148 SMs and measured slower than clusters of 4 single CTAs)
+  if (2 * (H / kCh) > 6 || t_tiles < 2 || resident_clusters(ctx, kPair, H) <= 0)
+    return {kSingle, resident_clusters(ctx, kSingle, H) > 0 ? rounds(kSingle, t_tiles) : 0};
+  const int64_t wide = rounds(kPair, (t_tiles + 1) / 2);
+  if (H % 192 == 0 && resident_clusters(ctx, kNarrow, H) > 0) {
+    const int64_t narrow = rounds(kNarrow, t_tiles);
+    if (192 * narrow < 256 * wide && (narrow <= 2 || K <= H)) return {kNarrow, narrow};
+  }
+  return {kPair, wide};
+}
+
+// One kernel, or the GEMM and the LayerNorm with an int16 tensor between them?  The GEMM's tiles are independent (74
+// CTA pairs), so it may need fewer rounds than the clusters, which leave 12 to 16 SMs idle and step through whole rows of
+// tiles.  Two kernels are taken when they save a fifth of the rounds: a smaller saving is lost on the extra tensor (us per
+// layer, fused / two kernels: 32768 tokens x 1024, 8 rounds / 7, 615 / 617; 20480 x 1024, 5 / 5, 407 / 411).  With a long
+// reduction only instead of single CTAs: pairs load it faster than the GEMM saves rounds, and read the operand as the
+// FFN1 kernel writes it best (18944 tokens x 768, K = 3072: 209 / 215).
+//   9472 tokens x 1024 (3 rounds / 2), both projections  165 / 152 us per layer
+//   18944 tokens x 768 (3.75 / 3), output projection     209 / 204 us per layer
+bool gemm_ln_beats_two(const ibert_ctx* ctx, int64_t T, int H, int K) {
+  const ShapeChoice c = choose_shape(ctx, T, H, K);
+  if (K > H && c.shape != kSingle) return true;
+  const int pairs = std::max(1, ctx->num_sms / 2);
+  const int64_t fused = c.rounds * (c.shape == kNarrow ? 192 : kCh);
+  const int64_t two = ((T + 255) / 256 * (H / kCh) + pairs - 1) / pairs * kCh;
+  return 5 * two > 4 * fused;
 }
 
 int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t T, int H, int K,
@@ -504,48 +571,10 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
   a.pb = epi.d_b; a.bias = epi.d_bias; a.b_i = d_b_i; a.B_i = d_B_i;
   a.ln = ln;
   a.status = ctx->d_status;
-  const int n_slices = H / kCh;
   const int64_t t_tiles = (T + kTok - 1) / kTok;
-  // the kernel's instances: single CTAs, CTA pairs (two token tiles per cluster step), single CTAs of 192 channels
-  // (narrow); resident clusters of each from the occupancy query, cached
-  enum Shape { kSingle, kPair, kNarrow };
-  const auto instance = [](Shape sh, bool xt) {
-    if (sh == kPair) return xt ? gemm_ln_kernel<true, true> : gemm_ln_kernel<true>;
-    if (sh == kNarrow) return xt ? gemm_ln_kernel<false, true, 192> : gemm_ln_kernel<false, false, 192>;
-    return xt ? gemm_ln_kernel<false, true> : gemm_ln_kernel<false>;
-  };
-  const auto width = [&](Shape sh) { return sh == kPair ? 2 * n_slices : sh == kNarrow ? H / 192 : n_slices; };
-  static int max_clusters[kMaxDevices][3][2 * kMaxCta + 1] = {{{0}}};
-  const auto resident = [&](Shape sh) {
-    const int cl = width(sh);
-    int& slot = max_clusters[ctx->device % kMaxDevices][sh][cl];
-    if (slot == 0) {
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(cl * ctx->num_sms);
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = kAlloc;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr; cfg.numAttrs = 1;
-      int n = 0;
-      for (bool xt : {true, false})
-        if (cudaFuncSetAttribute(instance(sh, xt), cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, instance(sh, xt), &cfg) != cudaSuccess) {
-          cudaGetLastError();
-          n = 0;
-          break;
-        }
-      slot = n >= 1 ? n : -1;
-    }
-    return slot;
-  };
-  // CTA pairs when the cluster stays within 6 CTAs and there are tiles for both halves (clusters of 8, H = 1024,
-  // fit only 15 times on the 148 SMs and measured slower than clusters of 4 single CTAs)
-  Shape shape = 2 * n_slices <= 6 && t_tiles >= 2 && resident(kPair) > 0 ? kPair : kSingle;
-  if (shape == kPair && H % 192 == 0 && choose_narrow((t_tiles + 1) / 2, resident(kPair), t_tiles, resident(kNarrow), K > H))
-    shape = kNarrow;
-  if (resident(shape) <= 0) return IBERT_ERR_CUDA;
+  const Shape shape = choose_shape(ctx, T, H, K).shape;
+  const int width = cluster_width(shape, H), n_resident = resident_clusters(ctx, shape, H);
+  if (n_resident <= 0) return IBERT_ERR_CUDA;
   const bool pair = shape == kPair, narrow = shape == kNarrow;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)H};
@@ -560,9 +589,9 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
     if ((rc = encode_tensor_map(&mr, res, 2, dims, str, obox, 0))) return rc;
     if ((rc = encode_tensor_map(&mo, out, 2, dims, str, obox, 0))) return rc;
   }
-  const int clusters = (int)std::min<int64_t>(pair ? (t_tiles + 1) / 2 : t_tiles, resident(shape));
-  return launch_pdl(instance(shape, x_transposed), dim3(clusters * width(shape)), dim3(kThreads), (size_t)kAlloc, ctx->stream,
-                    width(shape), mx, mw, mr, mo, a);
+  const int clusters = (int)std::min<int64_t>(pair ? (t_tiles + 1) / 2 : t_tiles, n_resident);
+  return launch_pdl(instance(shape, x_transposed), dim3(clusters * width), dim3(kThreads), (size_t)kAlloc, ctx->stream, width,
+                    mx, mw, mr, mo, a);
 }
 
 }  // namespace ibert

@@ -257,6 +257,7 @@ struct AttnConsts {
 // out = LN(requant_Q16(x w^T + bias) + rescale(res)).  `gemm_ln_supported` tells whether the
 // shapes and constants allow it; otherwise run launch_gemm_i8 (Q16) followed by launch_layernorm.
 bool gemm_ln_supported(int H, int K, const GemmEpilogue& epi, const LnConsts& ln);
+bool gemm_ln_beats_two(const ibert_ctx* ctx, int64_t T, int H, int K);
 int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t T, int H, int K,
                       const GemmEpilogue& epi, const int8_t* res, const LnConsts& ln, const int32_t* d_b_i,
                       const int64_t* d_B_i, int8_t* out, bool x_transposed = false);

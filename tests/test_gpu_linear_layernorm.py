@@ -122,3 +122,15 @@ def test_encoder_layer_rounds_of_narrow_tiles(B):
     ctx().check()
     layer.close()
     assert_same(host(out), oracle.encoder_layer(params[0], x, B, L).out, f"encoder layer {B}x{L}")
+
+
+# sizes at which two kernels need fewer rounds of tiles than the clusters, chosen by size alone; the third
+# row has a tile of tokens too many
+@pytest.mark.parametrize("M,N,K", [(4225, 1024, 256), (4600, 1024, 1040), (4609, 1024, 256), (18900, 768, 256)])
+def test_linear_layernorm_by_rounds_of_tiles(M, N, K):
+    p = _problem(M, N, K, M + N + K)
+    x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
+    out, _ = ctx().ibert_linear_layernorm_i8(dev(x), S_x, dev(w), S_w, dev(bias), S_mid, dev(res), S_res,
+                                             gamma, beta, S_out)
+    ctx().check()
+    assert_same(host(out), _oracle(*p), f"linear+LN {M}x{N}x{K}")
