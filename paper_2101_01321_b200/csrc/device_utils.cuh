@@ -65,6 +65,14 @@ __device__ __forceinline__ int32_t sext_byte(uint32_t w, int k) {
   return r;
 }
 
+// the int8 residual in byte j of w, rescaled, plus add: the byte lands above 16 bits of rounding offset by one permute
+__device__ __forceinline__ int32_t residual_high_add(uint32_t w, int j, int32_t hk, int32_t hm, int32_t add) {
+  int32_t u, d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(u) : "r"(w), "r"(hk), "r"(0x8054 + j * 0x1100));
+  asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(u), "r"(hm), "r"(add));
+  return d;
+}
+
 // 16-bit half h of a word as a sign-extended int32, likewise in one permute
 __device__ __forceinline__ int32_t sext_half(uint32_t w, int h) {
   int32_t r;

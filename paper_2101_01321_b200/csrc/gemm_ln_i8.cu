@@ -74,7 +74,10 @@ struct GemmLnArgs {
 // transposing store: a stage's token tile is then [128 K rows][128 tokens], an MN-major A operand
 // (instruction-descriptor bit 15; 1 KB from one group of eight K rows to the next).
 // CH: channels per CTA = MMA N, 256 or 192 (single CTAs only; see choose_shape).
-template <bool PAIR, bool XT = false, int CH = kCh>
+// RH: the residual is rescaled by one multiply-high (LnConsts::res_high) instead of multiply-add, shift and addition
+// (16384 x 768: K = 768 29.4 -> 28.7 us, K = 3072 38.8 -> 38.4; with 192 channels per CTA it spills and loses,
+// 4096 x 768 12.3 -> 12.6).
+template <bool PAIR, bool XT, int CH, bool RH>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_res, const __grid_constant__ CUtensorMap map_out,
@@ -287,8 +290,8 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           for (int i = 0; i < kChunk; ++i) {
             const int2 cb = s_cb[col + i];
             const int32_t q16 = clamp_sym(requant_upper((int32_t)v[i] + cb.y, cb.x), 32767);
-            const int32_t rv = sext_byte(rw[i >> 2], i & 3);
-            const int32_t val = q16 + ((rv * ln.res_nb + ln.res_nhalf) >> ln.res_nc);   // the residual, rescaled (narrow form)
+            const int32_t val = RH ? residual_high_add(rw[i >> 2], i & 3, ln.res_hk, ln.res_hm, q16)
+                                   : q16 + ((sext_byte(rw[i >> 2], i & 3) * ln.res_nb + ln.res_nhalf) >> ln.res_nc);
             v[i] = (uint32_t)val;
             s1 += val;
             s2 += (uint64_t)((int64_t)val * (int64_t)val);
@@ -467,11 +470,13 @@ bool gemm_ln_supported(int H, int K, const GemmEpilogue& epi, const LnConsts& ln
 // the kernel's instances: single CTAs, CTA pairs (two token tiles per cluster step), single CTAs of 192 channels
 enum Shape { kSingle, kPair, kNarrow };
 
-static auto instance(Shape sh, bool xt) {
-  if (sh == kPair) return xt ? gemm_ln_kernel<true, true> : gemm_ln_kernel<true>;
-  if (sh == kNarrow) return xt ? gemm_ln_kernel<false, true, 192> : gemm_ln_kernel<false, false, 192>;
-  return xt ? gemm_ln_kernel<false, true> : gemm_ln_kernel<false>;
+template <bool RH>
+static auto instance_of(Shape sh, bool xt) {
+  if (sh == kPair) return xt ? gemm_ln_kernel<true, true, kCh, RH> : gemm_ln_kernel<true, false, kCh, RH>;
+  if (sh == kNarrow) return xt ? gemm_ln_kernel<false, true, 192, false> : gemm_ln_kernel<false, false, 192, false>;
+  return xt ? gemm_ln_kernel<false, true, kCh, RH> : gemm_ln_kernel<false, false, kCh, RH>;
 }
+static auto instance(Shape sh, bool xt, bool rh) { return rh ? instance_of<true>(sh, xt) : instance_of<false>(sh, xt); }
 
 static int cluster_width(Shape sh, int H) { return sh == kPair ? 2 * (H / kCh) : sh == kNarrow ? H / 192 : H / kCh; }
 
@@ -490,9 +495,9 @@ static int resident_clusters(const ibert_ctx* ctx, Shape sh, int H) {
     attr[0].val.clusterDim.x = cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    for (bool xt : {true, false})
-      if (cudaFuncSetAttribute(instance(sh, xt), cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
-          cudaOccupancyMaxActiveClusters(&n, instance(sh, xt), &cfg) != cudaSuccess) {
+    for (int form = 0; form < 4; ++form)
+      if (cudaFuncSetAttribute(instance(sh, form & 1, form & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&n, instance(sh, form & 1, form & 2), &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
         break;
@@ -590,7 +595,7 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
     if ((rc = encode_tensor_map(&mo, out, 2, dims, str, obox, 0))) return rc;
   }
   const int clusters = (int)std::min<int64_t>(pair ? (t_tiles + 1) / 2 : t_tiles, n_resident);
-  return launch_pdl(instance(shape, x_transposed), dim3(clusters * width), dim3(kThreads), (size_t)kAlloc, ctx->stream, width,
+  return launch_pdl(instance(shape, x_transposed, ln.res_high != 0), dim3(clusters * width), dim3(kThreads), (size_t)kAlloc, ctx->stream, width,
                     mx, mw, mr, mo, a);
 }
 

@@ -337,6 +337,26 @@ int make_ln_residual(double S_r, double S, LnConsts* k) {
       if (same) { k->res_narrow = 1; k->res_nb = (int32_t)nb; k->res_nc = nc; k->res_nhalf = (int32_t)nhalf; }
     }
   }
+  // high form: the low 16 bits of the operand hold the rounding offset (in units of 2^-16 of r), the multiplier
+  // is the ratio times 2^16; the offset comes from the same intersection of intervals
+  k->res_high = k->res_hm = k->res_hk = 0;
+  if (k->c_r >= 8 && k->c_r <= 31) {
+    const int64_t base = ((int64_t)k->b_r << 16) >> k->c_r;
+    static const int kTry[7] = {0, 1, -1, 2, -2, 3, -3};
+    for (int t = 0; t < 7 && !k->res_high; ++t) {
+      const int64_t m = base + kTry[t];
+      if (m <= 0 || m >= (int64_t(1) << 31)) continue;
+      // floor((65536 r + h) m / 2^32) = exact  <=>  exact 2^32 <= (65536 r + h) m < (exact + 1) 2^32
+      int64_t lo = 0, hi = 65535;
+      for (int r = -128; r <= 127 && lo <= hi; ++r) {
+        const int64_t exact = ((int64_t)r * k->b_r + (int64_t(1) << (k->c_r - 1))) >> k->c_r;
+        const auto ceil_div = [m](int64_t x) { return x >= 0 ? (x + m - 1) / m : -(-x / m); };
+        lo = std::max(lo, ceil_div(exact * (int64_t(1) << 32)) - r * 65536);
+        hi = std::min(hi, ceil_div((exact + 1) * (int64_t(1) << 32)) - 1 - r * 65536);
+      }
+      if (lo <= hi) { k->res_high = 1; k->res_hm = (int32_t)m; k->res_hk = (int32_t)((lo + hi) / 2); }
+    }
+  }
   return IBERT_OK;
 }
 

@@ -74,6 +74,8 @@ struct LnConsts {
   // the residual rescale in 32-bit arithmetic: (r * res_nb + res_nhalf) >> res_nc with a 24-bit multiplier,
   // offered (res_narrow != 0) only when the host has checked all 256 int8 values against the exact form
   int32_t res_nb, res_nc, res_nhalf, res_narrow;
+  // the same as one multiply-high, ((r << 16) + res_hk) * res_hm >> 32; also checked on all int8 values (res_high != 0)
+  int32_t res_hm, res_hk, res_high;
 };
 
 int dyadic(double m, int32_t* b, int32_t* c);

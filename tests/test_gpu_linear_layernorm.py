@@ -134,3 +134,17 @@ def test_linear_layernorm_by_rounds_of_tiles(M, N, K):
                                              gamma, beta, S_out)
     ctx().check()
     assert_same(host(out), _oracle(*p), f"linear+LN {M}x{N}x{K}")
+
+
+# residual scales from 1/3 to about 1000 times the sum's: the multiply-high form exists for nearly all of the small
+# ratios and not for all of the large ones
+@pytest.mark.parametrize("res_ratio", [0.002, 0.011, 0.13, 0.7, 2.9, 5.1, 5.3, 5.5, 5.7, 5.9])
+def test_linear_layernorm_residual_forms(res_ratio):
+    M, N, K = 5000, 768, 128
+    p = _problem(M, N, K, 77, res_ratio)
+    x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
+    ctx().ibert_set_fusion(1)
+    out, _ = ctx().ibert_linear_layernorm_i8(dev(x), S_x, dev(w), S_w, dev(bias), S_mid, dev(res), S_res,
+                                             gamma, beta, S_out)
+    ctx().check()
+    assert_same(host(out), _oracle(*p), f"residual at {S_res / S_mid:.3g} times the scale of the sum")
