@@ -237,7 +237,8 @@ __device__ __forceinline__ uint32_t isqrt_of_quotient(uint64_t ss, uint32_t C) {
 // returns for n = floor(ss / C).  A 64-bit integer division costs on the order of a hundred
 // instructions here, so instead of iterating x <- (x + n/x)/2 a group of GROUP lanes (32 or 16; ss is the group's) finds
 // the same integer by a radix-GROUP search: in each round its lanes test GROUP candidates with one multiply each.
-// Needs s < 2^25 and ss < 2^61 / C.
+// Needs s < 2^25 (GROUP = 16: 2^24, six rounds; a seventh would test candidates up to 15 2^24, whose s^2 C passes
+// 64 bits) and C < 2^12.  The rounds are those of the larger root of a warp: more of them change nothing.
 template <int GROUP = 32>
 __device__ __forceinline__ uint32_t warp_isqrt_of_quotient(uint64_t ss, uint32_t C, int lane) {
   constexpr int kDigit = GROUP == 32 ? 5 : 4;
@@ -245,7 +246,7 @@ __device__ __forceinline__ uint32_t warp_isqrt_of_quotient(uint64_t ss, uint32_t
   uint32_t base = 0;
   // ss / C < 2^bits bounds the result below 2^ceil(bits / 2): rounds above that cannot set a digit
   const int bits = 64 - __clzll((long long)(ss | 1ull)) - (31 - __clz((int)C));
-  int need = min(max((bits + 1) >> 1, 1), 25);
+  int need = min(max((bits + 1) >> 1, 1), GROUP == 32 ? 25 : 24);
   if constexpr (GROUP != 32) need = __reduce_max_sync(0xffffffffu, need);
   for (int shift = kDigit * ((need + kDigit - 1) / kDigit - 1); shift >= 0; shift -= kDigit) {
     const uint32_t cand = base + ((uint32_t)li << shift);

@@ -374,6 +374,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       break;
     }
     const uint8_t* sq = ring + (size_t)slot * slot_bytes;
+    const bool second = R == 1 || group * R + 1 < rows;         // (an odd row count: the last group has one row)
     int32_t v[R][VPL][4];
     uint32_t rw[R][VPL];
 #pragma unroll
@@ -381,7 +382,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
 #pragma unroll
       for (int j = 0; j < VPL; ++j) {
         const int col = 4 * (j * 32 + lane);
-        if (FULL || col < C) {
+        if ((FULL || col < C) && (h == 0 || second)) {           // (a row that was not copied counts as zeros)
           load_q4(reinterpret_cast<const QT*>(sq + h * q_bytes) + col, v[h][j], false);
           rw[h][j] = *reinterpret_cast<const uint32_t*>(sq + R * q_bytes + h * r_bytes + col);
         } else {
@@ -428,7 +429,6 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       norm[h] = R == 1 ? own : LnNorm{__shfl_sync(0xffffffffu, own.scale, 16 * h), __shfl_sync(0xffffffffu, own.shift, 16 * h),
                                       __shfl_sync(0xffffffffu, own.rho, 16 * h)};
     int8_t* orow = out + group * R * C;
-    const bool second = R == 1 || group * R + 1 < rows;
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
       const int col = 4 * (j * 32 + lane);

@@ -161,3 +161,27 @@ def test_rowops_error_codes_on_device_context():
                                 np.ones(2048), np.zeros(2048), 0.02)
     assert e.value.code == -2
     assert ctx().ibert_last_status() == 0
+
+
+# From 24 rows per SM on a warp of the streaming kernel takes two rows together: row counts on both sides of the switch
+# (148 SMs: 3552) and of a grid with one pair of rows per warp (C > 768: 4736, else 7104), odd ones with a last pair of
+# one row.  Shared memory is filled before each call by an int16 call whose every 32-bit word, Q16 values and residuals
+# alike, is 2^26 + 2^20 - 1: read as an int32 row it has wrapped sums (sum 2^30 - 2^10, squares below sum^2 / C), whose
+# "variance" is as large as 64 bits go -- statistics that a row beside it must not see.
+@pytest.mark.parametrize("C", [256, 512, 768, 1008, 1024])
+@pytest.mark.parametrize("dtype", [np.int32, np.int16])
+def test_layernorm_of_row_pairs(C, dtype):
+    c, rng = ctx(), np.random.default_rng(C)
+    gamma, beta, S, S_r, S_out = rng.normal(1.0, 0.1, C), rng.normal(0.0, 0.1, C), 1e-3, 2e-5, 4.5 / 127.0
+    word = np.array([2 ** 26 + 2 ** 20 - 1], np.int32)
+    fill_q, fill_r = dev(np.tile(word.view(np.int16), (7104, 512))), dev(np.tile(word.view(np.int8), (7104, 256)))
+    q = rng.integers(-20000, 20001, (7105, C)).astype(np.int32)
+    r = rng.integers(-127, 128, (7105, C)).astype(np.int8)
+    want = oracle.layernorm(q, S, r, S_r, gamma, beta, S_out)[0]
+    qd, rd = dev(q.astype(dtype)), dev(r)
+    for rows in (3551, 3552, 3553, 3555, 4001, 4721, 4735, 4736, 4737, 7103, 7105):
+        c.ibert_layernorm_i(fill_q, S, fill_r, S_r, np.ones(1024), np.zeros(1024), S_out)
+        c.check()                                             # (the filling blocks have left their SMs)
+        out, _ = c.ibert_layernorm_i(qd[:rows], S, rd[:rows], S_r, gamma, beta, S_out)
+        assert_same(host(out), want[:rows], f"layernorm {rows}x{C}")
+    c.check()
