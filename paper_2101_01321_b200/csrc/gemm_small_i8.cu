@@ -332,7 +332,7 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   }
   if (!ok) atomicCAS(a.status, 0, IBERT_ERR_TIMEOUT);
   ptx::tc_fence_before_sync();
-  __syncthreads();
+  ok = __syncthreads_and(ok);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tile.tmem_base, a.tmem_cols);
@@ -364,8 +364,16 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   }
   if (!ptx::mbar_wait_cluster(bar_part, 0)) ok = false;
   ok = __all_sync(0xffffffffu, ok);
-  if (!ok) {                                                 // (a peer gave up; its records may never come)
+  // After an expired wait nothing is stored, and nobody leaves while a peer may still send records here: the barrier of
+  // the cluster waits for the threads that have not exited, and a peer that has all its records has sent its own.
+  auto give_up = [&] {
     atomicCAS(a.status, 0, IBERT_ERR_TIMEOUT);
+    ptx::cluster_sync();
+#pragma unroll 1
+    for (int i = 0; i < 10000 && !ptx::mbar_test_cluster(bar_part, 0); ++i);   // records still on their way
+  };
+  if (TPW == 1 && !ok) {
+    give_up();
     return;
   }
 
@@ -406,7 +414,10 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       // (the token's own records are consumed: the first one's place takes the result)
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(s_part + threadIdx.x * 16), "r"(pr.scale), "r"(pr.shift), "r"(pr.rho), "r"(0) : "memory");
     }
-    __syncthreads();
+    if (!__syncthreads_and(ok)) {                            // (several tokens per warp: the warps of a CTA meet here)
+      give_up();
+      return;
+    }
   }
   // pass 4: normalize, affine + requantize, store
   const int32_t bb[4] = {bv.x, bv.y, bv.z, bv.w};

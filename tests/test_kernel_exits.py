@@ -1,0 +1,53 @@
+"""How the kernels leave, read from their source: what only shows after a wait has run out cannot be run on a shared GPU."""
+import re
+from pathlib import Path
+
+import pytest
+
+CSRC = Path(__file__).resolve().parent.parent / "paper_2101_01321_b200" / "csrc"
+
+
+def _kernels():
+    """(name, body without comments) of every __global__ function."""
+    for path in sorted(CSRC.glob("*.cu")):
+        text = re.sub(r"//[^\n]*", "", path.read_text())
+        for m in re.finditer(r"__global__\s+void\b[^{;]*?(\w+_kernel)\s*\([^{;]*\)\s*\{", text):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+            yield m.group(1), text[m.end():i - 1]
+
+
+KERNELS = dict(_kernels())
+
+
+def test_kernels_are_found():
+    assert {"gemm_ln_small_kernel", "gemm_small_kernel", "attention_small_kernel", "gemm_ln_kernel", "gemm_splitk_kernel",
+            "gemm_i8_kernel", "layernorm_pipe_kernel"} <= set(KERNELS)
+
+
+def _lambdas(body):
+    """{name: text} of the lambdas of a kernel, and the body without them."""
+    found, rest = {}, body
+    while m := re.search(r"auto\s+(\w+)\s*=\s*\[[&=]?\]\s*(?:\([^)]*\))?\s*\{", rest):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(rest[i], 0)
+            i += 1
+        found[m.group(1)], rest = rest[m.end():i - 1], rest[:m.start()] + rest[i:]
+    return found, rest
+
+
+@pytest.mark.parametrize("name", sorted(n for n, b in KERNELS.items() if "map_to_cta" in b))
+def test_no_cta_leaves_while_a_peer_may_write_to_it(name):
+    """A kernel that reaches into a peer's shared memory leaves early only behind a barrier of its cluster, and at its
+    end behind one or behind the wait that counts what every peer sends."""
+    body = KERNELS[name]
+    lambdas, main = _lambdas(body)
+    barriers = ["cluster_sync"] + [n for n, text in lambdas.items() if "cluster_sync()" in text]
+    for m in re.finditer(r"\breturn\s*;", main):
+        before = main[:m.start()].rstrip()
+        assert re.search(rf"\b({'|'.join(barriers)})\(\)\s*;$", before), f"{name}: a return without a cluster barrier"
+    last = max(m.end() for m in re.finditer(r"map_to_cta|ld_cluster|st_async|mbar_arrive_remote|bulk_copy_to_cta", body))
+    assert re.search(r"cluster_sync\(\)|mbar_wait_cluster\(", body[last:]), f"{name}: nothing holds a CTA at its end"
