@@ -204,7 +204,7 @@ attention_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::mma_commit(bar_mma);
       }
     }
-    __syncwarp();
+    ok = __all_sync(0xffffffffu, ok);       // (the warp goes on together: one lane alone waited for V)
   }
   // ---- epilogue: copy 0's lanes, 16 of the 64 context values per thread
   const int q_row = qt * rows + row;

@@ -51,3 +51,32 @@ def test_no_cta_leaves_while_a_peer_may_write_to_it(name):
         assert re.search(rf"\b({'|'.join(barriers)})\(\)\s*;$", before), f"{name}: a return without a cluster barrier"
     last = max(m.end() for m in re.finditer(r"map_to_cta|ld_cluster|st_async|mbar_arrive_remote|bulk_copy_to_cta", body))
     assert re.search(r"cluster_sync\(\)|mbar_wait_cluster\(", body[last:]), f"{name}: nothing holds a CTA at its end"
+
+
+def _end_of_block(text, i):
+    """Position behind the block whose opening brace lies before `i`."""
+    depth = 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+    return i
+
+
+@pytest.mark.parametrize("name", sorted(KERNELS))
+def test_no_warp_vote_that_an_elected_lane_may_miss(name):
+    """What one elected lane found out (`ok` of a wait that ran out) is voted on by its whole warp before any branch on
+    it holds a vote or barrier: a lane that skips the branch would leave the others waiting there for good."""
+    body = KERNELS[name]
+    for m in re.finditer(r"if \([^;{}]*elect_one\(\)\)\s*\{", body):
+        end = _end_of_block(body, m.end())
+        if not re.search(r"\bok\s*=", body[m.end():end]):
+            continue
+        vote = re.search(r"__all_sync\(|__syncthreads_and\(|__any_sync\(", body[end:])
+        if not vote:
+            continue
+        for cond in re.finditer(r"if \(([^;{}]*)\)\s*(\{)?", body[end:end + vote.start()]):
+            if not re.search(r"\bok\b", cond.group(1)):
+                continue
+            at = end + cond.end()
+            stop = _end_of_block(body, at) if cond.group(2) else body.index(";", at)
+            assert stop < end + vote.start(), f"{name}: a vote inside `if ({cond.group(1)})`"
