@@ -16,10 +16,11 @@ constexpr int kThreads = 256;
 // ----------------------------------------------------------------------------- i-GELU
 // Each thread converts 4 int4 vectors (16 values); vector j of a thread sits 32 vectors
 // after vector j-1 so that every load and store instruction of a warp is contiguous.
-// FORM: kGeluAny takes every constant set; the others are the upper-word form of i-GELU without / with the pre-shift
-// of the erf argument and without / with a lower clamp (GeluConsts::low_free).  Bound by the ALU pipe in the general
-// form (12 of 20 instructions per element), close to HBM without the shift and the clamp: 2^24 elements 16.7 -> 14.5 us.
-enum { kGeluAny = 0, kGeluPlain = 1, kGeluShift = 2, kGeluClamp = 3, kGeluShiftClamp = 4 };
+// FORM: the upper-word form of i-GELU without / with the pre-shift of the erf argument and without / with a lower clamp
+// (GeluConsts::low_free), that of h-GELU, and both functions with the 64-bit product for the other constant sets.  Bound
+// by the ALU pipe with shift and clamp (12 of 20 instructions per element), close to HBM without: 2^24 elements
+// 16.7 -> 14.5 us.  One form per instance: chosen per element at run time h-GELU takes 15.5 us instead of 13.1.
+enum { kGeluPlain, kGeluShift, kGeluClamp, kGeluShiftClamp, kGeluExact, kHgelu, kHgeluExact };
 template <int FORM>
 __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restrict__ q, int64_t n,
                                                         GeluConsts k, int8_t* __restrict__ out) {
@@ -34,12 +35,12 @@ __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restric
   const int4* q4 = reinterpret_cast<const int4*>(q);
   uint32_t* o4 = reinterpret_cast<uint32_t*>(out);
   auto gelu = [&](int32_t x) {
-    if constexpr (FORM != kGeluAny) {
+    if constexpr (FORM == kHgelu) return max(ihgelu_upper(x, k), -127);
+    else if constexpr (FORM == kHgeluExact) return ihgelu_to_int8(clamp_sym(x, 32767), k, half);
+    else if constexpr (FORM == kGeluExact) return igelu_q16_to_int8(clamp_sym(x, 32767), k, half);
+    else {
       const int32_t r = igelu_magnitude_upper<FORM == kGeluShift || FORM == kGeluShiftClamp>(x, k, rnd_f);
       return FORM == kGeluClamp || FORM == kGeluShiftClamp ? max(r, -127) : r;
-    } else {
-      if (k.hard) return k.fast ? max(ihgelu_upper(x, k), -127) : ihgelu_to_int8(clamp_sym(x, 32767), k, half);
-      return k.fast ? max(igelu_magnitude_upper(x, k, rnd_f), -127) : igelu_q16_to_int8(clamp_sym(x, 32767), k, half);
     }
   };
   for (int64_t base = warp_global * 128; base < n_vec; base += warp_count * 128) {
@@ -705,7 +706,9 @@ int launch_gelu(ibert_ctx* ctx, const int32_t* q, int64_t n, const GeluConsts& k
   const int64_t warps = ((n >> 2) + 127) / 128 + 1;
 #define IBERT_GELU(F) \
   return launch_pdl(gelu_kernel<F>, dim3(wave_grid(ctx, gelu_kernel<F>, warps)), dim3(kThreads), 0, ctx->stream, 1, q, n, k, out)
-  if (k.hard || !k.fast) IBERT_GELU(kGeluAny);
+  if (k.hard && k.fast) IBERT_GELU(kHgelu);
+  if (k.hard) IBERT_GELU(kHgeluExact);
+  if (!k.fast) IBERT_GELU(kGeluExact);
   if (k.low_free && k.s_in == 0) IBERT_GELU(kGeluPlain);
   if (k.low_free) IBERT_GELU(kGeluShift);
   if (k.s_in == 0) IBERT_GELU(kGeluClamp);
