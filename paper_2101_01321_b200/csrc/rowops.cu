@@ -20,11 +20,13 @@ constexpr int kThreads = 256;
 // (GeluConsts::low_free), that of h-GELU, and both functions with the 64-bit product for the other constant sets.  Bound
 // by the ALU pipe with shift and clamp (12 of 20 instructions per element), close to HBM without: 2^24 elements
 // 16.7 -> 14.5 us.  One form per instance: chosen per element at run time h-GELU takes 15.5 us instead of 13.1.
+// The next kernel may start once a block has stored its last values, not before: its blocks would take the places
+// of this one's second and third wave.  us, trigger first / last: 2^17 elements 1.69 / 1.64, 2^20 2.60 / 2.13, 2^21
+// 3.57 / 2.93, 5 10^6 5.11 / 5.25, 2^24 13.65 / 13.61.
 enum { kGeluPlain, kGeluShift, kGeluClamp, kGeluShiftClamp, kGeluExact, kHgelu, kHgeluExact };
 template <int FORM>
 __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restrict__ q, int64_t n,
                                                         GeluConsts k, int8_t* __restrict__ out) {
-  ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int64_t half = rounding_half(k.c);
   const int64_t n_vec = n >> 2;
@@ -56,6 +58,7 @@ __global__ void __launch_bounds__(kThreads) gelu_kernel(const int32_t* __restric
       if (idx < n_vec) __stcs(o4 + idx, pack4_sat_s8(gelu(v[j].x), gelu(v[j].y), gelu(v[j].z), gelu(v[j].w)));
     }
   }
+  ptx::grid_dep_launch();
   // ragged tail (n not a multiple of 4)
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int64_t tail = n_vec << 2;
