@@ -386,7 +386,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
 #pragma unroll
       for (int j = 0; j < VPL; ++j) {
         const int col = 4 * (j * 32 + lane);
-        if ((FULL || col < C) && (h == 0 || second)) {           // (a row that was not copied counts as zeros)
+        if (FULL || col < C) {                                   // (a row that was not copied: whatever lies there)
           load_q4(reinterpret_cast<const QT*>(sq + h * q_bytes) + col, v[h][j], false);
           rw[h][j] = *reinterpret_cast<const uint32_t*>(sq + R * q_bytes + h * r_bytes + col);
         } else {
@@ -421,7 +421,8 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       // a lane's share is below 2^50 (|v| <= 2^21, at most 64 values): two 25-bit halves reduce as 32-bit sums
       t2 = (uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)t2 & 0x1ffffffu) +
            ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(t2 >> 25)) << 25);
-      if (h == 0 || lane >= 16) { sum = t; s2 = t2; }            // (two rows: the upper half-warp takes the second)
+      // (two rows: the upper half-warp takes the second -- if there is one, for the root search is shared by both)
+      if (h == 0 || (lane >= 16 && second)) { sum = t; s2 = t2; }
     }
     int32_t mu = sum / C;                            // mu = floor(sum / C)
     if (sum - mu * C < 0) mu -= 1;
