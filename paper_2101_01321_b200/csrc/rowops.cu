@@ -378,7 +378,9 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       break;
     }
     const uint8_t* sq = ring + (size_t)slot * slot_bytes;
-    const bool second = R == 1 || group * R + 1 < rows;         // (an odd row count: the last group has one row)
+    // (an odd row count: the last group has one row, and in place of the other lies whatever was there.  Its
+    // statistics are discarded; all they share with the first row's is the number of rounds of the root search, of
+    // which more than a row needs change nothing)
     int32_t v[R][VPL][4];
     uint32_t rw[R][VPL];
 #pragma unroll
@@ -386,7 +388,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
 #pragma unroll
       for (int j = 0; j < VPL; ++j) {
         const int col = 4 * (j * 32 + lane);
-        if (FULL || col < C) {                                   // (a row that was not copied: whatever lies there)
+        if (FULL || col < C) {
           load_q4(reinterpret_cast<const QT*>(sq + h * q_bytes) + col, v[h][j], false);
           rw[h][j] = *reinterpret_cast<const uint32_t*>(sq + R * q_bytes + h * r_bytes + col);
         } else {
@@ -421,8 +423,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       // a lane's share is below 2^50 (|v| <= 2^21, at most 64 values): two 25-bit halves reduce as 32-bit sums
       t2 = (uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)t2 & 0x1ffffffu) +
            ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(t2 >> 25)) << 25);
-      // (two rows: the upper half-warp takes the second -- if there is one, for the root search is shared by both)
-      if (h == 0 || (lane >= 16 && second)) { sum = t; s2 = t2; }
+      if (h == 0 || lane >= 16) { sum = t; s2 = t2; }            // (two rows: the upper half-warp takes the second)
     }
     int32_t mu = sum / C;                            // mu = floor(sum / C)
     if (sum - mu * C < 0) mu -= 1;
@@ -434,6 +435,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       norm[h] = R == 1 ? own : LnNorm{__shfl_sync(0xffffffffu, own.scale, 16 * h), __shfl_sync(0xffffffffu, own.shift, 16 * h),
                                       __shfl_sync(0xffffffffu, own.rho, 16 * h)};
     int8_t* orow = out + group * R * C;
+    const bool second = R == 1 || group * R + 1 < rows;
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
       const int col = 4 * (j * 32 + lane);
