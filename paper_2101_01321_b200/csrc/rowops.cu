@@ -799,12 +799,17 @@ static int launch_layernorm_t(ibert_ctx* ctx, const QT* q, const int8_t* r, int6
   const int vpl = (k.C + 127) / 128;
   const bool fast = vec && k.out_fast && (!k.has_res || k.res_fast);
   if (fast && k.has_res && k.res_narrow && k.C % 16 == 0 && k.C <= 1024) {
-    // streaming variant: per-warp ring of row slots filled by bulk async copies.  Two rows per warp once every warp of
-    // the resident wave has work that way; below, one row per warp keeps more warps busy
+    // streaming variant: per-warp ring of row slots filled by bulk async copies.  Two rows per warp once the warps of the
+    // resident wave have work that way; below, one row per warp keeps more warps busy (us, one row / two, int32 input:
+    // C = 256: 3800 rows 3.93 / 3.69; C = 512: 4300 4.94 / 5.24, 5000 5.92 / 5.38; C = 768: 4300 6.27 / 6.81, 5000
+    // 7.44 / 6.93; C = 1024: 3553 6.67 / 6.45).  Above 768 channels two CTAs are resident with two rows per warp and two or three
+    // with one: the second round of pairs starts where one row per warp fills its rounds (6500 rows 9.58 / 10.71,
+    // 7500 10.41 / 10.93, 9000 12.19 / 10.91; int16 9.15 / 10.21, 10.46 / 10.37, 13.06 / 10.39).
     // (one-row slots are double-buffered, two-row slots single: the registers are the second buffer)
     const size_t smem = (size_t)(kThreads / 32) * 2 * (size_t)k.C * (sizeof(QT) + 1) + (kThreads / 32) * 2 * 8 +
                         (size_t)k.C * 12;                  // rows in flight, barriers, the two tables
-    const bool two = rows >= (int64_t)ctx->num_sms * 3 * (kThreads / 32);
+    const int64_t sms = ctx->num_sms;
+    const bool two = k.C <= 256 ? rows >= 24 * sms : k.C <= 768 ? rows >= 32 * sms : rows >= 24 * sms && (rows <= 40 * sms || rows >= 48 * sms);
     // one wave of resident CTAs: by registers three per SM (two for two rows of more than 768 channels), fewer when
     // the row slots take more shared memory (C = 1024 with int32 input: two)
     const int by_regs = two && k.C > 768 ? 2 : 3;
