@@ -800,16 +800,18 @@ static int launch_layernorm_t(ibert_ctx* ctx, const QT* q, const int8_t* r, int6
   const bool fast = vec && k.out_fast && (!k.has_res || k.res_fast);
   if (fast && k.has_res && k.res_narrow && k.C % 16 == 0 && k.C <= 1024) {
     // streaming variant: per-warp ring of row slots filled by bulk async copies.  Two rows per warp once the warps of the
-    // resident wave have work that way; below, one row per warp keeps more warps busy (us, one row / two, int32 input:
-    // C = 256: 3800 rows 3.93 / 3.69; C = 512: 4300 4.94 / 5.24, 5000 5.92 / 5.38; C = 768: 4300 6.27 / 6.81, 5000
-    // 7.44 / 6.93; C = 1024: 3553 6.67 / 6.45).  Above 768 channels two CTAs are resident with two rows per warp and two or three
-    // with one: the second round of pairs starts where one row per warp fills its rounds (6500 rows 9.58 / 10.71,
-    // 7500 10.41 / 10.93, 9000 12.19 / 10.91; int16 9.15 / 10.21, 10.46 / 10.37, 13.06 / 10.39).
+    // resident wave have work that way; below, one row per warp keeps more warps busy.  From 257 to 768 channels the
+    // two cross later, int16 rows just past one full wave of single rows, int32 rows a third further (us with one row /
+    // with two, behind an unrelated kernel and, in brackets, call behind call; 1.6 us of the former are that kernel):
+    //   C = 256 int32   3553 rows 5.1 / 5.0 (3.1 / 3.6)   3800 5.4 / 5.0 (3.9 / 3.7)   4735 5.6 / 5.1
+    //   C = 768 int16   3553 rows 6.5 / 6.9 (4.5 / 6.4)   3800 7.4 / 7.0 (5.4 / 6.4)   4735 7.5 / 7.1
+    //   C = 768 int32   3553 rows 6.7 / 7.4 (4.7 / 6.7)   4000 7.4 / 7.4 (5.5 / 6.8)   4737 7.6 / 7.7 (7.0 / 6.8)   7000 9.8 / 9.1
+    //   C = 1024 int32  3553 rows 7.8 / 8.3 (6.7 / 6.5)   3800 8.7 / 8.3 (6.9 / 6.5)   7000 11.6 / 10.5 (9.6 / 10.8)
     // (one-row slots are double-buffered, two-row slots single: the registers are the second buffer)
     const size_t smem = (size_t)(kThreads / 32) * 2 * (size_t)k.C * (sizeof(QT) + 1) + (kThreads / 32) * 2 * 8 +
                         (size_t)k.C * 12;                  // rows in flight, barriers, the two tables
-    const int64_t sms = ctx->num_sms;
-    const bool two = k.C <= 256 ? rows >= 24 * sms : k.C <= 768 ? rows >= 32 * sms : rows >= 24 * sms && (rows <= 40 * sms || rows >= 48 * sms);
+    const int line = k.C <= 256 || k.C > 768 ? 24 : sizeof(QT) == 4 ? 32 : 25;       // rows per SM
+    const bool two = rows >= (int64_t)ctx->num_sms * line;
     // one wave of resident CTAs: by registers three per SM (two for two rows of more than 768 channels), fewer when
     // the row slots take more shared memory (C = 1024 with int32 input: two)
     const int by_regs = two && k.C > 768 ? 2 : 3;
