@@ -851,7 +851,7 @@ static int encoder_layer_common(ibert_ctx* ctx, const ibert_layer* ly, const int
   // holds one channel of 32 tokens, which are contiguous bytes of that layout
   const bool qkv_t = ctx->qkv_layout_mode != 1 && !cu_seqlens && ly->fast_qkv == 1 &&
                      attention_takes_transposed(B, L, ly->attn) &&
-                     !(ctx->qkv_layout_mode == 0 && ctx->splitk_mode == 0 && gemm_small_takes(ctx, T, 3 * H, H));
+                     !(ctx->qkv_layout_mode == 0 && ctx->splitk_mode == 0 && gemm_small_takes(ctx, T, 3 * H, H, true));
   e.out_transposed = qkv_t;
   { ProfileScope ps(ctx, IBERT_K_GEMM_QKV); rc = launch_gemm_i8(ctx, x, ly->w_qkv, T, 3 * H, H, e, qkv); }
   e.out_transposed = false;

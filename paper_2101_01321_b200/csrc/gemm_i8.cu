@@ -523,7 +523,7 @@ int launch_gemm_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, 
       if ((!int8_ok && !gelu_ok) || M % 16 != 0) return IBERT_ERR_ARG;
     }
     // one wave of small tiles
-    if (ctx->splitk_mode == 0 && !epi.out_transposed && gemm_small_takes(ctx, M, N, K))
+    if (ctx->splitk_mode == 0 && !epi.out_transposed && gemm_small_takes(ctx, M, N, K, epi.w_static))
       return launch_gemm_small_i8(ctx, x, w, M, N, K, epi, out);
     int split = (ctx->splitk_mode == 1 || epi.fast == 2 || epi.out_transposed) ? 1 : gemm_splitk_width(ctx, M, N, K);
     if ((ctx->splitk_mode == 2 || ctx->splitk_mode == 4) && K > 128 && epi.fast != 2 && !epi.out_transposed &&

@@ -30,6 +30,7 @@ constexpr int kWSpan = kCh * kSpan, kWBytes = kCh * kBK;
 constexpr int kMaxStages = 8;
 constexpr int kIssuers = 2;        // MMA-issuing warps
 constexpr int kMaxTok = 128;       // tokens per tile (plain form)
+constexpr int kMaxTokLateW = 96;   // the same when the weights are no layer's own
 constexpr int kMaxTokLn = 64;      // tokens per tile (LayerNorm form)
 constexpr int kMaxCluster = 8;     // CTAs per token tile (LayerNorm form): H <= 1024
 constexpr int kMaxSmallThreads = 512;
@@ -452,10 +453,14 @@ uint32_t tmem_columns(int n) {
   return c;
 }
 
-// tokens per tile that give one wave of CTAs, or 0 when the problem is larger than that
-int small_tile_tokens(const ibert_ctx* ctx, int64_t M, int N) {
+// Tokens per tile that give one wave of CTAs, or 0 when the problem is larger than that.  Weights that may not be read
+// ahead of the dependency wait leave the two-stage ring of 112 and 128 tokens without its head start, and the large
+// tiles are faster there (single linear layers, us, this kernel / large tiles: 765 x 2304 x 768, 96 tokens, 4.5 / 4.6;
+// 1021 x 2304 x 768, 128 tokens, 5.0 / 4.3; 1725 x 1024 x 4096, 96 tokens, 8.6 / 10.3; 2301 x 1024 x 4096, 128 tokens,
+// 12.0 / 8.7).  Inside a layer it is the other way round: Base 4 x 256 34.7 / 42.0 us, 7 x 128 31.2 / 32.9.
+int small_tile_tokens(const ibert_ctx* ctx, int64_t M, int N, bool w_static) {
   const int c_tiles = (N + kCh - 1) / kCh, t_max = ctx->num_sms / c_tiles;
-  if (t_max < 1 || M > (int64_t)t_max * kMaxTok) return 0;
+  if (t_max < 1 || M > (int64_t)t_max * (w_static ? kMaxTok : kMaxTokLateW)) return 0;
   const int per = (int)((M + t_max - 1) / t_max);
   return std::max((per + 15) & ~15, 16);
 }
@@ -537,14 +542,14 @@ SmallArgs small_args(ibert_ctx* ctx, int64_t M, int N, int K, int nt, int extra_
 
 }  // namespace
 
-bool gemm_small_takes(const ibert_ctx* ctx, int64_t M, int N, int K) {
-  return M > 0 && K >= 256 && K % 16 == 0 && small_tile_tokens(ctx, M, N) > 0;
+bool gemm_small_takes(const ibert_ctx* ctx, int64_t M, int N, int K, bool w_static) {
+  return M > 0 && K >= 256 && K % 16 == 0 && small_tile_tokens(ctx, M, N, w_static) > 0;
 }
 
 int launch_gemm_small_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int N, int K,
                          const GemmEpilogue& epi, void* out) {
-  if (!gemm_small_takes(ctx, M, N, K)) return IBERT_ERR_ARG;
-  const SmallArgs a = small_args(ctx, M, N, K, small_tile_tokens(ctx, M, N), 0, epi, out);
+  if (!gemm_small_takes(ctx, M, N, K, epi.w_static)) return IBERT_ERR_ARG;
+  const SmallArgs a = small_args(ctx, M, N, K, small_tile_tokens(ctx, M, N, epi.w_static), 0, epi, out);
   CUtensorMap mw, mx;
   if (int rc = operand_maps(&mw, &mx, w, x, M, N, K, a.nt)) return rc;
   const int grid = ((N + kCh - 1) / kCh) * (int)((M + a.nt - 1) / a.nt);

@@ -213,7 +213,7 @@ int launch_gemm_splitk_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int6
 
 // One-wave kernels for small token counts (128 channels x 16..128 tokens per CTA; with LayerNorm a cluster of
 // H / 128 CTAs per 16..64 tokens).  The two predicates tell whether the problem is one wave or less.
-bool gemm_small_takes(const ibert_ctx* ctx, int64_t M, int N, int K);
+bool gemm_small_takes(const ibert_ctx* ctx, int64_t M, int N, int K, bool w_static);
 int launch_gemm_small_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int N, int K,
                          const GemmEpilogue& epi, void* out);
 bool gemm_ln_small_supported(const ibert_ctx* ctx, int64_t M, int H, int K, const GemmEpilogue& epi, const LnConsts& ln);

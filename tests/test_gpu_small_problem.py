@@ -6,6 +6,7 @@ import pytest
 
 import oracle
 from gpu_util import assert_same, ctx, dev, host
+from paper_2101_01321_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -23,7 +24,7 @@ def _linear_problem(M, N, K, seed):
 # one token; a tile and one past it; channel and K tails; the longest ring; the largest one-wave sizes of a wide
 # and a narrow layer and the first size past each
 @pytest.mark.parametrize("M,N,K", [(1, 128, 256), (16, 144, 272), (17, 2304, 768), (33, 272, 400), (129, 768, 3072),
-                                   (50, 4096, 1024), (113, 320, 4096), (768, 3072, 768), (769, 3072, 768),
+                                   (50, 4096, 1024), (113, 320, 4096), (576, 3072, 768), (577, 3072, 768), (768, 3072, 768), (769, 3072, 768),
                                    (1024, 2304, 768), (1025, 2304, 768)])
 def test_linear_kinds(M, N, K):
     x, w, bias, S_w, S_x, amax = _linear_problem(M, N, K, M + N + K)
@@ -37,6 +38,17 @@ def test_linear_kinds(M, N, K):
     out, _ = ctx().ibert_linear_hgelu_i8(dev(x), S_in, dev(w), S_w, dev(bias), S_mid, S_out)
     assert_same(host(out), oracle.hgelu(mid, S_mid, S_out)[0], "hgelu")
     ctx().check()
+
+
+# layers whose QKV or FFN1 GEMM has the widest one-wave tiles (112 and 128 tokens), which only layer-owned weights take
+@pytest.mark.parametrize("B,L", [(8, 109), (8, 125), (5, 151), (9, 114)])
+def test_encoder_layer_widest_tiles(B, L):
+    x, params = synth.make_model(0, B, layers=1, H=768, heads=12, F=3072, L=L)
+    layer = ctx().ibert_layer_create(params[0])
+    out, _ = ctx().ibert_encoder_layer(layer, dev(x), B, L)
+    ctx().check()
+    layer.close()
+    assert_same(host(out), oracle.encoder_layer(params[0], x, B, L).out, f"encoder layer {B}x{L}")
 
 
 # 1, 2, 3, 5, 6 and 8 CTAs per cluster (channel counts that are and are not powers of two); 1 to 4 tokens per warp
