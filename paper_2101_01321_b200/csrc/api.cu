@@ -1161,6 +1161,12 @@ int ibert_selftest_exp_division(double S, int32_t* q_ln2_out) {
       if ((nf > 31 ? 0u : (uint32_t)(tf * tf + k.q_c) >> nf) != want) return IBERT_ERR_VALUE_RANGE;
     }
   }
+  for (uint32_t d = 0; d <= k.d_max; ++d) {      // the quotient of clamped distances, again by the exponential
+    const uint32_t z = d / k.q_ln2, n = z + (uint32_t)k.s_out, zf = (uint32_t)(((uint64_t)(d + (uint32_t)k.row_add) * (uint64_t)k.row_m) >> 32);
+    const int32_t t = k.q_b - (int32_t)(d - z * k.q_ln2), tf = k.q_b - (int32_t)(d - zf * k.q_ln2);
+    const uint32_t nf = zf + (uint32_t)k.s_out;
+    if ((nf > 31 ? 0u : (uint32_t)(tf * tf + k.q_c) >> nf) != (n > 31 ? 0u : (uint32_t)(t * t + k.q_c) >> n)) return IBERT_ERR_VALUE_RANGE;
+  }
   if (k.wide_post >= 0) {            // the unclamped form used on attention scores: every d < 2^21
     for (uint32_t d = 0; d < (1u << 21); ++d) {
       const uint32_t z = (uint32_t)(((uint64_t)d * (uint64_t)k.wide_m) >> 32) >> k.wide_post;

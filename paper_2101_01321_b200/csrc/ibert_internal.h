@@ -35,9 +35,13 @@ struct ExpConsts {
   // the quotient and the post-shift in one multiply-high (attention scores): with the distance d' offset to
   // D = d' + s_out q_ln2 + fold_add,  umulhi(D, fold_m) = floor(d' / q_ln2) + s_out -- the whole shift count of
   // Algorithm 3 -- wherever e is not zero, and a count that still shifts everything out beyond.  fold_m = 0:
-  // not available (q_ln2 < 16, and a few q_ln2 above 16645)
+  // not available (q_ln2 < 16, and 16716)
   uint32_t fold_m;
   int32_t fold_add;
+  // the quotient alone for distances clamped to d_max (standalone i-softmax): umulhi(d' + row_add, row_m) =
+  // floor(d' / q_ln2) wherever e is not zero, and a count that still shifts everything out beyond.  Every scale has it.
+  uint32_t row_m;
+  int32_t row_add;
 };
 
 // i-GELU (Algorithm 2) followed by requantization to int8

@@ -95,10 +95,6 @@ __global__ void __launch_bounds__(kThreads) gelu_lut_kernel(const int32_t* __res
 }
 
 // ----------------------------------------------------------------------------- i-softmax
-// One warp per row; a lane keeps VPL int4 vectors (4*VPL scores) in registers.
-// VEC: rows are 16-byte aligned (L % 4 == 0) and loaded/stored as vectors.
-// DIV 0..2: how i-exp divides by q_ln2.  (softmax_group_kernel takes every scale but the coarsest.)
-
 // table[i] = i-exp of the pre-shifted distance i, for i = 0 .. d_max
 __global__ void __launch_bounds__(kThreads) exp_table_kernel(ExpConsts k, uint32_t* __restrict__ table) {
   const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
@@ -106,70 +102,6 @@ __global__ void __launch_bounds__(kThreads) exp_table_kernel(ExpConsts k, uint32
   const uint32_t d = i << k.s_in;
   const int mode = exp_div_mode(k);
   table[i] = mode == 0 ? iexp_dist<0>(d, k) : (mode == 1 ? iexp_dist<1>(d, k) : iexp_dist<2>(d, k));
-}
-
-template <int VPL, bool VEC, int DIV>
-__global__ void __launch_bounds__(kThreads) softmax_kernel(const int32_t* __restrict__ q, int64_t rows,
-                                                           int L, ExpConsts k, uint8_t* __restrict__ out) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
-  const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
-  for (int64_t row = warp_global; row < rows; row += warp_count) {
-    const int32_t* qr = q + row * L;
-    uint8_t* orow = out + row * L;
-    int32_t v[VPL][4];
-    int32_t mx = INT32_MIN;
-#pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-      const int col = 4 * (j * 32 + lane);
-      if (VEC) {
-        if (col < L) {
-          const int4 t = __ldcs(reinterpret_cast<const int4*>(qr + col));
-          v[j][0] = t.x; v[j][1] = t.y; v[j][2] = t.z; v[j][3] = t.w;
-        } else {
-          v[j][0] = v[j][1] = v[j][2] = v[j][3] = INT32_MIN;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[j][i] = (col + i < L) ? qr[col + i] : INT32_MIN;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) mx = max(mx, v[j][i]);
-    }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    uint32_t sum = 0;
-#pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-      const int col = 4 * (j * 32 + lane);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t dist = (uint32_t)mx - (uint32_t)v[j][i];
-        uint32_t e = 0u;
-        if (col + i < L) {
-          e = iexp_dist<DIV>(dist, k);
-        }
-        v[j][i] = (int32_t)e;
-        sum += e;
-      }
-    }
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    const RowDivisor rd = make_row_divisor(sum, k.p_max);
-#pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-      const int col = 4 * (j * 32 + lane);
-      uint32_t p[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = softmax_quotient((uint32_t)v[j][i], rd);
-      if (VEC) {
-        if (col < L)
-          __stcs(reinterpret_cast<uint32_t*>(orow + col), p[0] | (p[1] << 8) | (p[2] << 16) | (p[3] << 24));
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (col + i < L) orow[col + i] = (uint8_t)p[i];
-      }
-    }
-  }
 }
 
 // ----------------------------------------------------------------------------- i-LayerNorm
@@ -560,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, VPL > 4 ? 3 : 4) softmax_group_kerne
   ptx::grid_dep_wait();
   const int64_t total = rows * L;
   const int4* q4 = reinterpret_cast<const int4*>(q);
-  const int32_t wk = k.q_b - k.s_out * (int32_t)k.q_ln2 + k.fold_add;
+  const int32_t wk = k.q_b - k.s_out * (int32_t)k.q_ln2 + k.row_add;
   for (int64_t row0 = warp_global * kRows; row0 < rows; row0 += warp_count * kRows) {
     const int64_t row = row0 + lane / LPR;
     const bool live = row < rows;
@@ -609,8 +541,8 @@ __global__ void __launch_bounds__(kThreads, VPL > 4 ? 3 : 4) softmax_group_kerne
         else {
           // d' = min(d >> s_in, 31 q_ln2); n = floor(d' / q_ln2) + s_out; e = ((q_b - r)^2 + q_c) >> n
           if constexpr (EXP == kExpFoldShift) d >>= k.s_in;
-          d = min(d, k.d_max) + (uint32_t)k.fold_add;
-          const uint32_t n = __umulhi(d, k.fold_m) + (uint32_t)k.s_out;
+          d = min(d, k.d_max) + (uint32_t)k.row_add;
+          const uint32_t n = __umulhi(d, k.row_m) + (uint32_t)k.s_out;
           const int32_t t = (int32_t)(n * k.q_ln2) + (wk - (int32_t)d);
           v[j][i] = shr_clamped((uint32_t)(t * t + k.q_c), n);
         }
@@ -731,64 +663,41 @@ int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const 
                    const uint32_t* exp_table) {
   if (rows == 0) return IBERT_OK;
   const bool vec = (L % 4) == 0;
-  const int vpl = (L + 127) / 128;   // vectors per lane
-  const int div = exp_div_mode(k);
-#define IBERT_SM2(V, D)                                                                                       \
-  do {                                                                                                        \
-    if (vec) softmax_kernel<V, true, D><<<wave_grid(ctx, softmax_kernel<V, true, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out);   \
-    else softmax_kernel<V, false, D><<<wave_grid(ctx, softmax_kernel<V, false, D>, rows), kThreads, 0, ctx->stream>>>(q, rows, L, k, out);      \
-  } while (0)
-#define IBERT_SM(V)                 \
-  do {                              \
-    if (div == 0) IBERT_SM2(V, 0);  \
-    else if (div == 1) IBERT_SM2(V, 1); \
-    else IBERT_SM2(V, 2);           \
-  } while (0)
-  if (exp_table || k.fold_m != 0) {
-    // lanes per row: the fewest (4 to 32) that hold the row in at most four vectors each; L > 509: 32 of eight
-    const int vecs = (L + (vec ? 0 : 3) + 3) / 4;
-    int lpr = 4;
-    while (lpr < 32 && vecs > 4 * lpr) lpr *= 2;
-    const int vpl_g = std::max((vecs + lpr - 1) / lpr, 2);
-    const bool full = vec && L == 4 * lpr * vpl_g;
-    const int form = exp_table ? kExpTable : (k.s_in == 0 ? kExpFold : kExpFoldShift);
-    const int64_t warps = (rows + 32 / lpr - 1) / (32 / lpr);
-#define IBERT_SG3(LPR, VPL, FULL, EXP)                                                                          \
-  return launch_pdl(softmax_group_kernel<LPR, VPL, FULL, EXP>,                                                  \
-                    dim3(wave_grid(ctx, softmax_group_kernel<LPR, VPL, FULL, EXP>, warps)), dim3(kThreads), 0,   \
+  // lanes per row: the fewest (4 to 32) that hold the row in at most four vectors each; L > 509: 32 of eight
+  const int vecs = (L + (vec ? 0 : 3) + 3) / 4;
+  int lpr = 4;
+  while (lpr < 32 && vecs > 4 * lpr) lpr *= 2;
+  const int vpl = std::max((vecs + lpr - 1) / lpr, 2);
+  const bool full = vec && L == 4 * lpr * vpl;
+  const int form = exp_table ? kExpTable : (k.s_in == 0 ? kExpFold : kExpFoldShift);
+  const int64_t warps = (rows + 32 / lpr - 1) / (32 / lpr);
+#define IBERT_SG3(LPR, VPL, FULL, EXP)                                                                       \
+  return launch_pdl(softmax_group_kernel<LPR, VPL, FULL, EXP>,                                               \
+                    dim3(wave_grid(ctx, softmax_group_kernel<LPR, VPL, FULL, EXP>, warps)), dim3(kThreads), 0, \
                     ctx->stream, 1, q, rows, L, k, out, exp_table)
-#define IBERT_SG2(LPR, VPL, FULL)                                  \
-  do {                                                             \
-    if (form == kExpFold) IBERT_SG3(LPR, VPL, FULL, kExpFold);     \
+#define IBERT_SG2(LPR, VPL, FULL)                                             \
+  do {                                                                        \
+    if (form == kExpFold) IBERT_SG3(LPR, VPL, FULL, kExpFold);                \
     else if (form == kExpFoldShift) IBERT_SG3(LPR, VPL, FULL, kExpFoldShift); \
-    else IBERT_SG3(LPR, VPL, FULL, kExpTable);                     \
+    else IBERT_SG3(LPR, VPL, FULL, kExpTable);                                \
   } while (0)
-#define IBERT_SG(LPR)                                  \
-  do {                                                 \
-    if (vpl_g == 2) IBERT_SG2(LPR, 2, false);          \
-    else if (vpl_g == 3) IBERT_SG2(LPR, 3, false);     \
-    else if (full) IBERT_SG2(LPR, 4, true);            \
-    else IBERT_SG2(LPR, 4, false);                     \
+#define IBERT_SG(LPR)                            \
+  do {                                           \
+    if (vpl == 2) IBERT_SG2(LPR, 2, false);      \
+    else if (vpl == 3) IBERT_SG2(LPR, 3, false); \
+    else if (full) IBERT_SG2(LPR, 4, true);      \
+    else IBERT_SG2(LPR, 4, false);               \
   } while (0)
-    if (vpl_g > 8) IBERT_SG2(32, 9, false);            // (1022 and 1023 elements off a 16-byte boundary)
-    else if (vpl_g > 4) IBERT_SG2(32, 8, false);
-    else if (lpr == 4) IBERT_SG(4);
-    else if (lpr == 8) IBERT_SG(8);
-    else if (lpr == 16) IBERT_SG(16);
-    else IBERT_SG(32);
-    return IBERT_ERR_ARG;
+  if (vpl > 8) IBERT_SG2(32, 9, false);            // (1022 and 1023 elements off a 16-byte boundary)
+  else if (vpl > 4) IBERT_SG2(32, 8, false);
+  else if (lpr == 4) IBERT_SG(4);
+  else if (lpr == 8) IBERT_SG(8);
+  else if (lpr == 16) IBERT_SG(16);
+  else IBERT_SG(32);
+  return IBERT_ERR_ARG;
 #undef IBERT_SG
 #undef IBERT_SG2
 #undef IBERT_SG3
-  }
-  // scales so coarse (q_ln2 < 16) or so odd that the one multiply-high does not exist
-  if (vpl <= 1) IBERT_SM(1);
-  else if (vpl <= 2) IBERT_SM(2);
-  else if (vpl <= 4) IBERT_SM(4);
-  else IBERT_SM(8);
-#undef IBERT_SM
-#undef IBERT_SM2
-  return check_launch();
 }
 
 template <typename QT>

@@ -97,3 +97,12 @@ def test_exp_division_by_multiplication_is_exact_for_every_distance(lib):
         seen.add(q.value.bit_length())
     assert len(seen) >= 12                     # divisors of many sizes were exercised
     assert lib.ibert_selftest_exp_division(0.7, None) == -3
+
+
+def test_exp_quotient_of_the_row_kernel_exists_for_every_divisor(lib):
+    """The coarsest scales (divisors 1 to 40), the finest ones and 16716, whose folded multiplier does not exist."""
+    for q_ln2 in [*range(1, 41), *range(16600, 16788, 7), 16716]:
+        q = C.c_int32()
+        S = math.log(2.0) / (q_ln2 + 0.5)
+        assert lib.ibert_selftest_exp_division(S, C.byref(q)) == 0, q_ln2
+        assert q.value == q_ln2

@@ -83,6 +83,21 @@ def test_softmax_extreme_inputs_and_scales():
     ctx().check()
 
 
+# the coarsest scales (divisors of the exponential 1 to 3, on both sides of 16) and one whose folded multiplier does not
+# exist, at row lengths around the 16-byte vectors and lane groups
+@pytest.mark.parametrize("q_ln2", [1, 2, 3, 15, 16, 16716])
+@pytest.mark.parametrize("L", [1, 3, 31, 33, 64, 101, 128, 130, 509, 512, 1021, 1024])
+def test_softmax_scales_at_the_ends(q_ln2, L):
+    S = float(np.log(2.0)) / (q_ln2 + 0.5)
+    rng = np.random.default_rng(L)
+    q = np.rint(rng.standard_normal((67, L)) * rng.choice([0.5, 2.0, 8.0], (67, 1)) / S).astype(np.int32)
+    q[0], q[1], q[2] = -2 ** 31, 2 ** 31 - 1, np.arange(L) - 2 ** 31
+    for p_max in (255, 127):
+        out, _ = ctx().ibert_softmax_i(dev(q), S, p_max)
+        assert_same(host(out), oracle.softmax(q, S, p_max)[0], f"softmax q_ln2={q_ln2} L={L}")
+    ctx().check()
+
+
 @pytest.mark.parametrize("rows,C", [(3, 8), (5, 17), (64, 768), (33, 1024), (4, 2047), (2, 1), (9, 260), (0, 768),
                                     (7, 1536)])
 @pytest.mark.parametrize("residual", [True, False])
