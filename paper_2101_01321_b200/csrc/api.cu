@@ -591,6 +591,7 @@ int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const
   epi.d_b = (const int32_t*)d_b;
   epi.d_c = (const int32_t*)d_c;
   const LnPath path = linear_ln_path(ctx, M, N, K, epi, k);
+  if (path == LN_LARGE) make_ln_residual_high(&k);
   if (path == LN_TWO && (rc = ensure_workspace(ctx, (size_t)M * N * 2 + 256))) return rc;
   rc = linear_ln(ctx, path, x, w, M, N, K, epi, res, k, (const int32_t*)d_bi, (const int64_t*)d_Bi,
                  static_cast<int16_t*>(ctx->ws), out);
@@ -768,6 +769,7 @@ int ibert_layer_create(ibert_ctx* ctx, const ibert_layer_desc* d, ibert_layer** 
     k->has_res = 1;
     rc = make_ln_residual(S_res, S_sum, k);
     if (rc != IBERT_OK) return;
+    make_ln_residual_high(k);
     std::vector<int32_t> b_i;
     std::vector<int64_t> B_i;
     rc = make_ln_tables(g, be, H, S_o, k, &b_i, &B_i);

@@ -344,8 +344,14 @@ int make_ln_residual(double S_r, double S, LnConsts* k) {
       if (same) { k->res_narrow = 1; k->res_nb = (int32_t)nb; k->res_nc = nc; k->res_nhalf = (int32_t)nhalf; }
     }
   }
-  // high form: the low 16 bits of the operand hold the rounding offset (in units of 2^-16 of r), the multiplier
-  // is the ratio times 2^16; the offset comes from the same intersection of intervals
+  return IBERT_OK;
+}
+
+// High form: the low 16 bits of the operand hold the rounding offset (in units of 2^-16 of r), the multiplier is the
+// ratio times 2^16; the offset comes from the same intersection of intervals.  It is half a unit of the result, so it
+// fits from a ratio of 1/2 on (every ratio tried up to 32, fewer above).  The search takes 2 us, as long as all other
+// constants of a LayerNorm call: for the kernel that reads it (launch_gemm_ln_i8) only.
+void make_ln_residual_high(LnConsts* k) {
   k->res_high = k->res_hm = k->res_hk = 0;
   if (k->c_r >= 8 && k->c_r <= 31) {
     const int64_t base = ((int64_t)k->b_r << 16) >> k->c_r;
@@ -364,7 +370,6 @@ int make_ln_residual(double S_r, double S, LnConsts* k) {
       if (lo <= hi) { k->res_high = 1; k->res_hm = (int32_t)m; k->res_hk = (int32_t)((lo + hi) / 2); }
     }
   }
-  return IBERT_OK;
 }
 
 // dyadic_bits over an array of up to kTableStep values in loops without branches (the compiler vectorizes them): b, c

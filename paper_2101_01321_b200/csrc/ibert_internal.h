@@ -78,7 +78,8 @@ struct LnConsts {
   // the residual rescale in 32-bit arithmetic: (r * res_nb + res_nhalf) >> res_nc with a 24-bit multiplier,
   // offered (res_narrow != 0) only when the host has checked all 256 int8 values against the exact form
   int32_t res_nb, res_nc, res_nhalf, res_narrow;
-  // the same as one multiply-high, ((r << 16) + res_hk) * res_hm >> 32; also checked on all int8 values (res_high != 0)
+  // the same as one multiply-high, ((r << 16) + res_hk) * res_hm >> 32; also checked on all int8 values (res_high != 0;
+  // only make_ln_residual_high sets it)
   int32_t res_hm, res_hk, res_high;
 };
 
@@ -90,6 +91,7 @@ int make_hgelu_consts(double S, double S_out, GeluConsts* k);
 int make_ln_tables(const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
                    std::vector<int32_t>* b_i, std::vector<int64_t>* B_i);
 int make_ln_residual(double S_r, double S, LnConsts* k);
+void make_ln_residual_high(LnConsts* k);      // after it: res_high, where launch_gemm_ln_i8 will run
 // per-output-channel dyadic multipliers of a linear layer; S_out_cols (N entries) or S_out
 // (b, c); `upper`: the upper-word form, when every column has one (*fits)
 int make_linear_tables(double S_x, const double* S_w, int N, const double* S_out_cols, double S_out,
