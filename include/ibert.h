@@ -182,27 +182,30 @@ int ibert_layer_destroy(ibert_layer* layer);
    x: device int8 [M, K]; w: device int8 [N, K] with host scales S_w[N]; bias: device int32 [N] at
    scale S_x*S_w[n], or NULL; res: device int8 [M, N] at host scale S_res; gamma, beta: host
    double [N]; out: device int8 [M, N] at S_out (*S_ret).  The result is bit-identical to
-   ibert_linear_i8(kind 1, S_mid) followed by ibert_layernorm_i.  When N is a multiple of 256 (at
-   most 1024), the constants fit the 32-bit forms and M is large enough for its 128-row tiles to
-   occupy half of the SMs, a single kernel computes it on a cluster of N/256 CTAs per tile and the
-   Q16 tensor never reaches memory; otherwise the two kernels run back to back through the
-   context's workspace, which holds the Q16 tensor as int16.
+   ibert_linear_i8(kind 1, S_mid) followed by ibert_layernorm_i.  The kernels are chosen by size: one kernel on
+   clusters of N/128 CTAs with 16 to 64 rows each while M is one wave of them (N a multiple of 128, at most 1024;
+   K at least 256), one kernel on clusters of N/256 (N = 768 also N/192) CTAs per 128-row tile once those
+   tiles occupy half of the SMs (N a multiple of 256, at most 1024) -- both only if the constants fit the 32-bit
+   forms, and then the Q16 tensor never reaches memory.  Otherwise, and where the GEMM alone needs a fifth fewer rounds
+   of tiles than the clusters, GEMM and LayerNorm run back to back through the context's workspace, which
+   holds the Q16 tensor as int16.
    Errors: as ibert_linear_i8 and ibert_layernorm_i. */
 int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const int8_t* w, const double* S_w,
                               const int32_t* bias, int64_t M, int N, int K, double S_mid,
                               const int8_t* res, double S_res, const double* gamma, const double* beta,
                               double S_out, int8_t* out, double* S_ret);
 
-/* How ibert_linear_layernorm_i8 and ibert_encoder_layer choose between the single cluster kernel and
-   the two-kernel sequence (the results are identical): mode 0 (default) by problem size, 1 the
-   cluster kernel whenever shapes and constants allow it, 2 never.  No counterpart in the paper:
-   a tuning and testing switch.  Returns IBERT_ERR_ARG for another mode. */
+/* How ibert_linear_layernorm_i8 and ibert_encoder_layer choose between the kernels above (the results are identical):
+   mode 0 (default) by problem size, 1 the 128-row cluster kernel whenever shapes and constants allow it (else the two
+   kernels), 2 always the two kernels.  No counterpart in the paper: a tuning and testing switch.  Returns
+   IBERT_ERR_ARG for another mode. */
 int ibert_set_fusion(ibert_ctx* ctx, int mode);
 
-/* How the linear layers (ibert_linear_i8, ibert_linear_gelu_i8, ibert_linear_hgelu_i8 and the GEMMs
-   inside ibert_encoder_layer that are not taken by the cluster kernel above) treat problems with
-   fewer 128 x 128 output tiles than SMs: mode 0 (default) splits K over a cluster of 2 or 4 CTAs
-   per tile when that engages more SMs, 1 never splits, 2 and 4 force that width whenever K > 128.
+/* Which GEMM kernels the linear layers run (ibert_linear_i8, ibert_linear_gelu_i8, ibert_linear_hgelu_i8 and the
+   GEMMs inside ibert_encoder_layer that no cluster kernel above takes): mode 0 (default) by size -- tiles of 128
+   channels x 16 to 128 tokens (96 where the weights are not a layer's own) while they are one wave of CTAs, else tiles
+   of 128 to 256 x 128 to 256; 1 the large tiles only; 2 and 4 split K of every 128 x 128 tile over a cluster of that
+   many CTAs whenever K > 128.  A mode other than 0 also keeps the small-row cluster kernel above out.
    INT32 accumulation is exact, so the results are identical in every mode.  No counterpart in the
    paper: a tuning and testing switch.  Returns IBERT_ERR_ARG for another mode. */
 int ibert_set_split_k(ibert_ctx* ctx, int mode);

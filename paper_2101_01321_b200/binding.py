@@ -190,7 +190,7 @@ class Context:
         _chk(lib().ibert_set_fusion(self.h, mode), "ibert_set_fusion")
 
     def ibert_set_split_k(self, mode: int) -> None:
-        """0: split K of small GEMMs by size (default); 1: never; 2 / 4: force that cluster width."""
+        """0: GEMM kernels by size (default); 1: the large tiles only; 2 / 4: K split over a cluster of that width."""
         _chk(lib().ibert_set_split_k(self.h, mode), "ibert_set_split_k")
 
     def ibert_set_qkv_layout(self, mode: int) -> None:

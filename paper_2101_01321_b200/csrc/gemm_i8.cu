@@ -516,7 +516,6 @@ int launch_gemm_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, 
                    const GemmEpilogue& epi, void* out) {
   if (M == 0) return IBERT_OK;
   {
-    // few output tiles (small batches): split K over a cluster instead of leaving most SMs idle
     if (epi.out_transposed) {
       const bool int8_ok = epi.kind == EPI_INT8 && epi.fast == 1;
       const bool gelu_ok = epi.kind == EPI_GELU && epi.fast != 0 && epi.gelu.fast != 0 && epi.gelu_table && ctx->gelu_table_mode == 0;
@@ -525,11 +524,10 @@ int launch_gemm_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, 
     // one wave of small tiles
     if (ctx->splitk_mode == 0 && !epi.out_transposed && gemm_small_takes(ctx, M, N, K, epi.w_static))
       return launch_gemm_small_i8(ctx, x, w, M, N, K, epi, out);
-    int split = (ctx->splitk_mode == 1 || epi.fast == 2 || epi.out_transposed) ? 1 : gemm_splitk_width(ctx, M, N, K);
-    if ((ctx->splitk_mode == 2 || ctx->splitk_mode == 4) && K > 128 && epi.fast != 2 && !epi.out_transposed &&
+    // K split over a cluster: by request alone (ibert_set_split_k)
+    if (ctx->splitk_mode > 1 && K > 128 && epi.fast != 2 && !epi.out_transposed &&
         ((M + 127) / 128) * ((N + 127) / 128) * ctx->splitk_mode <= 65535)
-      split = ctx->splitk_mode;
-    if (split > 1) return launch_gemm_splitk_i8(ctx, x, w, M, N, K, epi, out, split);
+      return launch_gemm_splitk_i8(ctx, x, w, M, N, K, epi, out, ctx->splitk_mode);
   }
   bool pair, wide;
   tile_shape(ctx, M, N, &pair, &wide);

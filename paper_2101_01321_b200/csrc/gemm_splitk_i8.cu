@@ -12,7 +12,8 @@
 //   3. after a cluster barrier sums, for its own 1/S of the tile's tokens, the partial sums of all
 //      S CTAs through distributed shared memory, applies the epilogue and stores the result,
 // so both the K walk and the epilogue are split S ways.  Integer addition is associative: the
-// result is bit-identical to the unsplit kernel's.
+// result is bit-identical to the unsplit kernel's.  Reached through ibert_set_split_k alone: wherever the
+// split pays by size, the one-wave kernels of gemm_small_i8.cu take the problem.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -250,15 +251,6 @@ int launch_inst(ibert_ctx* ctx, const CUtensorMap& mw, const CUtensorMap& mx, co
 }
 
 }  // namespace
-
-int gemm_splitk_width(const ibert_ctx* ctx, int64_t M, int N, int K) {
-  // Worth it only for a long K walk: the cluster barrier and the exchange of the partial sums cost
-  // about as much as four K blocks of a single CTA.
-  const int64_t tiles = ((M + kTok - 1) / kTok) * ((N + kCh - 1) / kCh);
-  const int k_blocks = (K + kBK - 1) / kBK;
-  if (k_blocks < 12 || tiles * 2 > ctx->num_sms) return 1;
-  return tiles * 4 <= ctx->num_sms ? 4 : 2;
-}
 
 int launch_gemm_splitk_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t M, int N, int K,
                           const GemmEpilogue& epi, void* out, int split) {

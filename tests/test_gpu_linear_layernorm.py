@@ -1,6 +1,7 @@
 """GPU parity (bit-exact) of linear + residual + i-LayerNorm as one operation against the oracle's
-linear layer (Q16 output) followed by its i-LayerNorm (Sec. 3.6, Eq. 16).  Shapes with N a
-multiple of 256 run the single cluster kernel; the others run the two kernels back to back."""
+linear layer (Q16 output) followed by its i-LayerNorm (Sec. 3.6, Eq. 16).  With the fusion forced, shapes with N a
+multiple of 256 run the 128-row cluster kernel and the others the two kernels back to back; by size, few rows run
+the small-row cluster kernel."""
 import numpy as np
 import pytest
 
@@ -136,8 +137,8 @@ def test_linear_layernorm_by_rounds_of_tiles(M, N, K):
     assert_same(host(out), _oracle(*p), f"linear+LN {M}x{N}x{K}")
 
 
-# residual scales from 1/3 to about 1000 times the sum's: the multiply-high form exists for nearly all of the small
-# ratios and not for all of the large ones
+# residual scales from 0.34 to about 1000 times the sum's: the multiply-high form exists for none below 1/2 (its offset
+# is half a unit of the result), for all tried up to 32 and for fewer and fewer above
 @pytest.mark.parametrize("res_ratio", [0.002, 0.011, 0.13, 0.7, 2.9, 5.1, 5.3, 5.5, 5.7, 5.9])
 def test_linear_layernorm_residual_forms(res_ratio):
     M, N, K = 5000, 768, 128

@@ -1,5 +1,5 @@
 """GPU parity (bit-exact) of the split-K cluster GEMM: every epilogue kind, both cluster widths forced,
-ragged M / N / K, K ranges that leave a CTA of the cluster without a block, and the size rule."""
+ragged M / N / K, K ranges that leave a CTA of the cluster without a block, and the unsplit modes."""
 import numpy as np
 import pytest
 
@@ -74,7 +74,7 @@ def test_split_k_generic_dyadic_form(split):
 
 @pytest.mark.parametrize("split", [0, 1], indirect=True)
 def test_size_rule_and_unsplit_agree(split):
-    """Mode 0 picks the width by size (these shapes split), mode 1 never splits: same bits."""
+    """Mode 0 picks the kernel by size (these shapes take one-wave tiles), mode 1 the large tiles: same bits."""
     for M, N, K in ((128, 768, 3072), (1024, 768, 768), (100, 2304, 768)):
         x, w, bias, S_w, S_x, amax = _problem(M, N, K, 5)
         out, _ = ctx().ibert_linear_i8(dev(x), S_x, dev(w), S_w, dev(bias), 1, amax / 20000.0)
