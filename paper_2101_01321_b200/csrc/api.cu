@@ -343,8 +343,8 @@ static int softmax_common(ibert_ctx* ctx, const int32_t* q, double S, int64_t ro
   if (L < 1 || L > 1024) return IBERT_ERR_SHAPE;
   if (rows > 0 && (!q || !out)) return IBERT_ERR_ARG;
   if (!aligned16(q) || !aligned16(out)) return IBERT_ERR_ALIGN;
-  ExpConsts k{};                                    // zeroed: the bytes are hashed below
-  int rc = make_exp_consts(S, p_max, &k);
+  RowExpConsts k{};                                 // zeroed: the bytes are hashed below
+  int rc = make_row_exp_consts(S, p_max, &k);
   if (rc) return rc;
   DeviceGuard guard(ctx->device);
   uint32_t* table = nullptr;
@@ -1143,8 +1143,8 @@ int ibert_encoder_graph_destroy(ibert_graph* g) {
 
 int ibert_selftest_exp_division(double S, int32_t* q_ln2_out) {
   return guarded([&]() -> int {
-  ExpConsts k;
-  int rc = make_exp_consts(S, 255, &k);
+  RowExpConsts k;
+  int rc = make_row_exp_consts(S, 255, &k);
   if (rc) return rc;
   if (q_ln2_out) *q_ln2_out = (int32_t)k.q_ln2;
   for (uint32_t d = 0; d <= k.d_max; ++d) {

@@ -78,6 +78,17 @@ static inline bool dyadic_bits(double m, int32_t* b, int32_t* c) {
 }
 int dyadic(double m, int32_t* b, int32_t* c) { return dyadic_bits(m, b, c) ? IBERT_OK : dyadic_general(m, b, c); }
 
+// A multiplier m and addend with umulhi(D + add, m) = floor(D / q) for every D <= d_top, or m = 0 (q = 0 asks for none)
+static void fold_multiplier(uint64_t q, uint64_t d_top, uint32_t* m, int32_t* add) {
+  *m = 0;
+  *add = 0;
+  if (q == 0) return;
+  const uint64_t up = ((uint64_t(1) << 32) + q - 1) / q, down = (uint64_t(1) << 32) / q;
+  const uint64_t e0 = up * q - (uint64_t(1) << 32), e1 = (uint64_t(1) << 32) - down * q;
+  if (d_top * e0 < (uint64_t(1) << 32)) *m = (uint32_t)up;
+  else if ((d_top + 1) * e1 <= (uint64_t(1) << 32)) { *m = (uint32_t)down; *add = 1; }
+}
+
 // Algorithm 3 constants.  The pre-shift s_in keeps q_b within 15 bits so that
 // (q_p + q_b)^2 + q_c stays below 2^31; the post-shift s_out keeps every
 // exponential below 2^21 so that a row of up to 1024 of them sums in int32.
@@ -143,23 +154,19 @@ int make_exp_consts(double S, int p_max, ExpConsts* k) {
   // D' = bl q: from there on the count is at least bl > log2 of the polynomial, so e = 0; the count is off by
   // at most one there (D' < 2^22), which moves the remainder by at most 16 past [0, q) and the polynomial
   // below 2^(bl + 1) with the count at least bl + 1 when it rounds up.  Needs q_b well above 16: q >= 16.
-  const uint64_t q = k->q_ln2, up = ((uint64_t(1) << 32) + q - 1) / q, down = (uint64_t(1) << 32) / q;
-  const uint64_t e0 = up * q - (uint64_t(1) << 32), e1 = (uint64_t(1) << 32) - down * q;
-  const auto multiplier = [&](uint64_t d_top, uint32_t* m, int32_t* add) {
-    *m = 0;
-    *add = 0;
-    if (d_top * e0 < (uint64_t(1) << 32)) *m = (uint32_t)up;
-    else if ((d_top + 1) * e1 <= (uint64_t(1) << 32)) { *m = (uint32_t)down; *add = 1; }
-  };
-  k->fold_m = 0;
-  k->fold_add = 0;
-  if (q >= 16) multiplier((uint64_t)bl * q, &k->fold_m, &k->fold_add);
-  // The quotient alone, of distances up to 31 q: exactness is needed up to (bl - s_out) q by the same argument, which
-  // every q <= 16787 has; below q = 16 it reaches to 31 q.  (q = 1: floor((d' + 1) (2^32 - 1) / 2^32) = d'.)
-  if (q == 1) { k->row_m = 0xffffffffu; k->row_add = 1; }
-  else multiplier(q < 16 ? (uint64_t)k->d_max : (uint64_t)(bl - k->s_out) * q, &k->row_m, &k->row_add);
-  if (k->row_m == 0) return IBERT_ERR_SCALE_RANGE;            // cannot happen
+  fold_multiplier(k->q_ln2 >= 16 ? k->q_ln2 : 0, (uint64_t)bl * k->q_ln2, &k->fold_m, &k->fold_add);
   return IBERT_OK;
+}
+
+// Exactness is needed up to (bl - s_out) q here, by the argument above; every q <= 16787 has it, and below q = 16 it
+// reaches to 31 q.  (q = 1: floor((d' + 1) (2^32 - 1) / 2^32) = d'.)
+int make_row_exp_consts(double S, int p_max, RowExpConsts* k) {
+  if (int rc = make_exp_consts(S, p_max, k)) return rc;
+  const uint64_t q = k->q_ln2;
+  const int bl = bit_length_u64((uint64_t)((int64_t)k->q_b * k->q_b + k->q_c));
+  if (q == 1) { k->row_m = 0xffffffffu; k->row_add = 1; }
+  else fold_multiplier(q, q < 16 ? (uint64_t)k->d_max : (uint64_t)(bl - k->s_out) * q, &k->row_m, &k->row_add);
+  return k->row_m != 0 ? IBERT_OK : IBERT_ERR_SCALE_RANGE;   // (never 0)
 }
 
 // Algorithm 2 constants plus the multiplier that takes round(g / 256) to int8 at S_out.

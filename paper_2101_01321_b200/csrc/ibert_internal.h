@@ -38,8 +38,12 @@ struct ExpConsts {
   // not available (q_ln2 < 16, and 16716)
   uint32_t fold_m;
   int32_t fold_add;
-  // the quotient alone for distances clamped to d_max (standalone i-softmax): umulhi(d' + row_add, row_m) =
-  // floor(d' / q_ln2) wherever e is not zero, and a count that still shifts everything out beyond.  Every scale has it.
+};
+
+// Standalone i-softmax: the quotient alone, for distances clamped to d_max.  umulhi(d' + row_add, row_m) =
+// floor(d' / q_ln2) wherever e is not zero, and a count that still shifts everything out beyond.  Every scale has it.
+// (A struct of its own: in ExpConsts the two words lengthen the parameters of the attention kernels for nothing.)
+struct RowExpConsts : ExpConsts {
   uint32_t row_m;
   int32_t row_add;
 };
@@ -85,6 +89,7 @@ struct LnConsts {
 
 int dyadic(double m, int32_t* b, int32_t* c);
 int make_exp_consts(double S, int p_max, ExpConsts* k);
+int make_row_exp_consts(double S, int p_max, RowExpConsts* k);
 int make_gelu_consts(double S, double S_out, GeluConsts* k);
 int make_hgelu_consts(double S, double S_out, GeluConsts* k);
 // per-channel multipliers b_i (int32) and addends B_i (int64, rounding constant included)
@@ -157,7 +162,7 @@ int launch_gelu(ibert_ctx* ctx, const int32_t* q, int64_t n, const GeluConsts& k
 // to `ramp_scratch` (65535 int32); and the look-up kernel that uses it
 int launch_gelu_table(ibert_ctx* ctx, const GeluConsts& k, int32_t* ramp_scratch, int8_t* table);
 int launch_gelu_lut(ibert_ctx* ctx, const int32_t* q, int64_t n, const int8_t* table, int8_t* out);
-int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const ExpConsts& k, uint8_t* out,
+int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const RowExpConsts& k, uint8_t* out,
                    const uint32_t* exp_table = nullptr);
 int launch_exp_table(ibert_ctx* ctx, const ExpConsts& k, uint32_t* table);
 // rows of the word table (as int32) and of the position table (token t: position t mod L) gathered

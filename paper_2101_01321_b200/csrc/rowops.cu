@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kThreads) gather_first_rows_kernel(const int8_
 enum { kExpFold = 0, kExpFoldShift = 1, kExpTable = 2 };
 template <int LPR, int VPL, bool FULL, int EXP>
 __global__ void __launch_bounds__(kThreads, VPL > 4 ? 3 : 4) softmax_group_kernel(const int32_t* __restrict__ q, int64_t rows, int L,
-                                                                     ExpConsts k, uint8_t* __restrict__ out,
+                                                                     RowExpConsts k, uint8_t* __restrict__ out,
                                                                      const uint32_t* __restrict__ table) {
   constexpr int kRows = 32 / LPR;
   const int lane = threadIdx.x & 31, li = lane % LPR;
@@ -659,7 +659,7 @@ int launch_exp_table(ibert_ctx* ctx, const ExpConsts& k, uint32_t* table) {
   return check_launch();
 }
 
-int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const ExpConsts& k, uint8_t* out,
+int launch_softmax(ibert_ctx* ctx, const int32_t* q, int64_t rows, int L, const RowExpConsts& k, uint8_t* out,
                    const uint32_t* exp_table) {
   if (rows == 0) return IBERT_OK;
   const bool vec = (L % 4) == 0;
