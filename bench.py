@@ -546,14 +546,14 @@ def run_ours(args):
         fig = figures.get((top, args.config, batch))
         if top == "attention":
             # i-softmax dominates: lane-operations on the ALU pipe per launch (ncu count when a capture of
-            # this workload is committed, else 11 per score element, the count of the config-2 capture)
-            lane_ops = fig["alu"] * 32.0 if fig else 11.0 * computed * cfg.L * cfg.heads
+            # this workload is committed, else 7.8 per score element, the count of the config-2 capture)
+            lane_ops = fig["alu"] * 32.0 if fig else 7.8 * computed * cfg.L * cfg.heads
             ach = lane_ops / (kern[top]["ms_per_launch"] * 1e-3) / 1e12
             roof = {"kernel": top, "bound": "alu", "achieved": ach, "peak": alu_peak,
                     "unit": "Tinstr/s (int32 lane-ops on the ALU pipe)", "frac": ach / alu_peak, "peak_source": alu_source,
                     "algorithmic": lane_ops,
                     "algorithmic_source": "ncu ALU-pipe instructions of the committed capture x 32" if fig else
-                                          "11 ALU-pipe lane-ops per score element (no ncu capture of this workload committed)"}
+                                          "7.8 ALU-pipe lane-ops per score element (no ncu capture of this workload committed)"}
         elif work[top]["ops"]:
             roof = {"kernel": top, "bound": "tensor", "achieved": kern[top]["tops"], "peak": int8_peak,
                     "unit": "TOP/s", "frac": kern[top]["tops"] / int8_peak,
