@@ -1,4 +1,4 @@
-"""How the kernels leave, read from their source: what only shows after a wait has run out cannot be run on a shared GPU."""
+"""How the kernels leave, read from their source: the ways out after a wait has run out are not provoked on a GPU."""
 import re
 from pathlib import Path
 
