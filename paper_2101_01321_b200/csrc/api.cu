@@ -5,6 +5,7 @@
 #include <cstring>
 #include <new>
 
+#include "device_utils.cuh"
 #include "ibert_internal.h"
 
 using namespace ibert;
@@ -1152,14 +1153,14 @@ int ibert_selftest_exp_division(double S, int32_t* q_ln2_out) {
     const uint32_t z = (uint32_t)(wide >> 32) >> k.div_post;
     if (z != d / k.q_ln2) return IBERT_ERR_VALUE_RANGE;
   }
-  if (k.fold_m != 0) {               // quotient and post-shift in one multiply-high: the exponential itself, every d < 2^21
+  if (iexp_takes_folded(k)) {        // quotient and post-shift in one multiply-high: the exponential itself, every d < 2^21
     for (uint32_t d = 0; d < (1u << 21); ++d) {
       const uint32_t dp = d >> k.s_in, z = dp / k.q_ln2;
       const int32_t t = k.q_b - (int32_t)(dp - z * k.q_ln2);
       const uint32_t n = z + (uint32_t)k.s_out, want = n > 31 ? 0u : (uint32_t)(t * t + k.q_c) >> n;
-      const uint32_t D = dp + (uint32_t)k.s_out * k.q_ln2 + (uint32_t)k.fold_add;
-      const uint32_t nf = (uint32_t)(((uint64_t)D * (uint64_t)k.fold_m) >> 32);
-      const int32_t tf = (int32_t)(nf * k.q_ln2) + (k.q_b + k.fold_add - (int32_t)D);
+      const int32_t mx = 1040000 - (int32_t)(d & 0xfffu), w = (mx - (int32_t)d + iexp_folded_offset(k, mx)) >> k.s_in;
+      const uint32_t nf = (uint32_t)((iexp_folded_addend(k) - (int64_t)w * (int64_t)k.fold_m) >> 32);
+      const int32_t tf = (int32_t)(nf * k.q_ln2) + w;
       if ((nf > 31 ? 0u : (uint32_t)(tf * tf + k.q_c) >> nf) != want) return IBERT_ERR_VALUE_RANGE;
     }
   }

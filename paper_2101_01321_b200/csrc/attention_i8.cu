@@ -582,11 +582,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       uint32_t sum = 0;
       if (ok && live) {
         for (int g = 0; g < G; ++g) mx = max(mx, s_max[g * 128 + row]);
-        // one loop per form of the exponential: exp_of turns a score into its exponential.  Bound by the
-        // multiply-add pipe: a multiply-high takes it four clocks, a multiply-add two.  Quotient and post-shift
-        // from one multiply-high, one of the two additions on the ALU pipe and bytes packed by permutes make a
-        // score 11.7 instructions over the three passes instead of 14.7 (probe: 18.7 instead of 21.1 clocks per
-        // warp and scheduler); B = 64, L = 512, 16 heads 262 -> 246 us, B = 128, L = 128, 12 heads 33.1 -> 31.0
+        // one loop per form of the exponential: exp_of turns a score into its exponential.  Bound by the two integer
+        // pipes together: a multiply-high takes the multiply-add pipe four clocks and the ALU pipe two, a multiply-add
+        // the former two, everything else the latter two.  So the shift count comes out of the distance's one term
+        // (iexp_folded) instead of a second, offset one: 8 and 7 clocks per score where it was 8 and 10, with a
+        // pre-shift 8 and 9 where it was 8 and 13.  B x L x heads, us: 64 x 512 x 16 244.7 -> 234.2, 32 x 256 x 16
+        // 37.2 -> 35.7; with a pre-shift 128 x 128 x 12 32.9 -> 29.9, 64 x 384 x 12 143.9 -> 132.8
         auto pass2 = [&](auto exp_of) {
           for (int c0 = c_begin; c0 < c_end; c0 += kW) {
             uint32_t v[kW];
@@ -605,19 +606,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
           }
         };
         const ExpConsts& ek = a.k.e;
-        if (ek.fold_m != 0) {
-          const uint32_t off = (uint32_t)ek.s_out * ek.q_ln2 + (uint32_t)ek.fold_add;
-          const int32_t qb = ek.q_b + ek.fold_add;
-          if (ek.s_in == 0) {
-            const uint32_t mxk = (uint32_t)mx + off;
-            const int32_t wk = qb - (int32_t)mxk;
-            pass2([&](uint32_t v) { return iexp_folded(mxk - v, add_alu((int32_t)v, wk, a.int_min), ek.fold_m, ek.q_ln2, ek.q_c); });
-          } else {
-            pass2([&](uint32_t v) {
-              const uint32_t D = (((uint32_t)mx - v) >> ek.s_in) + off;
-              return iexp_folded(D, qb - (int32_t)D, ek.fold_m, ek.q_ln2, ek.q_c);
-            });
-          }
+        if (iexp_takes_folded(ek)) {
+          const int64_t mk = iexp_folded_addend(ek);
+          const int32_t neg_m = -(int32_t)ek.fold_m, wk = iexp_folded_offset(ek, mx);
+          if (ek.s_in == 0)
+            pass2([&](uint32_t v) { return iexp_folded(add_alu((int32_t)v, wk, a.int_min), mk, neg_m, ek.q_ln2, ek.q_c); });
+          else
+            pass2([&](uint32_t v) { return iexp_folded((int32_t)(v + (uint32_t)wk) >> ek.s_in, mk, neg_m, ek.q_ln2, ek.q_c); });
         } else {
           pass2([&](uint32_t v) { return iexp_dist_wide((uint32_t)mx - v, ek); });
         }

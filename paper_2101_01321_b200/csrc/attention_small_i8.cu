@@ -144,14 +144,12 @@ attention_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   const ExpConsts& ek = a.k.e;
   if (active) {
     const uint32_t mx = (uint32_t)s_max[row];
-    if (ek.fold_m != 0) {
-      const uint32_t off = (uint32_t)ek.s_out * ek.q_ln2 + (uint32_t)ek.fold_add;
-      const int32_t qb = ek.q_b + ek.fold_add;
+    if (iexp_takes_folded(ek)) {
+      const int64_t mk = iexp_folded_addend(ek);
+      const int32_t neg_m = -(int32_t)ek.fold_m, wk = iexp_folded_offset(ek, (int32_t)mx);
 #pragma unroll
-      for (int i = 0; i < CPT; ++i) {
-        const uint32_t D = ((mx - v[i]) >> ek.s_in) + off;
-        v[i] = iexp_folded(D, qb - (int32_t)D, ek.fold_m, ek.q_ln2, ek.q_c);
-      }
+      for (int i = 0; i < CPT; ++i)
+        v[i] = iexp_folded((int32_t)(v[i] + (uint32_t)wk) >> ek.s_in, mk, neg_m, ek.q_ln2, ek.q_c);
     } else {
 #pragma unroll
       for (int i = 0; i < CPT; ++i) v[i] = iexp_dist_wide(mx - v[i], ek);

@@ -192,10 +192,21 @@ __device__ __forceinline__ uint32_t iexp_dist_wide(uint32_t d, const ExpConsts& 
 // fold it): left to itself the compiler puts additions on the multiply-add pipe, which the multiply-highs of
 // i-softmax keep busy for four clocks each
 __device__ __forceinline__ int32_t add_alu(int32_t a, int32_t b, int32_t int_min) { return __viaddmax_s32(a, b, int_min); }
-// The same when quotient and post-shift come from one multiply-high (ExpConsts::fold_m): `D` = pre-shifted
-// distance + s_out q_ln2 + fold_add, `w` = q_b + fold_add - D.
-__device__ __forceinline__ uint32_t iexp_folded(uint32_t D, int32_t w, uint32_t fold_m, uint32_t q_ln2, int32_t q_c) {
-  const uint32_t n = __umulhi(D, fold_m);                                // floor(d / q_ln2) + s_out
+// The same when quotient and post-shift come from one multiply-high (ExpConsts::fold_m), from w = q_b - s_out q_ln2 - d'
+// alone: with the distance offset to D = d' + s_out q_ln2 + fold_add = q_b + fold_add - w, the shift count is the upper
+// word of D fold_m = (q_b + fold_add) fold_m - w fold_m, whose first term is the same for all scores.
+// (a pre-shift above 12 -- score scales below 1e-8 -- would take the offset past 31 bits: iexp_dist_wide serves those)
+__host__ __device__ __forceinline__ bool iexp_takes_folded(const ExpConsts& k) { return k.fold_m != 0 && k.s_in <= 12; }
+__host__ __device__ __forceinline__ int64_t iexp_folded_addend(const ExpConsts& k) {
+  return (int64_t)(k.q_b + k.fold_add) * (int64_t)k.fold_m;
+}
+// w = (score + offset) >> s_in for a row with maximum mx: -(d >> s) = (2^s - 1 - d) >> s
+__host__ __device__ __forceinline__ int32_t iexp_folded_offset(const ExpConsts& k, int32_t mx) {
+  const uint32_t c = (uint32_t)k.q_b - (uint32_t)k.s_out * k.q_ln2;      // below 2^18 in magnitude
+  return (int32_t)(((c + 1u) << k.s_in) - 1u - (uint32_t)mx);
+}
+__device__ __forceinline__ uint32_t iexp_folded(int32_t w, int64_t mk, int32_t neg_m, uint32_t q_ln2, int32_t q_c) {
+  const uint32_t n = (uint32_t)requant_upper_add(w, neg_m, mk);          // floor(d' / q_ln2) + s_out
   const int32_t t = (int32_t)(n * q_ln2) + w;                            // q_b - r
   return shr_clamped((uint32_t)(t * t + q_c), n);
 }

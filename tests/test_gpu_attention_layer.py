@@ -59,6 +59,20 @@ def test_attention_coarse_score_scale(L, S_qk):
     ctx().check()
 
 
+@pytest.mark.parametrize("B,L,heads", [(2, 100, 2), (13, 130, 12)])       # few pairs, many pairs
+@pytest.mark.parametrize("s_in", [0, 1, 2, 12, 13, 20])
+def test_attention_pre_shift_of_the_distance(B, L, heads, s_in):
+    """Score scales whose i-exp argument is shifted by s_in; above 12 the unfolded quotient runs."""
+    S_qk = float(np.sqrt(8.0 * 6e-5 / 2.0 ** s_in))
+    assert oracle.exp_consts(S_qk * S_qk / 8.0)["s_in"] == s_in
+    H = heads * 64
+    rng = np.random.default_rng(s_in)
+    qkv = rng.integers(-127, 128, (B * L, 3 * H)).astype(np.int8)
+    out, _ = ctx().ibert_attention_i8(dev(qkv), B, L, H, heads, S_qk, S_qk, 0.02, 0.004, 255)
+    ctx().check()
+    assert_same(host(out), oracle.attention(qkv, B, L, H, heads, S_qk, S_qk, 0.02, 0.004, 255), "attention pre-shift")
+
+
 def _run_layers(x, params, B, L, fusion=0):
     c = ctx()
     c.ibert_set_fusion(fusion)
