@@ -47,12 +47,12 @@ constexpr int kOutBytes = kEpiWarps * kOutTile;
 constexpr int kResOff = kOutOff + kOutBytes;     // per epilogue warp: 2 x [32 tokens][32 B] of the residual
 constexpr int kCbOff = kResOff + 2 * kOutBytes;  // int2 {multiplier, bias} per channel
 constexpr int kLnOff = kCbOff + kCh * 8;         // int4 {b_i, 0, B_i lo, B_i hi} per channel
-// statistics of a tile: a block of 128 uint64 sums of squares followed by 128 int32 sums
+// statistics of a tile: 128 sums of the squares' low 24 bits, of the rest, and of the values
 constexpr int kStatBytes = kTok * 12;
 constexpr int kLocOff = kLnOff + kCh * 16;       // [3]: this CTA's partial sums, by tile index mod 3
 constexpr int kGatOff = kLocOff + 3 * kStatBytes;   // [2][kMaxCta]: every CTA's partial sums, by tile parity
-constexpr int kParOff = kGatOff + 2 * kMaxCta * kStatBytes;   // [2][128] int4: the token's LnNorm
-constexpr int kBarOff = kParOff + 2 * kTok * 16;
+constexpr int kParOff = kGatOff + 2 * kMaxCta * kStatBytes;   // [512] int4: per epilogue thread its token's LnNorm
+constexpr int kBarOff = kParOff + kEpiThreads * 16;
 constexpr int kAlloc = kBarOff + 512 + 1024;     // + slack to align the base to 1024 bytes
 static_assert(kAlloc <= 227 * 1024, "shared memory budget");
 
@@ -300,8 +300,9 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         }
         ptx::tmem_wait_st();
         uint8_t* loc = s_loc + (it % 3u) * kStatBytes;
-        atomicAdd(reinterpret_cast<unsigned long long*>(loc) + tok, (unsigned long long)s2);
-        atomicAdd(reinterpret_cast<int32_t*>(loc + kTok * 8) + tok, s1);
+        atomicAdd(reinterpret_cast<uint32_t*>(loc) + tok, (uint32_t)s2 & 0xffffffu);
+        atomicAdd(reinterpret_cast<uint32_t*>(loc) + kTok + tok, (uint32_t)(s2 >> 24));
+        atomicAdd(reinterpret_cast<int32_t*>(loc) + 2 * kTok + tok, s1);
       }
       ptx::fence_proxy_async_smem();
       __syncwarp();                                    // the residual buffers are consumed
@@ -323,45 +324,43 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         ptx::bulk_copy_to_cta(ptx::map_to_cta(dst, r), src, kStatBytes, ptx::map_to_cta(bar_stats + 8 * par, r));
       }
     };
-    // mean and inverse standard deviation of the tokens of tile `it` (warps 4..7, one token per
-    // thread); a barrier of all epilogue warps must follow before pass B reads them
+    // mean and inverse standard deviation of this thread's token of tile `it`.  The four warps of a lane quadrant each
+    // do it for themselves: with one of them for all, the other warps wait 2.4 of a tile's 15 thousand clocks for it at a
+    // barrier (32768 x 1024, K = 1024 67.8 -> 66.0 us; 16384 x 768, K = 768 28.4 -> 28.1, K = 3072 36.5 -> 35.9)
     auto params = [&](uint32_t it) {
       const uint32_t par = it & 1u, phase = (it >> 1) & 1u;
-      if (ew >= 4 && ew < 8) {
-        const int tk = e_tid - 128;
-        const int i = par * kTok + tk;
-        if (ok) ok = ptx::mbar_wait_cluster(bar_stats + 8 * par, phase);
-        ok = __all_sync(0xffffffffu, ok);
-        LnNorm norm = ln_norm(0, 1u);
-        if (ok) {
-          int32_t sum = 0;
-          uint64_t sumsq = 0;
-          for (int r = 0; r < n_slices; ++r) {
-            const uint8_t* blk = s_gat + (par * kMaxCta + r) * kStatBytes;
-            sumsq += reinterpret_cast<const unsigned long long*>(blk)[tk];
-            sum += reinterpret_cast<const int32_t*>(blk + kTok * 8)[tk];
-          }
-          // every CTA has this tile's blocks, so each has read the blocks of the tile before:
-          // that tile's own partial sums can be cleared for their next use three tiles on
-          if (it > 0) {
-            uint8_t* old = s_loc + ((it - 1) % 3u) * kStatBytes;
-            reinterpret_cast<unsigned long long*>(old)[tk] = 0;
-            reinterpret_cast<int32_t*>(old + kTok * 8)[tk] = 0;
-          }
-          int32_t mu = sum / C;                        // floor(sum / C)
-          if (sum - mu * C < 0) mu -= 1;
-          const int64_t ss = (int64_t)sumsq - 2 * (int64_t)mu * (int64_t)sum + (int64_t)C * (int64_t)mu * (int64_t)mu;
-          norm = ln_norm(mu, isqrt_of_quotient((uint64_t)ss, (uint32_t)C));
+      if (ok) ok = ptx::mbar_wait_cluster(bar_stats + 8 * par, phase);
+      ok = __all_sync(0xffffffffu, ok);
+      LnNorm norm{0, 0, 0};
+      if (ok) {
+        uint32_t lo = 0, hi = 0;
+        int32_t sum = 0;
+        for (int r = 0; r < n_slices; ++r) {
+          const uint32_t* blk = reinterpret_cast<const uint32_t*>(s_gat + (par * kMaxCta + r) * kStatBytes) + tok;
+          lo += blk[0];
+          hi += blk[kTok];
+          sum += (int32_t)blk[2 * kTok];
         }
-        s_par[i] = make_int4(norm.scale, norm.shift, norm.rho, 0);
+        // every CTA has this tile's blocks, so each has read the blocks of the tile before:
+        // that tile's own partial sums can be cleared for their next use three tiles on
+        if (it > 0 && part == 0) {
+          uint32_t* old = reinterpret_cast<uint32_t*>(s_loc + ((it - 1) % 3u) * kStatBytes) + tok;
+          old[0] = 0;
+          old[kTok] = 0;
+          old[2 * kTok] = 0;
+        }
+        const int32_t mu = ln_mean(sum, C, ln);
+        const uint64_t ss = ((uint64_t)hi << 24) + lo + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum));
+        norm = ln_norm(mu, ln_root(ss, (uint32_t)C, ln.root_k));
       }
+      s_par[e_tid] = make_int4(norm.scale, norm.shift, norm.rho, 0);
     };
     // pass B of tile `it`: normalize, affine + requantize to int8, store; frees the accumulator stage
     auto pass_b = [&](uint32_t it) {
       const uint32_t par = it & 1u;
       const int t0 = (int)tile_of(it) * kTok;
       if (ok) {
-        const int4 mr = s_par[par * kTok + tok];
+        const int4 mr = s_par[e_tid];
         const LnNorm norm{mr.x, mr.y, mr.z};
 #pragma unroll 1
         for (int ci = 0; ci < kPieces * kPerPiece; ++ci) {
@@ -436,7 +435,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             pass_a((uint32_t)(it + 1));
             decide((uint32_t)(it + 1));
           }
-          if (finish || do_a) ptx::named_bar_sync(1, kEpiThreads);
+          if (do_a) ptx::named_bar_sync(1, kEpiThreads);
           if (do_a) exchange((uint32_t)(it + 1));
           if (finish) pass_b((uint32_t)it);
         }

@@ -56,10 +56,6 @@ struct SmallArgs {
   const int32_t* b_i;
   const int64_t* B_i;
   LnConsts ln;
-  // floor(x / N) = umulhi(x, c_magic) >> c_shift for x < 2^29: c_magic = ceil(2^(32 + c_shift) / N) exceeds the
-  // exact quotient by less than N / N, so x times the excess stays below 2^(32 + c_shift) with N < 2^(c_shift + 1)
-  uint32_t c_magic;
-  int c_shift;
 };
 
 struct Tile {
@@ -379,12 +375,12 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   }
 
   // pass 3: mean and I-Sqrt of the variance (sum (v - mu)^2 = sum v^2 - 2 mu sum v + C mu^2 in integers).  One token
-  // per warp: the warp together, a round of the root's search tests 32 candidates -- the shortest chain.  More
+  // per warp: every lane the same, no exchange.  More
   // tokens: a thread per token, because the warp form repeats some 200 instructions for every token and CTA
   // (95 instructions per element at 48 tokens); encoder layer Large B = 7, L = 128 43.0 -> 40.4 us, Base B = 8,
   // L = 77 30.1 -> 29.7.
   const int C = a.N;
-  auto mean_of = [&](int32_t sum) { return (int32_t)(__umulhi((uint32_t)(sum + (C << 18)), a.c_magic) >> a.c_shift) - (1 << 18); };
+  auto mean_of = [&](int32_t sum) { return ln_mean(sum, C, ln); };
   LnNorm one{};
   if constexpr (TPW == 1) {
     uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
@@ -397,7 +393,7 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p1 >> 16) << 16) +
                            ((uint64_t)__reduce_add_sync(0xffffffffu, p2) << 25);
     const int32_t mu = mean_of(sum);
-    one = ln_norm(mu, warp_isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, lane));
+    one = ln_norm(mu, ln_root(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, ln.root_k));
   } else {
     if ((int)threadIdx.x < a.nt) {
       int32_t sum = 0;
@@ -411,7 +407,7 @@ gemm_ln_small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
         sumsq += (uint64_t)p1 + ((uint64_t)p2 << 25);
       }
       const int32_t mu = mean_of(sum);
-      const LnNorm pr = ln_norm(mu, isqrt_of_quotient(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C));
+      const LnNorm pr = ln_norm(mu, ln_root(sumsq + (uint64_t)((int64_t)mu * (int64_t)(C * mu - 2 * sum)), (uint32_t)C, ln.root_k));
       // (the token's own records are consumed: the first one's place takes the result)
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(s_part + threadIdx.x * 16), "r"(pr.scale), "r"(pr.shift), "r"(pr.rho), "r"(0) : "memory");
     }
@@ -587,9 +583,6 @@ int launch_gemm_ln_small_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, in
   if (!gemm_ln_small_supported(ctx, M, H, K, epi, ln)) return IBERT_ERR_ARG;
   const int cl = H / kCh, nt = small_ln_tile_tokens(ctx, M, cl), part_bytes = kMaxCluster * nt * 16;
   SmallArgs a = small_args(ctx, M, H, K, nt, part_bytes, epi, out);
-  while ((2 << a.c_shift) <= H) ++a.c_shift;                 // floor(log2 H); a power of two takes one less
-  if ((1 << a.c_shift) == H) --a.c_shift;
-  a.c_magic = (uint32_t)(((uint64_t(1) << (32 + a.c_shift)) + (uint64_t)H - 1) / (uint64_t)H);
   a.res = res; a.b_i = d_b_i; a.B_i = d_B_i; a.ln = ln;
   CUtensorMap mw, mx;
   if (int rc = operand_maps(&mw, &mx, w, x, M, H, K, nt)) return rc;

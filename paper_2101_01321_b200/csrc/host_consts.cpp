@@ -302,6 +302,11 @@ int make_ln_tables(const double* gamma, const double* beta, int C, double S_out,
     (*B_i)[i] = t - ((double)t > x ? 1 : 0) + half;      // floor; rounding constant folded in
   }
   k->c = c;
+  // with l = ceil(log2 C) and m = floor(2^(30+l) / C) + 1, m C exceeds 2^(30+l) by at most C <= 2^l: exact below 2^30
+  const int l = ceil_log2_u32((uint32_t)C);
+  k->mean_m = (uint32_t)((uint64_t(1) << (30 + l)) / (uint64_t)C + 1);
+  k->mean_sh = l - 2;
+  k->root_k = (uint32_t)std::min(4294967295.0, std::floor(4294967296.0 / std::sqrt((double)C)));
   // Upper-word form: the normalized value (|n| < 2^23) is produced pre-shifted by 32 - c, so
   // the shift must stay within 8 bits and the shifted addends within 62 bits.
   k->out_sh = 32 - c;

@@ -85,6 +85,10 @@ struct LnConsts {
   // the same as one multiply-high, ((r << 16) + res_hk) * res_hm >> 32; also checked on all int8 values (res_high != 0;
   // only make_ln_residual_high sets it)
   int32_t res_hm, res_hk, res_high;
+  // floor(x / C) = umulhi(x, mean_m) >> mean_sh for x < 2^30 (C >= 4), and floor(2^32 / sqrt(C)) for ln_root
+  uint32_t mean_m;
+  int32_t mean_sh;
+  uint32_t root_k;
 };
 
 int dyadic(double m, int32_t* b, int32_t* c);

@@ -149,3 +149,26 @@ def test_linear_layernorm_residual_forms(res_ratio):
                                              gamma, beta, S_out)
     ctx().check()
     assert_same(host(out), _oracle(*p), f"residual at {S_res / S_mid:.3g} times the scale of the sum")
+
+
+@pytest.mark.parametrize("ratio", [1.0, 37.0, 1500.0])          # |v| up to 127, 4699 and 190500
+@pytest.mark.parametrize("M,N,mode", [(9, 256, 0), (130, 768, 0), (130, 768, 1), (257, 1024, 1)])
+def test_variances_at_perfect_squares(M, N, mode, ratio):
+    """Zero projection and rows of +-a: the sum of squares is a^2 C, the largest value of one square root below the next;
+    one element more or less, and rows of a single value or none, sit on either side of a root's step."""
+    rng = np.random.default_rng(N + M)
+    x, w = np.zeros((M, 64), np.int8), rng.integers(-127, 128, (N, 64)).astype(np.int8)
+    a = rng.integers(0, 128, (M, 1))
+    res = np.where(np.arange(N) % 2 == 0, a, -a)
+    res[1::4, 0] = np.maximum(res[1::4, 0] - 1, -127)
+    res[2::4, 1] = np.minimum(res[2::4, 1] + 1, 127)
+    res[3::4] = 0
+    res[3::8, 5] = 1
+    res = res.astype(np.int8)
+    S_w, S_mid, bias = np.full(N, 2e-4), 1e-3, np.zeros(N, np.int32)
+    gamma, beta = 1.0 + 0.1 * rng.standard_normal(N), 0.1 * rng.standard_normal(N)
+    ctx().ibert_set_fusion(mode)
+    out, _ = ctx().ibert_linear_layernorm_i8(dev(x), 0.03, dev(w), S_w, dev(bias), S_mid, dev(res), ratio * S_mid, gamma, beta, 4.5 / 127)
+    ctx().check()
+    want, _ = oracle.layernorm(oracle.linear(x, 0.03, w, S_w, bias, 1, S_mid), S_mid, res, ratio * S_mid, gamma, beta, 4.5 / 127)
+    assert_same(host(out), want, "linear + LayerNorm at perfect squares")
