@@ -89,32 +89,28 @@ inline int gemm_class(int kind, int K) {
 
 namespace ibert {
 
-// Bounds the cache of constant tables: once it holds more than 4096 entries, everything is dropped
-// after the stream has gone idle.  Called at the START of an entry point, before it looks anything
-// up -- a call holds the pointers it got from the cache until its kernels are enqueued, so the
-// cache must never shrink in the middle of one.
+// Bounds the caches of constants: once there are more than 4096 tables, everything is dropped after the stream has
+// gone idle; the constants of operator calls, which point into the tables, go with them or above 1024 entries.
+// Called at the START of an entry point, before it looks anything up -- a call holds the pointers it got from the
+// cache until its kernels are enqueued, so the cache must never shrink in the middle of one.
 int trim_tables(ibert_ctx* ctx) {
+  if (ctx->consts.size() > 1024) ctx->consts.clear();
   if (ctx->tables.size() <= 4096) return IBERT_OK;
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IBERT_ERR_CUDA;
+  ctx->consts.clear();
   for (auto& kv : ctx->tables) cudaFree(kv.second.ptr);
   ctx->tables.clear();
   return IBERT_OK;
 }
 
 int cached_upload(ibert_ctx* ctx, const void* host, size_t bytes, uint64_t tag, void** dev) {
-  const uint64_t key = table_hash(host, bytes, tag * 0x9e3779b97f4a7c15ull + bytes);
-  auto it = ctx->tables.find(key);
-  if (it != ctx->tables.end()) {
-    // the hash only finds the candidate; the bytes decide
+  uint64_t key = table_hash(host, bytes, tag * 0x9e3779b97f4a7c15ull + bytes);
+  // the hash only finds the candidate; the bytes decide, and another table with the same hash lies one key further
+  for (auto it = ctx->tables.find(key); it != ctx->tables.end(); it = ctx->tables.find(++key))
     if (it->second.bytes == bytes && (bytes == 0 || std::memcmp(it->second.host.data(), host, bytes) == 0)) {
       *dev = it->second.ptr;
       return IBERT_OK;
     }
-    // two different tables with one hash: the newer one replaces the older once the stream is idle
-    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IBERT_ERR_CUDA;
-    cudaFree(it->second.ptr);
-    ctx->tables.erase(it);
-  }
   void* d = nullptr;
   if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) { cudaGetLastError(); return IBERT_ERR_NOMEM; }
   if (cudaMemcpyAsync(d, host, bytes, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess) {
@@ -129,6 +125,92 @@ int cached_upload(ibert_ctx* ctx, const void* host, size_t bytes, uint64_t tag, 
   *dev = d;
   return IBERT_OK;
 }
+
+namespace {
+
+// Constants of an operator call by the bytes they follow from: `scalars`, then the arrays.  Deriving them takes 3 to
+// 10 us a call for 768 to 3072 channels and finding their tables again by content as long as comparing the arrays
+// here (0.1 to 0.4 us), so a caller with its own graph pays for them once per layer and not once per call.
+// `derive` fills the entry; nothing is kept when it fails.
+struct Bytes {
+  const void* p;
+  size_t n;
+};
+template <typename Derive>
+int operator_consts(ibert_ctx* ctx, uint64_t tag, const double (&scalars)[5], const Bytes (&arrays)[2],
+                    const OperatorConsts** out, Derive&& derive) {
+  // a sample finds the candidate: the scalars, 32 words of each array
+  uint64_t key = table_hash(scalars, sizeof(scalars), tag);
+  for (const Bytes& a : arrays)
+    for (size_t i = 0, step = std::max<size_t>(a.n / 32, 8); i + 8 <= a.n; i += step) {
+      uint64_t w;
+      std::memcpy(&w, static_cast<const unsigned char*>(a.p) + i, 8);
+      key = (key ^ w) * 0x9e3779b97f4a7c15ull;
+      key ^= key >> 31;
+    }
+  const size_t total = sizeof(scalars) + arrays[0].n + arrays[1].n;
+  for (auto it = ctx->consts.find(key); it != ctx->consts.end(); it = ctx->consts.find(++key)) {
+    const std::vector<unsigned char>& from = it->second.from;
+    if (from.size() == total && std::memcmp(from.data(), scalars, sizeof(scalars)) == 0 &&
+        std::memcmp(from.data() + sizeof(scalars), arrays[0].p, arrays[0].n) == 0 &&
+        (arrays[1].n == 0 || std::memcmp(from.data() + sizeof(scalars) + arrays[0].n, arrays[1].p, arrays[1].n) == 0)) {
+      *out = &it->second;
+      return IBERT_OK;
+    }
+  }
+  OperatorConsts c;
+  if (int rc = derive(&c)) return rc;
+  c.from.resize(total);
+  std::memcpy(c.from.data(), scalars, sizeof(scalars));
+  std::memcpy(c.from.data() + sizeof(scalars), arrays[0].p, arrays[0].n);
+  if (arrays[1].n) std::memcpy(c.from.data() + sizeof(scalars) + arrays[0].n, arrays[1].p, arrays[1].n);
+  *out = &(ctx->consts[key] = std::move(c));
+  return IBERT_OK;
+}
+
+// per-channel requantization of a linear layer (upper_ok: the rest of its epilogue can run in the upper-word form)
+int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S_out, bool upper_ok, GemmEpilogue* epi) {
+  const OperatorConsts* k = nullptr;
+  const double scalars[5] = {S_x, S_out, (double)N, upper_ok ? 1.0 : 0.0, 1.0};
+  const Bytes arrays[2] = {{S_w, sizeof(double) * (size_t)N}, {nullptr, 0}};
+  int rc = operator_consts(ctx, 1, scalars, arrays, &k, [&](OperatorConsts* o) -> int {
+    std::vector<int32_t> b, c, upper;
+    bool fits = false;
+    if (int r = make_linear_tables(S_x, S_w, N, nullptr, S_out, &b, &c, &upper, &fits)) return r;
+    o->fast = upper_ok && fits;
+    if (o->fast) b.swap(upper);
+    if (int r = cached_upload(ctx, b.data(), b.size() * sizeof(int32_t), 21, &o->d_b)) return r;
+    o->d_c = o->d_b;                                    // (the upper-word form has no separate shifts)
+    return o->fast ? IBERT_OK : cached_upload(ctx, c.data(), c.size() * sizeof(int32_t), 22, &o->d_c);
+  });
+  if (rc) return rc;
+  epi->fast = k->fast ? 1 : 0;
+  epi->d_b = static_cast<const int32_t*>(k->d_b);
+  epi->d_c = static_cast<const int32_t*>(k->d_c);
+  return IBERT_OK;
+}
+
+// residual + LayerNorm (S_r: scale of the residual, 0 = none; S: scale of the sum)
+int ln_consts(ibert_ctx* ctx, double S_r, double S, const double* gamma, const double* beta, int C, double S_out,
+              const OperatorConsts** out) {
+  const double scalars[5] = {S_r, S, S_out, (double)C, 2.0};
+  const Bytes arrays[2] = {{gamma, sizeof(double) * (size_t)C}, {beta, sizeof(double) * (size_t)C}};
+  return operator_consts(ctx, 2, scalars, arrays, out, [&](OperatorConsts* o) -> int {
+    o->ln.C = C;
+    o->ln.has_res = S_r != 0.0;
+    if (o->ln.has_res) {
+      if (int r = make_ln_residual(S_r, S, &o->ln)) return r;
+      make_ln_residual_high(&o->ln);
+    }
+    std::vector<int32_t> b_i;
+    std::vector<int64_t> B_i;
+    if (int r = make_ln_tables(gamma, beta, C, S_out, &o->ln, &b_i, &B_i)) return r;
+    if (int r = cached_upload(ctx, b_i.data(), b_i.size() * sizeof(int32_t), 11, &o->d_b)) return r;
+    return cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &o->d_c);
+  });
+}
+
+}  // namespace
 
 }  // namespace ibert
 
@@ -398,30 +480,20 @@ static int layernorm_common(ibert_ctx* ctx, const void* q, bool q_is_i16, double
   if (rows > 0 && (!q || !out)) return IBERT_ERR_ARG;
   if (!aligned16(q) || !aligned16(out) || (r && !aligned16(r))) return IBERT_ERR_ALIGN;
   if (!good_scale(S) || !good_scale(S_out)) return IBERT_ERR_SCALE_RANGE;
-  LnConsts k{};
-  k.C = C;
-  k.has_res = r != nullptr;
-  if (r) {
-    int rc = make_ln_residual(S_r, S, &k);
-    if (rc) return rc;
-  }
-  std::vector<int32_t> b_i;
-  std::vector<int64_t> B_i;
-  int rc = make_ln_tables(gamma, beta, C, S_out, &k, &b_i, &B_i);
-  if (rc) return rc;
+  if (r && !good_scale(S_r)) return IBERT_ERR_SCALE_RANGE;
   DeviceGuard guard(ctx->device);
-  if ((rc = trim_tables(ctx))) return rc;
-  void *d_b = nullptr, *d_B = nullptr;
-  rc = cached_upload(ctx, b_i.data(), b_i.size() * sizeof(int32_t), 11, &d_b);
+  int rc = trim_tables(ctx);
   if (rc) return rc;
-  rc = cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &d_B);
-  if (rc) return rc;
+  const OperatorConsts* k = nullptr;
+  if ((rc = ln_consts(ctx, r ? S_r : 0.0, S, gamma, beta, C, S_out, &k))) return rc;
+  const int32_t* d_b = static_cast<const int32_t*>(k->d_b);
+  const int64_t* d_B = static_cast<const int64_t*>(k->d_c);
   {
     ProfileScope ps(ctx, IBERT_K_LAYERNORM);
     if (q_is_i16)
-      rc = launch_layernorm_i16(ctx, static_cast<const int16_t*>(q), r, rows, k, (const int32_t*)d_b, (const int64_t*)d_B, out);
+      rc = launch_layernorm_i16(ctx, static_cast<const int16_t*>(q), r, rows, k->ln, d_b, d_B, out);
     else
-      rc = launch_layernorm(ctx, static_cast<const int32_t*>(q), r, rows, k, (const int32_t*)d_b, (const int64_t*)d_B, out);
+      rc = launch_layernorm(ctx, static_cast<const int32_t*>(q), r, rows, k->ln, d_b, d_B, out);
   }
   if (rc == IBERT_OK && S_ret) *S_ret = S_out;
   return rc;
@@ -457,7 +529,7 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
   if (!w) return IBERT_ERR_ARG;
   if (!aligned16(x) || !aligned16(w) || !aligned16(out) || (bias && !aligned16(bias))) return IBERT_ERR_ALIGN;
   if (!good_scale(S_x)) return IBERT_ERR_SCALE_RANGE;
-  for (int n = 0; n < N && kind == EPI_RAW; ++n)                  // (the other kinds: make_linear_tables)
+  for (int n = 0; n < N && kind == EPI_RAW; ++n)                  // (the other kinds: linear_consts)
     if (!good_scale(S_w[n])) return IBERT_ERR_SCALE_RANGE;
   GemmEpilogue epi{};
   epi.kind = kind;
@@ -466,10 +538,7 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
   if (int rc = trim_tables(ctx)) return rc;
   if (kind != EPI_RAW) {
     const double S_acc_to = (kind == EPI_GELU || kind == EPI_HGELU) ? S_mid : S_out;
-    std::vector<int32_t> b, c, upper;
-    bool fits = false;
-    int rc = make_linear_tables(S_x, S_w, N, nullptr, S_acc_to, &b, &c, &upper, &fits);
-    if (rc) return rc;
+    int rc = IBERT_OK;
     // The epilogue runs in ONE form: the upper-word form needs the per-channel multipliers AND (for
     // the GELU kinds) the final multiplier to fit it.  The per-channel table is converted only then --
     // the generic epilogue reads the plain (b, c) pairs.
@@ -479,18 +548,10 @@ static int linear_common(ibert_ctx* ctx, const int8_t* x, double S_x, const int8
       if (rc) return rc;
       upper_ok = epi.gelu.fast != 0;
     }
-    epi.fast = (upper_ok && fits) ? 1 : 0;
-    if (epi.fast) b.swap(upper);
+    if ((rc = linear_consts(ctx, S_x, S_w, N, S_acc_to, upper_ok, &epi))) return rc;
     // i-GELU by table (the tile shapes with room for it use it)
     if (kind == EPI_GELU && epi.fast && ctx->gelu_table_mode == 0)
       if ((rc = cached_gelu_table(ctx, epi.gelu, &epi.gelu_table))) return rc;
-    void *d_b = nullptr, *d_c = nullptr;
-    rc = cached_upload(ctx, b.data(), b.size() * sizeof(int32_t), 21, &d_b);
-    if (rc) return rc;
-    d_c = d_b;                                          // (the upper-word form has no separate shifts)
-    if (!epi.fast && (rc = cached_upload(ctx, c.data(), c.size() * sizeof(int32_t), 22, &d_c))) return rc;
-    epi.d_b = (const int32_t*)d_b;
-    epi.d_c = (const int32_t*)d_c;
   }
   int rc;
   {
@@ -566,36 +627,17 @@ int ibert_linear_layernorm_i8(ibert_ctx* ctx, const int8_t* x, double S_x, const
   GemmEpilogue epi{};
   epi.kind = EPI_Q16;
   epi.d_bias = bias;
-  std::vector<int32_t> b, c, upper;
-  bool fits = false;
-  int rc = make_linear_tables(S_x, S_w, N, nullptr, S_mid, &b, &c, &upper, &fits);
-  if (rc) return rc;
-  epi.fast = fits ? 1 : 0;
-  if (fits) b.swap(upper);
-  LnConsts k{};
-  k.C = N;
-  k.has_res = 1;
-  rc = make_ln_residual(S_res, S_mid, &k);
-  if (rc) return rc;
-  std::vector<int32_t> b_i;
-  std::vector<int64_t> B_i;
-  rc = make_ln_tables(gamma, beta, N, S_out, &k, &b_i, &B_i);
-  if (rc) return rc;
+  if (!good_scale(S_res)) return IBERT_ERR_SCALE_RANGE;
   DeviceGuard guard(ctx->device);
-  if ((rc = trim_tables(ctx))) return rc;
-  void *d_b = nullptr, *d_c = nullptr, *d_bi = nullptr, *d_Bi = nullptr;
-  if ((rc = cached_upload(ctx, b.data(), b.size() * sizeof(int32_t), 21, &d_b))) return rc;
-  d_c = d_b;
-  if (!epi.fast && (rc = cached_upload(ctx, c.data(), c.size() * sizeof(int32_t), 22, &d_c))) return rc;
-  if ((rc = cached_upload(ctx, b_i.data(), b_i.size() * sizeof(int32_t), 11, &d_bi))) return rc;
-  if ((rc = cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &d_Bi))) return rc;
-  epi.d_b = (const int32_t*)d_b;
-  epi.d_c = (const int32_t*)d_c;
-  const LnPath path = linear_ln_path(ctx, M, N, K, epi, k);
-  if (path == LN_LARGE) make_ln_residual_high(&k);
+  int rc = trim_tables(ctx);
+  if (rc) return rc;
+  if ((rc = linear_consts(ctx, S_x, S_w, N, S_mid, true, &epi))) return rc;
+  const OperatorConsts* k = nullptr;
+  if ((rc = ln_consts(ctx, S_res, S_mid, gamma, beta, N, S_out, &k))) return rc;
+  const LnPath path = linear_ln_path(ctx, M, N, K, epi, k->ln);
   if (path == LN_TWO && (rc = ensure_workspace(ctx, (size_t)M * N * 2 + 256))) return rc;
-  rc = linear_ln(ctx, path, x, w, M, N, K, epi, res, k, (const int32_t*)d_bi, (const int64_t*)d_Bi,
-                 static_cast<int16_t*>(ctx->ws), out);
+  rc = linear_ln(ctx, path, x, w, M, N, K, epi, res, k->ln, static_cast<const int32_t*>(k->d_b),
+                 static_cast<const int64_t*>(k->d_c), static_cast<int16_t*>(ctx->ws), out);
   if (rc == IBERT_OK && S_ret) *S_ret = S_out;
   return rc;
   });
@@ -965,22 +1007,13 @@ static int embedding_common(ibert_ctx* ctx, const int32_t* ids, int64_t T, int L
   if (T > 0 && (!ids || !out)) return IBERT_ERR_ARG;
   if (!aligned16(word) || !aligned16(pos) || !aligned16(out)) return IBERT_ERR_ALIGN;
   if (!good_scale(S_word) || !good_scale(S_pos) || !good_scale(S_out)) return IBERT_ERR_SCALE_RANGE;
-  LnConsts k{};
-  k.C = H;
-  k.has_res = 1;
-  int rc = make_ln_residual(S_pos, S_word, &k);
+  DeviceGuard guard(ctx->device);
+  int rc = trim_tables(ctx);
   if (rc) return rc;
-  std::vector<int32_t> b_i;
-  std::vector<int64_t> B_i;
-  rc = make_ln_tables(gamma, beta, H, S_out, &k, &b_i, &B_i);
-  if (rc) return rc;
+  const OperatorConsts* k = nullptr;
+  if ((rc = ln_consts(ctx, S_pos, S_word, gamma, beta, H, S_out, &k))) return rc;
   if (S_ret) *S_ret = S_out;
   if (T == 0) return IBERT_OK;
-  DeviceGuard guard(ctx->device);
-  if ((rc = trim_tables(ctx))) return rc;
-  void *d_b = nullptr, *d_B = nullptr;
-  if ((rc = cached_upload(ctx, b_i.data(), b_i.size() * sizeof(int32_t), 11, &d_b))) return rc;
-  if ((rc = cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &d_B))) return rc;
   // gathered rows: q int32 [T, H] (word row) | r int8 [T, H] (position row)
   const size_t q_bytes = ((size_t)T * H * 4 + 255) & ~size_t(255);
   if ((rc = ensure_workspace(ctx, q_bytes + (size_t)T * H + 256))) return rc;
@@ -988,7 +1021,7 @@ static int embedding_common(ibert_ctx* ctx, const int32_t* ids, int64_t T, int L
   int8_t* r = reinterpret_cast<int8_t*>(static_cast<char*>(ctx->ws) + q_bytes);
   if ((rc = launch_embed_gather(ctx, ids, T, L, word, V, pos, H, q, r, cu_seqlens, B))) return rc;
   ProfileScope ps(ctx, IBERT_K_LAYERNORM);
-  return launch_layernorm(ctx, q, r, T, k, (const int32_t*)d_b, (const int64_t*)d_B, out);
+  return launch_layernorm(ctx, q, r, T, k->ln, static_cast<const int32_t*>(k->d_b), static_cast<const int64_t*>(k->d_c), out);
 }
 
 static int classifier_common(ibert_ctx* ctx, const int8_t* x, int B, int L, int H, double S_x, const int8_t* w,

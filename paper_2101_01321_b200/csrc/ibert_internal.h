@@ -116,6 +116,15 @@ struct DeviceTable {
   std::vector<unsigned char> host;   // the bytes that were uploaded: a hit must match them
 };
 
+// The constants of an operator call: device tables (owned by ibert_ctx::tables) and, with LayerNorm, its scalars
+struct OperatorConsts {
+  std::vector<unsigned char> from;   // the scales and per-channel arrays they were derived from: a hit must match them
+  void* d_b = nullptr;
+  void* d_c = nullptr;               // linear: shifts (d_b in the upper-word form); LayerNorm: addends
+  bool fast = false;                 // linear: multipliers in the upper-word form
+  LnConsts ln{};
+};
+
 }  // namespace ibert
 
 // launch-time state the kernels' launchers keep per device (function attributes are per device)
@@ -129,6 +138,8 @@ struct ibert_ctx {
   int64_t l2_bytes = 0;             // size of the L2 cache
   // derived constant tables already on the device, keyed by a hash of their host bytes
   std::map<uint64_t, ibert::DeviceTable> tables;
+  // constants of the single-operator calls, keyed by a hash of a sample of what they are derived from
+  std::map<uint64_t, ibert::OperatorConsts> consts;
   // look-up tables of ibert_gelu_lut_i, keyed by a hash of the GELU constants
   int splitk_mode = 0;     // 0: kernels by size, 1: the large tiles only, 2 / 4: K split over that many CTAs
   std::map<uint64_t, int8_t*> gelu_luts;
