@@ -421,41 +421,46 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
   const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();              // the kernel that wrote qkv has completed
-  // sequence of a work item (items of one sequence are consecutive: its heads)
-  auto seq_of = [&](int item) {
+  // A work item is one head of one sequence, items of one sequence are consecutive.  Padded batches step through them by
+  // a fixed stride, so head and sequence advance by additions: divisions lie on the way from one pair's last barrier to
+  // the next one's score MMAs (128 x 128 x 12 28.1 -> 27.5 us, 128 x 50 x 12 20.2 -> 19.7, 32 x 256 x 16 33.4 -> 32.9; with four
+  // query tiles per pair there is one such step in four: 64 x 512 x 16 221.3 -> 222.9).
+  struct Pair {
+    int head, batch;
+  };
+  const int step_head = (int)gridDim.x % a.heads, step_batch = (int)gridDim.x / a.heads;
+  auto pair_of = [&](int item) {
     const int s0 = item / a.heads;
-    if constexpr (PACKED) return sorted ? (int)s_order[s0] : s0;
-    else return s0;
+    Pair p{item - s0 * a.heads, s0};
+    if constexpr (PACKED) p.batch = sorted ? (int)s_order[s0] : s0;
+    return p;
+  };
+  auto stepped = [&](Pair p) {
+    p.head += step_head;
+    p.batch += step_batch;
+    if (p.head >= a.heads) { p.head -= a.heads; ++p.batch; }
+    return p;
   };
 
   // (packed: the tensor maps see one "batch" of all rows; a sequence starts at row cu[batch], and
   // rows loaded past its end -- the next sequence's, or zero fill past the last row -- are masked)
-  auto load_q = [&](int item, int qt, int buf) {
-    const int head = item % a.heads, batch = seq_of(item);
-    const int row0 = PACKED ? __ldg(a.lens + batch) : 0, zb = PACKED ? 0 : batch;
+  auto load_q = [&](Pair p, int qt, int buf) {
+    const int row0 = PACKED ? __ldg(a.lens + p.batch) : 0, zb = PACKED ? 0 : p.batch;
     ptx::mbar_arrive_expect_tx(bar_q0 + 8 * buf, (uint32_t)slab_bytes);
-    if constexpr (QT) ptx::tma_load_2d(ptx::smem_addr(sQ + buf * slab_bytes), &map_qk, bar_q0 + 8 * buf, batch * a.L + qt * 128, head * kHeadDim);
+    if constexpr (QT) ptx::tma_load_2d(ptx::smem_addr(sQ + buf * slab_bytes), &map_qk, bar_q0 + 8 * buf, p.batch * a.L + qt * 128, p.head * kHeadDim);
     else
-    ptx::tma_load_3d(ptx::smem_addr(sQ + buf * slab_bytes), &map_qk, bar_q0 + 8 * buf, head * kHeadDim, row0 + qt * 128, zb);
+    ptx::tma_load_3d(ptx::smem_addr(sQ + buf * slab_bytes), &map_qk, bar_q0 + 8 * buf, p.head * kHeadDim, row0 + qt * 128, zb);
   };
-  auto load_k = [&](int item) {
-    const int head = item % a.heads, batch = seq_of(item);
-    const int row0 = PACKED ? __ldg(a.lens + batch) : 0, zb = PACKED ? 0 : batch;
-    ptx::mbar_arrive_expect_tx(bar_k, (uint32_t)(a.n_slabs * slab_bytes));
+  // K (part 1) or V (part 2) of a pair
+  auto load_kv = [&](Pair p, int part) {
+    const int row0 = PACKED ? __ldg(a.lens + p.batch) : 0, zb = PACKED ? 0 : p.batch;
+    const uint32_t bar = part == 1 ? bar_k : bar_v;
+    const uint32_t dst = ptx::smem_addr(part == 1 ? sK : sVs);
+    ptx::mbar_arrive_expect_tx(bar, (uint32_t)(a.n_slabs * slab_bytes));
     for (int s = 0; s < a.n_slabs; ++s) {
-      if constexpr (QT) ptx::tma_load_2d(ptx::smem_addr(sK + s * slab_bytes), &map_qk, bar_k, batch * a.L + s * 128, a.H + head * kHeadDim);
+      if constexpr (QT) ptx::tma_load_2d(dst + s * slab_bytes, &map_qk, bar, p.batch * a.L + s * 128, part * a.H + p.head * kHeadDim);
       else
-      ptx::tma_load_3d(ptx::smem_addr(sK + s * slab_bytes), &map_qk, bar_k, a.H + head * kHeadDim, row0 + s * 128, zb);
-    }
-  };
-  auto load_v = [&](int item) {
-    const int head = item % a.heads, batch = seq_of(item);
-    const int row0 = PACKED ? __ldg(a.lens + batch) : 0, zb = PACKED ? 0 : batch;
-    ptx::mbar_arrive_expect_tx(bar_v, (uint32_t)(a.n_slabs * slab_bytes));
-    for (int s = 0; s < a.n_slabs; ++s) {
-      if constexpr (QT) ptx::tma_load_2d(ptx::smem_addr(sVs + s * slab_bytes), &map_qk, bar_v, batch * a.L + s * 128, 2 * a.H + head * kHeadDim);
-      else
-      ptx::tma_load_3d(ptx::smem_addr(sVs + s * slab_bytes), &map_qk, bar_v, 2 * a.H + head * kHeadDim, row0 + s * 128, zb);
+      ptx::tma_load_3d(dst + s * slab_bytes, &map_qk, bar, part * a.H + p.head * kHeadDim, row0 + s * 128, zb);
     }
   };
 
@@ -464,9 +469,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
   int qbuf = 0;
   bool ok = true;
   if (warp == 0 && (int)blockIdx.x < total && ptx::elect_one()) {
-    load_q(blockIdx.x, 0, 0);
-    load_k(blockIdx.x);
-    load_v(blockIdx.x);
+    const Pair p = pair_of((int)blockIdx.x);
+    load_q(p, 0, 0);
+    load_kv(p, 1);
+    load_kv(p, 2);
   }
 
   // Packed batches: sequences differ in length, so after its first (batch, head) pair a CTA draws the
@@ -478,12 +484,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
   int* s_next = reinterpret_cast<int*>(s_tmem + 1);
   int32_t* draw = a.status + 4;
   int next = 0;
-  for (int item = blockIdx.x, iter = 0; item < total && ok; item = next, ++iter) {
-    const int head = item % a.heads, batch = seq_of(item);
+  Pair cur = pair_of(min((int)blockIdx.x, total - 1)), nxt = cur;
+  for (int item = blockIdx.x, iter = 0; item < total && ok; item = next, cur = nxt, ++iter) {
+    const int head = cur.head, batch = cur.batch;
     if constexpr (PACKED) {
       if (tid == 0) s_next[iter & 1] = (int)gridDim.x + atomicAdd(draw, 1);
     } else {
       next = item + gridDim.x;
+      nxt = stepped(cur);
     }
     // valid keys of this sequence (key-padding mask): keys >= n take no part in max or sum and get
     // probability 0; the MMAs and the softmax only cover the 32-column chunks that hold valid keys
@@ -502,6 +510,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       ok = __syncthreads_and(ok);             // the draw of the next pair is visible
       if (!ok) break;
       next = s_next[iter & 1];
+      nxt = pair_of(min(next, total - 1));
     }
     // The operand barriers are waited on by warp 0 alone, which issues the MMAs: it also requests the next operands as
     // soon as the MMAs are done, so a warp that looked late could find the barrier two phases on and never see its
@@ -545,16 +554,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
         ptx::mma_commit(bar_mma);
         // the other Q buffer was read by the previous tile's score MMAs, which have completed
         if (a.q_bufs == 2) {
-          if (!last_tile) load_q(item, qt + 1, qbuf ^ 1);
-          else if (next < total) load_q(next, 0, qbuf ^ 1);
+          if (!last_tile) load_q(cur, qt + 1, qbuf ^ 1);
+          else if (next < total) load_q(nxt, 0, qbuf ^ 1);
         }
       }
       if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_mma, mma_phase));
       mma_phase ^= 1;
       // K is no longer read once the last tile's scores exist: fetch the next pair's K behind the softmax
       if (ok && warp == 0 && last_tile && next < total && ptx::elect_one()) {
-        load_k(next);
-        if (a.q_bufs == 1) load_q(next, 0, 0);      // single tile per pair: Q is as dead as K by now
+        load_kv(nxt, 1);
+        if (a.q_bufs == 1) load_q(nxt, 0, 0);      // single tile per pair: Q is as dead as K by now
       }
 
       // packed: a warp whose 32 query rows all lie past the sequence's end computes nothing (its rows of P
@@ -680,7 +689,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
       }
       ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_mma, mma_phase));
       mma_phase ^= 1;
-      if (ok && warp == 0 && last_tile && next < total && ptx::elect_one()) load_v(next);   // V was read by the MMAs that just completed
+      if (ok && warp == 0 && last_tile && next < total && ptx::elect_one()) load_kv(nxt, 2);   // V was read by the MMAs that just completed
 
       // ---- epilogue: the 64 context values of a row in two halves, taken by column groups 0 and 1
       // (by group 0 alone when there is only one).  Requantized by multiply-adds with a 64-bit addend; as a
