@@ -199,3 +199,32 @@ def test_layernorm_of_row_pairs(C, dtype):
         out, _ = c.ibert_layernorm_i(qd[:rows], S, rd[:rows], S_r, gamma, beta, S_out)
         assert_same(host(out), want[:rows], f"layernorm {rows}x{C}")
     c.check()
+
+
+def test_layernorm_constants_follow_every_element_of_their_arrays():
+    """The constants of a call are found again by a sample of what they derive from: arrays that differ in one element
+    outside it, or in their order, are others; so they are after more scales than are kept."""
+    rng = np.random.default_rng(5)
+    rows, C = 6, 256
+    q = rng.integers(-30000, 30001, (rows, C)).astype(np.int32)
+    r = rng.integers(-127, 128, (rows, C)).astype(np.int8)
+    gamma, beta = 1.0 + 0.1 * rng.standard_normal(C), 0.1 * rng.standard_normal(C)
+    others = []
+    for i in (1, 3, 129, 255):
+        g = gamma.copy()
+        g[i] = 2.0
+        others.append((g, beta))
+        b = beta.copy()
+        b[i] = 0.7
+        others.append((gamma, b))
+    pairs = [(gamma, beta), *others, (beta, gamma), (gamma, beta)]
+    want = [oracle.layernorm(q, 1e-4, r, 0.02, g, b, 0.04)[0] for g, b in pairs]
+    for _ in range(2):
+        for (g, b), w in zip(pairs, want):
+            assert_same(host(ctx().ibert_layernorm_i(dev(q), 1e-4, dev(r), 0.02, g, b, 0.04)[0]), w, "layernorm constants")
+    qd, rd = dev(q), dev(r)
+    for i in range(1100):
+        ctx().ibert_layernorm_i(qd, 1e-4, rd, 0.02, gamma, beta, 0.04 + 1e-5 * (i + 1))
+    for (g, b), w in zip(pairs, want):
+        assert_same(host(ctx().ibert_layernorm_i(qd, 1e-4, rd, 0.02, g, b, 0.04)[0]), w, "layernorm constants")
+    ctx().check()
