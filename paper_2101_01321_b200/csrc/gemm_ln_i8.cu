@@ -154,24 +154,31 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if constexpr (PAIR) { ptx::tmem_alloc_pair(ptx::smem_addr(s_tmem), 2 * kCh); ptx::tmem_relinquish_pair(); }
     else { ptx::tmem_alloc(ptx::smem_addr(s_tmem), 2 * kCh); ptx::tmem_relinquish(); }
   }
-  // statistics start at zero; the per-channel constants are weights, not outputs of the previous
-  // kernel, so they may be read before the grid dependency is resolved
-  for (int i = threadIdx.x; i < 3 * kStatBytes / 4; i += kThreads) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
-  for (int i = threadIdx.x; i < CH; i += kThreads) {
-    s_cb[i] = make_int2(__ldg(args.pb + n0 + i), args.bias ? __ldg(args.bias + n0 + i) : 0);
-    const int64_t B = __ldg(args.B_i + n0 + i);
-    s_ln[i] = make_int4(__ldg(args.b_i + n0 + i), 0, (int32_t)(uint32_t)B, (int32_t)(B >> 32));
-  }
+  // Statistics start at zero; the per-channel constants are weights, not outputs of the previous kernel, so they may be
+  // read before the grid dependency is resolved.  Where a CTA has all the work of its start on the way to the first loads
+  // (H = 768: pairs and 192-channel CTAs) the epilogue warps do it behind the first tile's main loop: 16384 x 768, K = 768
+  // 28.3 -> 27.6 us, K = 3072 36.8 -> 35.9.  With 256-channel CTAs of their own it is slower there: 8192 x 1024 21.3 -> 23.2.
+  constexpr bool kLateConstants = PAIR || CH == 192;
+  auto load_constants = [&](int tid, int step) {
+    for (int i = tid; i < 3 * kStatBytes / 4; i += step) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
+    for (int i = tid; i < CH; i += step) {
+      s_cb[i] = make_int2(__ldg(args.pb + n0 + i), args.bias ? __ldg(args.bias + n0 + i) : 0);
+      const int64_t B = __ldg(args.B_i + n0 + i);
+      s_ln[i] = make_int4(__ldg(args.b_i + n0 + i), 0, (int32_t)(uint32_t)B, (int32_t)(B >> 32));
+    }
+  };
+  if constexpr (!kLateConstants) load_constants(threadIdx.x, kThreads);
   ptx::tc_fence_before_sync();
-  ptx::cluster_sync();                 // barriers and statistics of every CTA are initialised
+  ptx::cluster_sync();                 // barriers of every CTA are initialised
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *s_tmem;
   bool ok = true;
   ptx::grid_dep_launch();
-  ptx::grid_dep_wait();                // x and res come from the previous kernels
+  if constexpr (!kLateConstants) ptx::grid_dep_wait();       // x and res come from the previous kernels
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
+    if constexpr (kLateConstants) ptx::grid_dep_wait();
     if (ptx::elect_one()) {
       uint32_t stage = 0, phase = 0;
       for (uint32_t it = 0; unit_of(it) < n_units && ok; ++it) {
@@ -249,6 +256,11 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const LnConsts ln = args.ln;
     const int C = ln.C;
     const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
+    if constexpr (kLateConstants) {
+      load_constants(e_tid, kEpiThreads);
+      ptx::grid_dep_wait();
+      ptx::named_bar_sync(1, kEpiThreads);
+    }
 
     // residual block of this warp for tile `it` (32 tokens x kWarpCh channels) into its private
     // buffers; rows past T read as zero.  Called by lane 0 once the buffers have been consumed.
