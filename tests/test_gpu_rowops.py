@@ -201,6 +201,27 @@ def test_layernorm_of_row_pairs(C, dtype):
     c.check()
 
 
+@pytest.mark.parametrize("C", [512, 752, 1024])
+def test_layernorm_of_row_pairs_at_perfect_squares(C):
+    """Rows of +-a up to the largest input: the variance is a perfect square, one element more or less puts it on either
+    side of a root's step; means of both signs, on and off a whole number."""
+    rng = np.random.default_rng(C)
+    rows = 4800
+    a = np.where(np.arange(rows) % 5 == 0, 1 << 20, np.rint(2.0 ** rng.uniform(0, 19.9, rows))).astype(np.int64)[:, None]
+    q = np.where(np.arange(C) % 2 == 0, a, -a)
+    q[1::4, 0] -= 1
+    q[2::4, 1] += 1
+    shift = rng.integers(-(1 << 18), 1 << 18, (rows, 1))
+    q[3::7] = (q[3::7] >> 1) + shift[3::7]
+    q[5::11, 3] = 0
+    q = np.clip(q, -(1 << 20), 1 << 20).astype(np.int32)
+    r = np.zeros((rows, C), np.int8)
+    gamma, beta = 1.0 + 0.1 * rng.standard_normal(C), 0.1 * rng.standard_normal(C)
+    out, _ = ctx().ibert_layernorm_i(dev(q), 1e-4, dev(r), 0.02, gamma, beta, 0.04)
+    ctx().check()
+    assert_same(host(out), oracle.layernorm(q, 1e-4, r, 0.02, gamma, beta, 0.04)[0], "layernorm at perfect squares")
+
+
 def test_layernorm_constants_follow_every_element_of_their_arrays():
     """The constants of a call are found again by a sample of what they derive from: arrays that differ in one element
     outside it, or in their order, are others; so they are after more scales than are kept."""
