@@ -237,7 +237,8 @@ __device__ __forceinline__ int32_t ln_normalize(int32_t v, const LnNorm& n) {
 // bits X in [1/4, 1) of ss, from a quadratic start 2.4 % off.  Two steps leave 1.2e-6, so for s < 2^18 the product with X
 // and `root_k` = floor(2^32 / sqrt(C)) is off by at most one, which the exact comparison settles.  (Bit by bit the root
 // took 18 dependent rounds; three Base layers of 8 x 77 86.4 -> 85.0 us with this form, of 1 x 128 58.1 -> 57.8.)
-// Needs ss < 2^60 and C >= 2.  STEPS = 3: s < 2^24.
+// Needs ss < 2^60 and C >= 2.  STEPS = 3: s < 2^24.  (Other sums -- the missing row of an odd row count -- give any
+// value: the shift count, negative from 2^60 on, must then be one that the shift takes.)
 template <int STEPS = 2>
 __device__ __forceinline__ uint32_t ln_root(uint64_t ss, uint32_t C, uint32_t root_k) {
   const int z = __clzll((long long)(ss | 1ull)) & ~1;
@@ -245,7 +246,7 @@ __device__ __forceinline__ uint32_t ln_root(uint64_t ss, uint32_t C, uint32_t ro
   uint32_t r = 0xAAEEF78Fu - __umulhi(x, 0xD24346FDu - __umulhi(x, 0x68DE4A2Du));       // Q30: 2.6708, 3.2854, 1.6386
 #pragma unroll
   for (int i = 0; i < STEPS; ++i) r = __umulhi(r, 0x30000000u - __umulhi(x, __umulhi(r, r))) << 3;
-  const uint32_t s = __umulhi(__umulhi(x, r), root_k) >> ((z >> 1) - 2);
+  const uint32_t s = shr_clamped(__umulhi(__umulhi(x, r), root_k), (uint32_t)((z >> 1) - 2));
   const uint64_t sq = (uint64_t)s * s * C;
   return sq > ss ? s - 1u : (sq + (uint64_t)(2u * s + 1u) * C <= ss ? s + 1u : s);
 }

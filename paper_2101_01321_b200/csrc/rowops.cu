@@ -311,8 +311,8 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     }
     const uint8_t* sq = ring + (size_t)slot * slot_bytes;
     // (an odd row count: the last group has one row, and in place of the other lies whatever was there.  Its
-    // statistics are discarded; all they share with the first row's is the number of rounds of the root search, of
-    // which more than a row needs change nothing)
+    // statistics are discarded, so the sums are unsigned and both square roots take any bits; all that it shares with
+    // the first row is the number of rounds of the root search, of which more than a row needs change nothing)
     int32_t v[R][VPL][4];
     uint32_t rw[R][VPL];
 #pragma unroll
@@ -341,21 +341,22 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     uint64_t s2 = 0;
 #pragma unroll
     for (int h = 0; h < R; ++h) {
-      int32_t t = 0;
+      uint32_t t = 0;
       uint64_t t2 = 0;
 #pragma unroll
       for (int j = 0; j < VPL; ++j)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          v[h][j][i] += (sext_byte(rw[h][j], i) * k.res_nb + k.res_nhalf) >> k.res_nc;   // the residual, rescaled (narrow form)
-          t += v[h][j][i];
+          const int32_t res = (sext_byte(rw[h][j], i) * k.res_nb + k.res_nhalf) >> k.res_nc;   // rescaled (narrow form)
+          v[h][j][i] = (int32_t)((uint32_t)v[h][j][i] + (uint32_t)res);
+          t += (uint32_t)v[h][j][i];
           t2 += (uint64_t)((int64_t)v[h][j][i] * (int64_t)v[h][j][i]);
         }
       t = __reduce_add_sync(0xffffffffu, t);
       // a lane's share is below 2^50 (|v| <= 2^21, at most 64 values): two 25-bit halves reduce as 32-bit sums
       t2 = (uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)t2 & 0x1ffffffu) +
            ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(t2 >> 25)) << 25);
-      if (h == 0 || lane >= 16) { sum = t; s2 = t2; }            // (two rows: the upper half-warp takes the second)
+      if (h == 0 || lane >= 16) { sum = (int32_t)t; s2 = t2; }            // (two rows: the upper half-warp takes the second)
     }
     // mu = floor(sum / C) and I-Sqrt(floor(ss / C)).  Row pairs of more than 256 channels: a product with the reciprocal,
     // off by one at most, and Newton's iteration in every lane, instead of a division and six rounds of votes (16384 x 768
@@ -364,13 +365,13 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     LnNorm own;
     if constexpr (R == 2 && VPL > 2) {
       int32_t mu = __mulhi(sum, (int32_t)k.mean_m) >> k.mean_sh;
-      const int32_t rest = sum - mu * C;
+      const int32_t rest = (int32_t)((uint32_t)sum - (uint32_t)mu * (uint32_t)C);
       mu += rest >= C ? 1 : (rest < 0 ? -1 : 0);
       own = ln_norm(mu, ln_root<3>(s2 + (uint64_t)((int64_t)mu * ((int64_t)C * mu - 2 * (int64_t)sum)), (uint32_t)C, k.root_k));
     } else {
       int32_t mu = sum / C;
       if (sum - mu * C < 0) mu -= 1;
-      const uint64_t ss = (uint64_t)((int64_t)s2 - 2 * (int64_t)mu * (int64_t)sum + (int64_t)C * (int64_t)mu * (int64_t)mu);
+      const uint64_t ss = s2 + (uint64_t)((int64_t)mu * ((int64_t)C * mu - 2 * (int64_t)sum));
       own = ln_norm(mu, warp_isqrt_of_quotient<32 / R>(ss, (uint32_t)C, lane));
     }
     LnNorm norm[R];
