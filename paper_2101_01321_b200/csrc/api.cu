@@ -191,20 +191,23 @@ int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S
 }
 
 // residual + LayerNorm (S_r: scale of the residual, 0 = none; S: scale of the sum)
+int derive_ln(double S_r, double S, const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
+              std::vector<int32_t>* b_i, std::vector<int64_t>* B_i) {
+  k->C = C;
+  k->has_res = S_r != 0.0;
+  if (k->has_res)
+    if (int rc = make_ln_residual(S_r, S, k)) return rc;
+  return make_ln_tables(gamma, beta, C, S_out, k, b_i, B_i);
+}
 int ln_consts(ibert_ctx* ctx, double S_r, double S, const double* gamma, const double* beta, int C, double S_out,
               const OperatorConsts** out) {
   const double scalars[5] = {S_r, S, S_out, (double)C, 2.0};
   const Bytes arrays[2] = {{gamma, sizeof(double) * (size_t)C}, {beta, sizeof(double) * (size_t)C}};
   return operator_consts(ctx, 2, scalars, arrays, out, [&](OperatorConsts* o) -> int {
-    o->ln.C = C;
-    o->ln.has_res = S_r != 0.0;
-    if (o->ln.has_res) {
-      if (int r = make_ln_residual(S_r, S, &o->ln)) return r;
-      make_ln_residual_high(&o->ln);
-    }
     std::vector<int32_t> b_i;
     std::vector<int64_t> B_i;
-    if (int r = make_ln_tables(gamma, beta, C, S_out, &o->ln, &b_i, &B_i)) return r;
+    if (int r = derive_ln(S_r, S, gamma, beta, C, S_out, &o->ln, &b_i, &B_i)) return r;
+    if (o->ln.has_res) make_ln_residual_high(&o->ln);
     if (int r = cached_upload(ctx, b_i.data(), b_i.size() * sizeof(int32_t), 11, &o->d_b)) return r;
     return cached_upload(ctx, B_i.data(), B_i.size() * sizeof(int64_t), 12, &o->d_c);
   });
@@ -1007,13 +1010,20 @@ static int embedding_common(ibert_ctx* ctx, const int32_t* ids, int64_t T, int L
   if (T > 0 && (!ids || !out)) return IBERT_ERR_ARG;
   if (!aligned16(word) || !aligned16(pos) || !aligned16(out)) return IBERT_ERR_ALIGN;
   if (!good_scale(S_word) || !good_scale(S_pos) || !good_scale(S_out)) return IBERT_ERR_SCALE_RANGE;
+  int rc = IBERT_OK;
+  if (T == 0) {                      // nothing to launch: the constants are checked, not uploaded
+    LnConsts ln{};
+    std::vector<int32_t> b_i;
+    std::vector<int64_t> B_i;
+    rc = derive_ln(S_pos, S_word, gamma, beta, H, S_out, &ln, &b_i, &B_i);
+    if (rc == IBERT_OK && S_ret) *S_ret = S_out;
+    return rc;
+  }
   DeviceGuard guard(ctx->device);
-  int rc = trim_tables(ctx);
-  if (rc) return rc;
+  if ((rc = trim_tables(ctx))) return rc;
   const OperatorConsts* k = nullptr;
   if ((rc = ln_consts(ctx, S_pos, S_word, gamma, beta, H, S_out, &k))) return rc;
   if (S_ret) *S_ret = S_out;
-  if (T == 0) return IBERT_OK;
   // gathered rows: q int32 [T, H] (word row) | r int8 [T, H] (position row)
   const size_t q_bytes = ((size_t)T * H * 4 + 255) & ~size_t(255);
   if ((rc = ensure_workspace(ctx, q_bytes + (size_t)T * H + 256))) return rc;

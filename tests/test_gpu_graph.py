@@ -89,3 +89,29 @@ def test_graph_creation_rejects_profiling_and_bad_arguments():
     with pytest.raises(binding.IbertError):
         binding.Graph(d, [layer_d], x_d, 1, 16, out_d)
     layer_d.close()
+
+
+def test_embedding_of_no_tokens_in_a_capture():
+    """Nothing to launch: the call checks its constants and enqueues or allocates nothing, so it may stand in a capture
+    although the context has not met its scales before."""
+    c = ctx()
+    stream = torch.cuda.Stream()
+    own = binding.Context(0, stream)
+    rng = np.random.default_rng(8)
+    word, pos = dev(rng.integers(-127, 128, (16, 64)).astype(np.int8)), dev(rng.integers(-127, 128, (4, 64)).astype(np.int8))
+    ids, out = torch.empty(0, dtype=torch.int32, device="cuda"), torch.empty((0, 64), dtype=torch.int8, device="cuda")
+    gamma, beta = 1.0 + 0.1 * rng.standard_normal(64), 0.1 * rng.standard_normal(64)
+    mark = torch.zeros(1, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        mark += 1
+        assert own.ibert_embedding_i8(ids, 4, word, 0.01, pos, 0.01, gamma, beta, 0.03, out=out)[1] == 0.03
+        mark += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert mark.item() == 2.0
+    with pytest.raises(binding.IbertError):                    # what is refused with tokens is refused without
+        c.ibert_embedding_i8(ids, 4, word, 0.01, pos, 0.01, np.full(64, np.nan), beta, 0.03, out=out)
+    own.check()
+    own.close()
