@@ -123,6 +123,7 @@ struct OperatorConsts {
   void* d_c = nullptr;               // linear: shifts (d_b in the upper-word form); LayerNorm: addends
   bool fast = false;                 // linear: multipliers in the upper-word form
   LnConsts ln{};
+  bool high_known = false;           // ln_consts_high has run
 };
 
 }  // namespace ibert
@@ -165,6 +166,7 @@ namespace ibert {
 // uploads `bytes` of host data once per distinct content; returns the device copy
 int cached_upload(ibert_ctx* ctx, const void* host, size_t bytes, uint64_t tag, void** dev);
 int trim_tables(ibert_ctx* ctx);   // bounds the cache; only at the start of an entry point
+uint64_t table_hash(const void* data, size_t bytes, uint64_t seed);
 
 // ---------------------------------------------------------------------------------------
 // Kernel launchers (each returns an IBERT_* code; all enqueue on ctx->stream)
@@ -218,6 +220,15 @@ struct GemmEpilogue {
   // work in front of it on the stream has finished
   bool w_static = false;
 };
+
+// Constants of operator calls, kept in ctx->consts by the content of what they follow from (S_r: scale of the residual,
+// 0 = none; S: scale of the sum; upper_ok: the rest of the epilogue can run in the upper-word form)
+int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S_out, bool upper_ok, GemmEpilogue* epi);
+int derive_ln(double S_r, double S, const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
+              std::vector<int32_t>* b_i, std::vector<int64_t>* B_i);
+int ln_consts(ibert_ctx* ctx, double S_r, double S, const double* gamma, const double* beta, int C, double S_out,
+              OperatorConsts** out);
+void ln_consts_high(OperatorConsts* k);       // adds LnConsts::res_high, for a call that runs launch_gemm_ln_i8
 
 // Upper-word form of a column set: true if for every n, c[n] >= 1 and b[n] << (32 - c[n]) fits
 // int32; then b is replaced by the shifted multipliers.
