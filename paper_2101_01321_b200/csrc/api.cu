@@ -70,14 +70,14 @@ inline int gemm_class(int kind, int K) {
 namespace ibert {
 
 // Bounds the caches of constants: once there are more than 4096 tables, everything is dropped after the stream has
-// gone idle; the constants of operator calls, which point into the tables, go with them or above 1024 entries.
+// gone idle, and the constants of operator calls, which point into the tables, with them.
 // Called at the START of an entry point, before it looks anything up -- a call holds the pointers it got from the
 // cache until its kernels are enqueued, so the cache must never shrink in the middle of one.
 int trim_tables(ibert_ctx* ctx) {
-  if (ctx->consts.size() > 1024) ctx->consts.clear();
+  trim_consts(ctx);
   if (ctx->tables.size() <= 4096) return IBERT_OK;
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IBERT_ERR_CUDA;
-  ctx->consts.clear();
+  drop_consts(ctx);
   for (auto& kv : ctx->tables) cudaFree(kv.second.ptr);
   ctx->tables.clear();
   return IBERT_OK;

@@ -438,7 +438,8 @@ int make_linear_tables(double S_x, const double* S_w, int N, const double* S_out
   c->resize(N);
   upper->resize(N);
   *fits = true;
-  // (single-operator calls derive these on every call: 3072 channels 30 us with frexp, ldexp and floor per channel)
+  // (single-operator calls derive these whenever their scales are new: 3072 channels 30 us with frexp, ldexp and floor
+  // per channel)
   double m[kTableStep];
   for (int n0 = 0; n0 < N; n0 += kTableStep) {
     const int len = std::min(kTableStep, N - n0);

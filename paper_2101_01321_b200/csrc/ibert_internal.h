@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <map>
+#include <set>
 #include <vector>
 
 #include "../../include/ibert.h"
@@ -124,6 +125,7 @@ struct OperatorConsts {
   bool fast = false;                 // linear: multipliers in the upper-word form
   LnConsts ln{};
   bool high_known = false;           // ln_consts_high has run
+  bool used = false;                 // found again since the last trim_consts
 };
 
 }  // namespace ibert
@@ -141,6 +143,9 @@ struct ibert_ctx {
   std::map<uint64_t, ibert::DeviceTable> tables;
   // constants of the single-operator calls, keyed by a hash of a sample of what they are derived from
   std::map<uint64_t, ibert::OperatorConsts> consts;
+  size_t consts_bytes = 0;
+  std::set<uint64_t> consts_seen;                  // keys met once (bounded)
+  ibert::OperatorConsts consts_once[2];            // constants of a call that has not kept them: linear, LayerNorm
   // look-up tables of ibert_gelu_lut_i, keyed by a hash of the GELU constants
   int splitk_mode = 0;     // 0: kernels by size, 1: the large tiles only, 2 / 4: K split over that many CTAs
   std::map<uint64_t, int8_t*> gelu_luts;
@@ -221,8 +226,11 @@ struct GemmEpilogue {
   bool w_static = false;
 };
 
-// Constants of operator calls, kept in ctx->consts by the content of what they follow from (S_r: scale of the residual,
+// Constants of operator calls, kept in ctx->consts by the content of what they follow from once they have returned; valid
+// until the next call of the same function (S_r: scale of the residual,
 // 0 = none; S: scale of the sum; upper_ok: the rest of the epilogue can run in the upper-word form)
+void trim_consts(ibert_ctx* ctx);             // bounds ctx->consts; only at the start of an entry point
+void drop_consts(ibert_ctx* ctx);
 int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S_out, bool upper_ok, GemmEpilogue* epi);
 int derive_ln(double S_r, double S, const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
               std::vector<int32_t>* b_i, std::vector<int64_t>* B_i);

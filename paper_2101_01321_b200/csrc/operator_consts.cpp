@@ -31,15 +31,16 @@ namespace {
 
 // Constants of an operator call by the bytes they follow from: `scalars`, then the arrays.  Deriving them takes 3 to
 // 10 us a call for 768 to 3072 channels and finding their tables again by content as long as comparing the arrays
-// here (0.1 to 0.4 us), so a caller with its own graph pays for them once per layer and not once per call.
-// `derive` fills the entry; nothing is kept when it fails.
+// here (0.1 to 0.4 us), so a caller with its own graph pays for them twice per layer and not once per call: the first
+// call leaves its key only.  Constants that never return (scales taken from every batch) then cost no copy of their
+// arrays and push nothing out.  `derive` fills the entry; nothing is kept when it fails.
 struct Bytes {
   const void* p;
   size_t n;
 };
 template <typename Derive>
 int operator_consts(ibert_ctx* ctx, uint64_t tag, const double (&scalars)[5], const Bytes (&arrays)[2],
-                    OperatorConsts** out, Derive&& derive) {
+                    OperatorConsts* once, OperatorConsts** out, Derive&& derive) {
   // a sample finds the candidate: the scalars, 32 words of each array
   uint64_t key = table_hash(scalars, sizeof(scalars), tag);
   for (const Bytes& a : arrays)
@@ -49,34 +50,63 @@ int operator_consts(ibert_ctx* ctx, uint64_t tag, const double (&scalars)[5], co
       key = (key ^ w) * 0x9e3779b97f4a7c15ull;
       key ^= key >> 31;
     }
+  const uint64_t sample = key;
   const size_t total = sizeof(scalars) + arrays[0].n + arrays[1].n;
   for (auto it = ctx->consts.find(key); it != ctx->consts.end(); it = ctx->consts.find(++key)) {
     const std::vector<unsigned char>& from = it->second.from;
     if (from.size() == total && std::memcmp(from.data(), scalars, sizeof(scalars)) == 0 &&
         std::memcmp(from.data() + sizeof(scalars), arrays[0].p, arrays[0].n) == 0 &&
         (arrays[1].n == 0 || std::memcmp(from.data() + sizeof(scalars) + arrays[0].n, arrays[1].p, arrays[1].n) == 0)) {
+      it->second.used = true;
       *out = &it->second;
       return IBERT_OK;
     }
   }
   OperatorConsts c;
   if (int rc = derive(&c)) return rc;
+  if (ctx->consts_seen.size() >= 4096) ctx->consts_seen.clear();
+  if (ctx->consts_seen.insert(sample).second) {
+    *once = std::move(c);
+    *out = once;
+    return IBERT_OK;
+  }
+  ctx->consts_seen.erase(sample);
   c.from.resize(total);
   std::memcpy(c.from.data(), scalars, sizeof(scalars));
   std::memcpy(c.from.data() + sizeof(scalars), arrays[0].p, arrays[0].n);
   if (arrays[1].n) std::memcpy(c.from.data() + sizeof(scalars) + arrays[0].n, arrays[1].p, arrays[1].n);
+  ctx->consts_bytes += total;
   *out = &(ctx->consts[key] = std::move(c));
   return IBERT_OK;
 }
 
 }  // namespace
 
-// per-channel requantization of a linear layer (upper_ok: the rest of its epilogue can run in the upper-word form)
+// Above 1024 entries or 16 MB, those that no call has found again since the last time go; all of them if that is not enough.
+void trim_consts(ibert_ctx* ctx) {
+  const auto above = [&] { return ctx->consts.size() > 1024 || ctx->consts_bytes > (size_t(16) << 20); };
+  if (!above()) return;
+  for (auto it = ctx->consts.begin(); it != ctx->consts.end();) {
+    if (it->second.used) {
+      it->second.used = false;
+      ++it;
+    } else {
+      ctx->consts_bytes -= it->second.from.size();
+      it = ctx->consts.erase(it);
+    }
+  }
+  if (above()) drop_consts(ctx);
+}
+void drop_consts(ibert_ctx* ctx) {
+  ctx->consts.clear();
+  ctx->consts_bytes = 0;
+}
+
 int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S_out, bool upper_ok, GemmEpilogue* epi) {
   OperatorConsts* k = nullptr;
   const double scalars[5] = {S_x, S_out, (double)N, upper_ok ? 1.0 : 0.0, 1.0};
   const Bytes arrays[2] = {{S_w, sizeof(double) * (size_t)N}, {nullptr, 0}};
-  int rc = operator_consts(ctx, 1, scalars, arrays, &k, [&](OperatorConsts* o) -> int {
+  int rc = operator_consts(ctx, 1, scalars, arrays, &ctx->consts_once[0], &k, [&](OperatorConsts* o) -> int {
     std::vector<int32_t> b, c, upper;
     bool fits = false;
     if (int r = make_linear_tables(S_x, S_w, N, nullptr, S_out, &b, &c, &upper, &fits)) return r;
@@ -93,7 +123,6 @@ int linear_consts(ibert_ctx* ctx, double S_x, const double* S_w, int N, double S
   return IBERT_OK;
 }
 
-// residual + LayerNorm (S_r: scale of the residual, 0 = none; S: scale of the sum)
 int derive_ln(double S_r, double S, const double* gamma, const double* beta, int C, double S_out, LnConsts* k,
               std::vector<int32_t>* b_i, std::vector<int64_t>* B_i) {
   k->C = C;
@@ -106,7 +135,7 @@ int ln_consts(ibert_ctx* ctx, double S_r, double S, const double* gamma, const d
               OperatorConsts** out) {
   const double scalars[5] = {S_r, S, S_out, (double)C, 2.0};
   const Bytes arrays[2] = {{gamma, sizeof(double) * (size_t)C}, {beta, sizeof(double) * (size_t)C}};
-  return operator_consts(ctx, 2, scalars, arrays, out, [&](OperatorConsts* o) -> int {
+  return operator_consts(ctx, 2, scalars, arrays, &ctx->consts_once[1], out, [&](OperatorConsts* o) -> int {
     std::vector<int32_t> b_i;
     std::vector<int64_t> B_i;
     if (int r = derive_ln(S_r, S, gamma, beta, C, S_out, &o->ln, &b_i, &B_i)) return r;

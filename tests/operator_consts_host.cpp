@@ -51,9 +51,77 @@ static int residual_search() {
   return 0;
 }
 
+// constants that never return leave nothing behind and push nothing out
+static int one_off() {
+  ibert_ctx ctx;
+  for (int call = 0; call < 2; ++call) CHECK(ln(ctx, 0.02, 0.04));
+  CHECK(ctx.consts.size() == 1);
+  for (int i = 0; i < 10000; ++i) {
+    trim_consts(&ctx);
+    CHECK(ln(ctx, 0.02 * (1.0 + 1e-6 * (i + 1)), 0.04));
+    device.clear();
+  }
+  CHECK(ctx.consts.size() == 1 && ctx.consts_seen.size() <= 4096);
+  const int before = uploads;
+  CHECK(ln(ctx, 0.02, 0.04));
+  CHECK(uploads == before);
+  return 0;
+}
+
+// what is in use stays when others pass through in numbers, and the copies of the arrays are bounded
+static int in_use() {
+  ibert_ctx ctx;
+  std::vector<double> S_w(100000, 1e-3);
+  GemmEpilogue e{};
+  for (int call = 0; call < 2; ++call) CHECK(ln(ctx, 0.02, 0.04));
+  for (int i = 0; i < 3000; ++i) {
+    for (int call = 0; call < 2; ++call) {
+      trim_consts(&ctx);
+      const int before = uploads;
+      CHECK(ln(ctx, 0.02, 0.04));
+      CHECK(uploads == before);
+      trim_consts(&ctx);
+      if (i % 10 == 0) CHECK(linear_consts(&ctx, 0.03, S_w.data(), (int)S_w.size(), 0.05 * (1.0 + 1e-5 * i), true, &e) == IBERT_OK);
+      else CHECK(ln(ctx, 0.02, 0.05 * (1.0 + 1e-5 * i)));
+      device.clear();
+    }
+    CHECK(ctx.consts.size() <= 1025);
+    size_t bytes = 0;
+    for (auto& kv : ctx.consts) bytes += kv.second.from.size();
+    CHECK(bytes == ctx.consts_bytes && bytes <= (size_t(16) << 20) + 8 * S_w.size() + 64);
+  }
+  return 0;
+}
+
+// one array element outside the sample, and the form of the rest of the epilogue, make other constants
+static int linear_keys() {
+  ibert_ctx ctx;
+  std::vector<double> S_w(3072, 1e-3), other = S_w;
+  other[1] = 1.5e-3;
+  for (int call = 0; call < 4; ++call) {
+    for (int form = 0; form < 4; ++form) {
+      const std::vector<double>& s = form & 1 ? other : S_w;
+      GemmEpilogue e{};
+      CHECK(linear_consts(&ctx, 0.03, s.data(), 3072, 0.05, (form & 2) != 0, &e) == IBERT_OK);
+      CHECK(e.fast == (form >> 1));
+      int32_t b = 0, c = 0;
+      for (int i : {0, 1, 2, 3071}) {
+        CHECK(dyadic((0.03 * s[i]) / 0.05, &b, &c) == IBERT_OK);
+        if (form & 2) CHECK(e.d_b[i] == (int32_t)((int64_t)b << (32 - c)));
+        else CHECK(e.d_b[i] == b && e.d_c[i] == c);
+      }
+    }
+  }
+  CHECK(ctx.consts.size() == 4);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   for (int i = 0; i < C; ++i) { gamma_[i] = 1.0 + 0.1 * std::sin(i); beta_[i] = 0.1 * std::cos(3 * i); }
   if (argc < 2) return 2;
   if (!std::strcmp(argv[1], "residual_search")) return residual_search();
+  if (!std::strcmp(argv[1], "one_off")) return one_off();
+  if (!std::strcmp(argv[1], "in_use")) return in_use();
+  if (!std::strcmp(argv[1], "linear_keys")) return linear_keys();
   return 2;
 }

@@ -20,7 +20,7 @@ def program(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("check", ["residual_search"])
+@pytest.mark.parametrize("check", ["residual_search", "one_off", "in_use", "linear_keys"])
 def test_operator_constants(program, check):
     r = subprocess.run([program, check], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
