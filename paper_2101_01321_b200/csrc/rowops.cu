@@ -3,6 +3,7 @@
 // 128-bit coalesced loads of the int32 inputs, all arithmetic in registers, packed int8
 // stores.  Rows are owned by one warp and reduced with warp shuffles.
 #include <algorithm>
+#include <type_traits>
 
 #include "device_utils.cuh"
 #include "sm100_ptx.cuh"
@@ -254,6 +255,9 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
                       const int32_t* __restrict__ b_i, const int64_t* __restrict__ B_i, int8_t* __restrict__ out,
                       int32_t* status) {
   extern __shared__ __align__(128) uint8_t ln_smem[];
+  // (row groups of a warp; 32 bits where 64 would spill: int32 pairs of 257 to 768 channels, 16384 x 768 from HBM 18.7 ->
+  // 18.2 us, 32768 x 640 26.8 -> 26.1, 8192 x 768 10.8 -> 11.0; int16 pairs lose 2 % with it, 1024 channels keep their time)
+  using Index = std::conditional_t<R == 2 && (VPL == 4 || VPL == 6) && sizeof(QT) == 4, uint32_t, int64_t>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int C = k.C;
   const uint32_t q_bytes = (uint32_t)C * (uint32_t)sizeof(QT), r_bytes = (uint32_t)C;
@@ -263,9 +267,10 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
   // the per-channel tables, copied once per CTA: every row reads all of them
   int64_t* s_B = reinterpret_cast<int64_t*>(ln_smem + (size_t)(kThreads / 32) * DEPTH * slot_bytes + (kThreads / 32) * DEPTH * 8);
   int32_t* s_b = reinterpret_cast<int32_t*>(s_B + C);
-  const int64_t groups = (rows + R - 1) / R;
-  const int64_t warp_global = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
-  const int64_t warp_count = ((int64_t)gridDim.x * kThreads) >> 5;
+  const Index groups = (Index)((rows + R - 1) / R);
+  const Index warp_global = (Index)(((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5);
+  const Index warp_count = (Index)(((int64_t)gridDim.x * kThreads) >> 5);
+
   for (int i = threadIdx.x; i < C; i += kThreads) {        // constants, not outputs of the previous kernel
     s_b[i] = __ldg(b_i + i);
     s_B[i] = __ldg(B_i + i);
@@ -274,10 +279,10 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
 
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();              // the kernel that produced q (and r) has completed
-  auto issue = [&](int64_t group, int slot) {
+  auto issue = [&](Index group, int slot) {
     const uint32_t bar = ptx::smem_addr(bars + slot);
     const uint32_t dst = ptx::smem_addr(ring + (size_t)slot * slot_bytes);
-    const int64_t row = group * R;
+    const int64_t row = (int64_t)group * R;
     const uint32_t n = (uint32_t)min((int64_t)R, rows - row);
     ptx::mbar_arrive_expect_tx(bar, n * (q_bytes + r_bytes));
     ptx::bulk_load_1d(dst, q + row * C, n * q_bytes, bar);
@@ -287,7 +292,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     for (int s = 0; s < DEPTH; ++s) ptx::mbar_init(ptx::smem_addr(bars + s), 1);
     ptx::fence_mbar_init();
     for (int s = 0; s < DEPTH; ++s) {
-      const int64_t group = warp_global + (int64_t)s * warp_count;
+      const Index group = warp_global + (Index)s * warp_count;
       if (group < groups) issue(group, s);
     }
   }
@@ -295,7 +300,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
 
   int slot = 0;
   uint32_t phase = 0;
-  for (int64_t group = warp_global; group < groups; group += warp_count) {
+  for (Index group = warp_global; group < groups; group += warp_count) {
     const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_addr(bars + slot), phase));
     if (!ok) {
       if (lane == 0) atomicCAS(status, 0, IBERT_ERR_TIMEOUT);
@@ -305,7 +310,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
         int s2 = slot + j;
         uint32_t ph2 = phase;
         if (s2 >= DEPTH) { s2 -= DEPTH; ph2 ^= 1; }
-        if (group + (int64_t)j * warp_count < groups) ptx::mbar_wait(ptx::smem_addr(bars + s2), ph2);
+        if (group + (Index)j * warp_count < groups) ptx::mbar_wait(ptx::smem_addr(bars + s2), ph2);
       }
       break;
     }
@@ -330,7 +335,7 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
       }
     __syncwarp();                                    // every lane has its copy: the slot can be refilled
     if (lane == 0) {
-      const int64_t next = group + (int64_t)DEPTH * warp_count;
+      const Index next = group + (Index)DEPTH * warp_count;
       if (next < groups) issue(next, slot);
     }
     if (++slot == DEPTH) { slot = 0; phase ^= 1; }
@@ -360,8 +365,8 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     }
     // mu = floor(sum / C) and I-Sqrt(floor(ss / C)).  Row pairs of more than 256 channels: a product with the reciprocal,
     // off by one at most, and Newton's iteration in every lane, instead of a division and six rounds of votes (16384 x 768
-    // 14.9 -> 14.5 us with int32, 14.7 -> 14.2 with int16 input, inputs from HBM 18.7 -> 18.7 and 16.6 -> 16.2; 32768 x 512 21.1
-    // -> 20.4; at 256 channels 20000 rows behind each other 9.0 -> 10.3, so those and single rows keep the search)
+    // 14.9 -> 14.3 us with int32, 14.7 -> 14.2 with int16 input, inputs from HBM 18.7 -> 18.2 and 16.6 -> 16.2; 32768 x 512 20.7
+    // -> 20.1; at 256 channels 20000 rows behind each other 9.0 -> 10.3, so those and single rows keep the search)
     LnNorm own;
     if constexpr (R == 2 && VPL > 2) {
       int32_t mu = __mulhi(sum, (int32_t)k.mean_m) >> k.mean_sh;
@@ -379,8 +384,8 @@ layernorm_pipe_kernel(const QT* __restrict__ q, const int8_t* __restrict__ r, in
     for (int h = 0; h < R; ++h)
       norm[h] = R == 1 ? own : LnNorm{__shfl_sync(0xffffffffu, own.scale, 16 * h), __shfl_sync(0xffffffffu, own.shift, 16 * h),
                                       __shfl_sync(0xffffffffu, own.rho, 16 * h)};
-    int8_t* orow = out + group * R * C;
-    const bool second = R == 1 || group * R + 1 < rows;
+    int8_t* orow = out + (int64_t)group * R * C;
+    const bool second = R == 1 || (int64_t)group * R + 1 < rows;
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
       const int col = 4 * (j * 32 + lane);
