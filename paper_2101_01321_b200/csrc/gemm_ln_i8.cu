@@ -75,8 +75,8 @@ struct GemmLnArgs {
 // (instruction-descriptor bit 15; 1 KB from one group of eight K rows to the next).
 // CH: channels per CTA = MMA N, 256 or 192 (single CTAs only; see choose_shape).
 // RH: the residual is rescaled by one multiply-high (LnConsts::res_high) instead of multiply-add, shift and addition
-// (16384 x 768: K = 768 29.4 -> 28.7 us, K = 3072 38.8 -> 38.4; with 192 channels per CTA it spills and loses,
-// 4096 x 768 12.3 -> 12.6).
+// (16384 x 768: K = 768 27.4 -> 26.5 us, K = 3072 34.4 -> 33.8; with 192 channels per CTA it spills and loses,
+// 4096 x 768 12.0 -> 12.2, 24576 x 768 39.9 -> 41.1).
 template <bool PAIR, bool XT, int CH, bool RH>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
@@ -99,7 +99,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   // at a time from TMEM.  48-byte rows keep the staging accesses free of bank conflicts.
   constexpr int kWarpCh = CH / 4;
   constexpr int kRowB = CH == 256 ? 32 : 48;
-  constexpr int kChunk = CH == 256 ? 32 : 16;
+  constexpr int kChunk = CH == 256 && (RH || !PAIR) ? 32 : 16;   // (pairs without RH spill more with 32: 16384 x 768 28.1 -> 27.4 us)
   constexpr int kPieces = kWarpCh / kRowB, kPerPiece = kRowB / kChunk;
   constexpr int kTile = 32 * kRowB;
   // output staging: its own block, or (CH = 192) the space that the smaller operand stages leave
@@ -155,10 +155,11 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     else { ptx::tmem_alloc(ptx::smem_addr(s_tmem), 2 * kCh); ptx::tmem_relinquish(); }
   }
   // Statistics start at zero; the per-channel constants are weights, not outputs of the previous kernel, so they may be
-  // read before the grid dependency is resolved.  Where a CTA has all the work of its start on the way to the first loads
-  // (H = 768: pairs and 192-channel CTAs) the epilogue warps do it behind the first tile's main loop: 16384 x 768, K = 768
-  // 28.3 -> 27.6 us, K = 3072 36.8 -> 35.9.  With 256-channel CTAs of their own it is slower there: 8192 x 1024 21.3 -> 23.2.
-  constexpr bool kLateConstants = PAIR || CH == 192;
+  // read before the grid dependency is resolved.  In CTA pairs the epilogue warps do it behind the first tile's main loop:
+  // 8192 x 256, K = 256 11.0 -> 10.4 us, 8192 x 512, K = 512 13.2 -> 11.9, 16384 x 768, K = 768 27.9 -> 26.5, K = 3072 35.0
+  // -> 34.0.  CTAs of their own do it in front: with 256 channels it is slower behind (8192 x 1024 20.9 -> 22.8), with 192 it
+  // spills (8192 x 768, K = 3072 24.4 -> 24.7).
+  constexpr bool kLateConstants = PAIR;
   auto load_constants = [&](int tid, int step) {
     for (int i = tid; i < 3 * kStatBytes / 4; i += step) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
     for (int i = tid; i < CH; i += step) {
@@ -266,6 +267,8 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     // buffers; rows past T read as zero.  Called by lane 0 once the buffers have been consumed.
     auto issue_res = [&](uint32_t it) {
       const int t0 = (int)tile_of(it) * kTok;
+      constexpr int kUnroll = PAIR || RH || CH == 192 ? kPieces : 1;   // (no RH: fewer spills, 8192 x 1024 22.1 -> 21.0 us)
+#pragma unroll kUnroll
       for (int b = 0; b < kPieces; ++b) {
         ptx::mbar_arrive_expect_tx(my_res + 8 * b, kTile);
         ptx::tma_load_2d(ptx::smem_addr(res0 + b * kTile), &map_res, my_res + 8 * b, n0 + part * kWarpCh + b * kRowB,
@@ -285,11 +288,11 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 #pragma unroll 1
         for (int ci = 0; ci < kPieces * kPerPiece; ++ci) {
           const int col = part * kWarpCh + ci * kChunk;
-          const int piece = kPieces == 1 ? 0 : ci;
+          const int piece = kPieces == 1 ? 0 : ci / kPerPiece, within = kPieces == 1 ? ci : ci % kPerPiece;
           uint32_t v[kChunk];
           ptx::tmem_ld(t_lane + par * kCh + col, v);
           const bool got = __all_sync(0xffffffffu, ptx::mbar_wait(my_res + 8 * piece, it & 1u));   // one fill per tile
-          const uint8_t* rsrc = res0 + lane * kRowB + (kPieces == 1 ? ci * kChunk : ci * kTile);
+          const uint8_t* rsrc = res0 + lane * kRowB + piece * kTile + within * kChunk;
           uint32_t rw[kChunk / 4];
 #pragma unroll
           for (int i = 0; i < kChunk / 16; ++i) {
@@ -377,7 +380,8 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 #pragma unroll 1
         for (int ci = 0; ci < kPieces * kPerPiece; ++ci) {
           const int col = part * kWarpCh + ci * kChunk;
-          const bool first = kPieces > 1 || ci == 0, last = kPieces > 1 || ci == kPerPiece - 1;   // of a store's chunks
+          const int within = kPieces == 1 ? ci : ci % kPerPiece;
+          const bool first = within == 0, last = within == kPerPiece - 1;   // of a store's chunks
           uint32_t v[kChunk];
           ptx::tmem_ld(t_lane + par * kCh + col, v);
           ptx::tmem_wait_ld();
@@ -398,7 +402,7 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             }
             w[i >> 2] = pack4_sat_s8(o[0], o[1], o[2], o[3]);
           }
-          uint8_t* row = stage0 + lane * kRowB + (kPieces == 1 ? ci * kChunk : 0);
+          uint8_t* row = stage0 + lane * kRowB + within * kChunk;
 #pragma unroll
           for (int i = 0; i < kChunk / 16; ++i)
             *reinterpret_cast<uint4*>(row + 16 * i) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);

@@ -151,6 +151,18 @@ def test_linear_layernorm_residual_forms(res_ratio):
     assert_same(host(out), _oracle(*p), f"residual at {S_res / S_mid:.3g} times the scale of the sum")
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 256, 64), (129, 256, 128), (300, 512, 144), (515, 768, 272), (260, 1024, 128)])
+def test_linear_layernorm_residual_below_the_sums_scale(M, N, K):
+    """No multiply-high form: the epilogue in 16 columns at a time for pairs of tiles (and single ones of 256 channels)."""
+    p = _problem(M, N, K, M, 0.002)
+    x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
+    assert S_res < 0.5 * S_mid
+    ctx().ibert_set_fusion(1)
+    out, _ = ctx().ibert_linear_layernorm_i8(dev(x), S_x, dev(w), S_w, dev(bias), S_mid, dev(res), S_res, gamma, beta, S_out)
+    ctx().check()
+    assert_same(host(out), _oracle(*p), f"linear+LN {M}x{N}x{K}")
+
+
 @pytest.mark.parametrize("ratio", [1.0, 37.0, 1500.0])          # |v| up to 127, 4699 and 190500
 @pytest.mark.parametrize("M,N,mode", [(9, 256, 0), (130, 768, 0), (130, 768, 1), (257, 1024, 1)])
 def test_variances_at_perfect_squares(M, N, mode, ratio):

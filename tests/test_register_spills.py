@@ -19,7 +19,7 @@ def _spills(source, tmp_path):
     return {name: int(st) + int(ld) for name, st, ld in found}
 
 
-@pytest.mark.parametrize("source,kernel,allowed", [("rowops.cu", "layernorm_pipe_kernel", 0)])
+@pytest.mark.parametrize("source,kernel,allowed", [("rowops.cu", "layernorm_pipe_kernel", 0), ("gemm_ln_i8.cu", "gemm_ln_kernel", 64)])
 def test_spills(source, kernel, allowed, tmp_path):
     spills = {k: v for k, v in _spills(source, tmp_path).items() if k.startswith(kernel)}
     assert len(spills) > 3
