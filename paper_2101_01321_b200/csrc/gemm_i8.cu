@@ -361,11 +361,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
               if constexpr (FAST) o = clamp_sym(ihgelu_upper(requant_upper_add(a, cur_pb, cur_padd), gk), 127);
               else o = ihgelu_to_int8(requant_add(a, cur_pb, cur_padd, cur_pc, 32767), gk, gelu_half);
             } else if constexpr (KIND == kEpiGeluTable || KIND == kEpiGeluTableT) {
-              // Token-major results take the shared-memory port a byte at a time, so every fourth element is computed on
-              // the integer pipes instead of looked up (16384 x 3072 x 768 37.6 -> 35.5 us, 8192 x 4096 x 1024 28.1 ->
-              // 26.8, 4096 x 3072 x 768 14.4 -> 13.8; Base layer of 20 x 200 68.7 -> 68.1).  With the transposed result the
-              // port is less busy and the look-up alone is the faster form (Base layer of 128 x 128 146.4 / 148.3).
-              if (KIND == kEpiGeluTable && i % 4 == 3) {
+              // Token-major results take the shared-memory port a byte at a time, so in CTA pairs every fourth element is
+              // computed on the integer pipes instead of looked up (16384 x 3072 x 768 36.6 -> 34.8 us, 8192 x 4096 x 1024
+              // 27.3 -> 26.3, 2048 x 3072 x 768 10.7 -> 10.3).  The 128-token tiles of single CTAs are a wave or less, where
+              // eight warps leave the port idle: looked up alone 1010 x 3072 x 768 7.0 us, mixed 7.3.  With the transposed
+              // result the port is less busy and the look-up alone is the faster form (Base layer of 128 x 128 146.4 / 148.3).
+              if (PAIR && KIND == kEpiGeluTable && i % 4 == 3) {
                 o = clamp_sym(igelu_magnitude_upper(requant_upper_add(a, cur_pb, cur_padd), gk, gelu_rnd), 127);
               } else {
                 // |requantized value| < 2^30 (upper word of a product of two int32): the sum cannot wrap
