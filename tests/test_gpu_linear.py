@@ -183,3 +183,27 @@ def test_constant_table_cache_survives_its_own_trimming():
             out, _ = ctx().ibert_linear_i8(xd, 0.03, wd, S_w, bd, 0, 0.05)
             assert_same(host(out), oracle.linear(x, 0.03, w, S_w, bias, 0, 0.05), "odd call")
     ctx().check()
+
+
+def test_linear_constants_follow_every_element_and_the_epilogues_form():
+    """The constants of a call are found again by a sample of its scales: arrays that differ in one element outside it are
+    others, and so are those of a GELU whose final multiplier has no upper-word form and of a Q16 result at its scale."""
+    M, N, K = 24, 768, 128
+    x, w, bias, S_w, S_x, amax = _problem(M, N, K, 21)
+    S_mid = 6.0 / 32767.0
+    S_x = S_x * (6.0 / amax)
+    other = S_w.copy()
+    other[1] *= 1.75
+    other[766] *= 0.5
+    xd, wd, bd = dev(x), dev(w), dev(bias)
+    mids = [oracle.linear(x, S_x, w, s, bias, 1, S_mid) for s in (S_w, other)]
+    tiny = 1e-6                                                # multiplier of 1/2 and more behind the GELU
+    for _ in range(3):                                         # met, kept, found
+        for s, mid in zip((S_w, other), mids):
+            out, _ = ctx().ibert_linear_gelu_i8(xd, S_x, wd, s, bd, S_mid, tiny)
+            assert_same(host(out), oracle.gelu(mid, S_mid, tiny)[0], "generic epilogue")
+            out, _ = ctx().ibert_linear_i8(xd, S_x, wd, s, bd, 1, S_mid)
+            assert_same(host(out), mid, "upper-word epilogue")
+            out, _ = ctx().ibert_linear_gelu_i8(xd, S_x, wd, s, bd, S_mid, 6.0 / 127.0)
+            assert_same(host(out), oracle.gelu(mid, S_mid, 6.0 / 127.0)[0], "upper-word GELU")
+    ctx().check()

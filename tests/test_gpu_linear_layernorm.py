@@ -164,12 +164,16 @@ def test_linear_layernorm_residual_below_the_sums_scale(M, N, K):
 
 
 @pytest.mark.parametrize("ratio", [1.0, 37.0, 1500.0])          # |v| up to 127, 4699 and 190500
-@pytest.mark.parametrize("M,N,mode", [(9, 256, 0), (130, 768, 0), (130, 768, 1), (257, 1024, 1)])
-def test_variances_at_perfect_squares(M, N, mode, ratio):
+# K = 64: two kernels by size, the large-tile cluster kernel when forced; K = 256 by size: the one-wave cluster kernel with
+# 16 tokens per tile (one per warp) and with 32, 48 and 64
+@pytest.mark.parametrize("M,N,mode,K", [(9, 256, 0, 64), (130, 768, 0, 64), (130, 768, 1, 64), (257, 1024, 1, 64),
+                                        (300, 256, 1, 64), (16, 768, 0, 256), (321, 768, 0, 256), (600, 768, 0, 256),
+                                        (900, 768, 0, 256), (1300, 768, 0, 256), (130, 256, 0, 256), (700, 1024, 0, 256)])
+def test_variances_at_perfect_squares(M, N, mode, K, ratio):
     """Zero projection and rows of +-a: the sum of squares is a^2 C, the largest value of one square root below the next;
     one element more or less, and rows of a single value or none, sit on either side of a root's step."""
     rng = np.random.default_rng(N + M)
-    x, w = np.zeros((M, 64), np.int8), rng.integers(-127, 128, (N, 64)).astype(np.int8)
+    x, w = np.zeros((M, K), np.int8), rng.integers(-127, 128, (N, K)).astype(np.int8)
     a = rng.integers(0, 128, (M, 1))
     res = np.where(np.arange(N) % 2 == 0, a, -a)
     res[1::4, 0] = np.maximum(res[1::4, 0] - 1, -127)
