@@ -157,9 +157,10 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   // Statistics start at zero; the per-channel constants are weights, not outputs of the previous kernel, so they may be
   // read before the grid dependency is resolved.  In CTA pairs the epilogue warps do it behind the first tile's main loop:
   // 8192 x 256, K = 256 11.0 -> 10.4 us, 8192 x 512, K = 512 13.2 -> 11.9, 16384 x 768, K = 768 27.9 -> 26.5, K = 3072 35.0
-  // -> 34.0.  CTAs of their own do it in front: with 256 channels it is slower behind (8192 x 1024 20.9 -> 22.8), with 192 it
-  // spills (8192 x 768, K = 3072 24.4 -> 24.7).
-  constexpr bool kLateConstants = PAIR;
+  // -> 34.0.  So do CTAs of 192 channels: a Base model of 32 x 128 778.4 -> 773.8 us, where each layer's constants come from
+  // beyond the SM's caches (on the same layer over and over the spills it brings show, 8192 x 768, K = 3072 24.4 -> 24.7).
+  // With 256-channel CTAs of their own it is slower: 8192 x 1024 20.9 -> 22.8.
+  constexpr bool kLateConstants = PAIR || CH == 192;
   auto load_constants = [&](int tid, int step) {
     for (int i = tid; i < 3 * kStatBytes / 4; i += step) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
     for (int i = tid; i < CH; i += step) {
