@@ -810,8 +810,10 @@ static int encoder_layer_common(ibert_ctx* ctx, const ibert_layer* ly, const int
   // the FFN1 result between its GEMM and the cluster kernel: transposed ([F][T]) where both sides take it
   // (the table epilogue of a CTA-pair sized problem on one side, the fused kernel on the other)
   // (a tensor that no longer fits L2 comes back from HBM, where the fused kernel's channel-major tiles --
-  // 128 rows of 128 bytes, T bytes apart -- read slower than token-major ones: T = 32768, F = 4096, 128 MB,
-  // loses 1.5 % of the step)
+  // 128 rows of 128 bytes, T bytes apart -- read slower than token-major ones.  Stacks of 12 Base and 8 Large layers, us,
+  // token-major / channel-major; inside the rule: Base 4096 tokens 747 / 741, 8192 1163 / 1137, 16384 1804 / 1761, Large 4096
+  // 630 / 621, 8192 984 / 963, 12288 1370 / 1335; beyond half of L2: Base 24576 2669 / 2673, 32768 3430 / 3389, Large 16384
+  // 1786 / 1845, 20480 2198 / 2266, 32768 3668 / 3722)
   const bool g_pays = T >= 4096 && (int64_t)T * F <= ctx->l2_bytes / 2;
   const bool g_t = path2 == LN_LARGE && ctx->qkv_layout_mode != 1 && (g_pays || ctx->qkv_layout_mode == 2) && ly->gelu_table &&
                    ctx->gelu_table_mode == 0 && ly->fast_f1 != 0 && ly->gelu.fast != 0 &&

@@ -423,8 +423,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
   ptx::grid_dep_wait();              // the kernel that wrote qkv has completed
   // A work item is one head of one sequence, items of one sequence are consecutive.  Padded batches step through them by
   // a fixed stride, so head and sequence advance by additions: divisions lie on the way from one pair's last barrier to
-  // the next one's score MMAs (128 x 128 x 12 28.1 -> 27.5 us, 128 x 50 x 12 20.2 -> 19.7, 32 x 256 x 16 33.4 -> 32.9; with four
-  // query tiles per pair there is one such step in four: 64 x 512 x 16 221.3 -> 222.9).
+  // the next one's score MMAs (divided / added, us: 60 x 100 x 12 15.1 / 14.3, 128 x 50 x 12 20.1 / 19.6, 128 x 128 x 12 27.6 /
+  // 27.4, 32 x 256 x 16 33.8 / 32.7, 64 x 512 x 16 223.6 / 222.5).
   struct Pair {
     int head, batch;
   };
@@ -596,8 +596,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
         // pipes together: a multiply-high takes the multiply-add pipe four clocks and the ALU pipe two, a multiply-add
         // the former two, everything else the latter two.  So the shift count comes out of the distance's one term
         // (iexp_folded) instead of a second, offset one: 8 and 7 clocks per score where it was 8 and 10, with a
-        // pre-shift 8 and 9 where it was 8 and 13.  B x L x heads, us: 64 x 512 x 16 244.7 -> 234.2, 32 x 256 x 16
-        // 37.2 -> 35.7; with a pre-shift 128 x 128 x 12 32.9 -> 29.9, 64 x 384 x 12 143.9 -> 132.8
+        // pre-shift 8 and 9 where it was 8 and 13.  With the packing of pass 3 and the carry pairs of the epilogue, B x L x
+        // heads, us: 64 x 512 x 16 243.3 -> 222.4, 32 x 256 x 16 36.9 -> 32.7; with a pre-shift 128 x 128 x 12 32.6 -> 27.2,
+        // 64 x 384 x 12 143.1 -> 124.3
         auto pass2 = [&](auto exp_of) {
           for (int c0 = c_begin; c0 < c_end; c0 += kW) {
             uint32_t v[kW];
@@ -636,7 +637,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
         for (int g = 0; g < G; ++g) sum += s_sum[g * 128 + row];
         const RowDivisor rd = make_row_divisor(max(sum, 1u), a.k.e.p_max);   // sum = 0 only without valid keys
         // (bound by the ALU pipe -- a shift and three quarters of a permute per score beside the multiply-high --, so
-        // one of three packing steps goes to the multiply-add pipe: 64 x 512 x 16 234.6 -> 232.6 us)
+        // one of three packing steps goes to the multiply-add pipe: 64 x 512 x 16 222.4 us, by permutes alone 225.1)
         auto pass3 = [&](auto quotient) {
           for (int c0 = c_begin; c0 < c_end; c0 += kW) {
             uint32_t v[kW];
@@ -693,7 +694,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_qk, const AttnArgs a) {
 
       // ---- epilogue: the 64 context values of a row in two halves, taken by column groups 0 and 1
       // (by group 0 alone when there is only one).  Requantized by multiply-adds with a 64-bit addend; as a
-      // product and a separate rounding bit 29.7 instead of 28.1 us at 128 x 128 x 12, 232.6 instead of 222.5 at 64 x 512 x 16
+      // product and a separate rounding bit 28.9 instead of 27.2 us at 128 x 128 x 12, 230.2 instead of 222.4 at 64 x 512 x 16
       if (ok && grp < 2 && live) {
         ptx::tc_fence_after_sync();
         const int64_t half = rounding_half(a.k.c), half32 = int64_t(1) << 31;

@@ -341,8 +341,9 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       }
     };
     // mean and inverse standard deviation of this thread's token of tile `it`.  The four warps of a lane quadrant each
-    // do it for themselves: with one of them for all, the other warps wait 2.4 of a tile's 15 thousand clocks for it at a
-    // barrier (32768 x 1024, K = 1024 67.8 -> 66.0 us; 16384 x 768, K = 768 28.4 -> 28.1, K = 3072 36.5 -> 35.9)
+    // do it for themselves, which spares a barrier in front of pass B.  With ln_root it is short enough that one of them
+    // for all measures the same: 4096 x 256 10.5 us against 10.4, 8192 x 512 12.1 / 11.9, 16384 x 768 26.6 / 26.7, 32768 x
+    // 768 46.9 / 47.9, 16384 x 1024 35.1 / 35.3
     auto params = [&](uint32_t it) {
       const uint32_t par = it & 1u, phase = (it >> 1) & 1u;
       if (ok) ok = ptx::mbar_wait_cluster(bar_stats + 8 * par, phase);
