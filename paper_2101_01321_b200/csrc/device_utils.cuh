@@ -34,10 +34,16 @@ __device__ __forceinline__ int32_t requant_upper_add(int32_t v, int32_t b2, int6
 }
 
 // The same requantization when the host could pre-shift the multiplier (b2 = b << (32 - c)): (v * b2 + 2^31) >> 32, not
-// yet clamped.  (A product whose upper word is corrected by bit 31 of the lower one issues in the same time alone, but
-// its correction is ALU work, which binds most of the loops around it: i-GELU of 2^24 values 14.2 -> 13.6 us, three
-// Base layers of 1 x 128 59.4 -> 58.1 us, of 8 x 77 88.1 -> 86.4.)
+// yet clamped.  (The form below issues in the same time alone, but its correction is ALU work, which binds most of the
+// loops around it: i-GELU of 2^24 values 14.2 -> 13.6 us, three Base layers of 1 x 128 59.4 -> 58.1 us, of 8 x 77 88.1 ->
+// 86.4.)
 __device__ __forceinline__ int32_t requant_upper(int32_t v, int32_t b2) { return requant_upper_add(v, b2, int64_t(1) << 31); }
+
+// The same as a product whose upper word is corrected by bit 31 of the lower one (a register less).
+__device__ __forceinline__ int32_t requant_upper_product(int32_t v, int32_t b2) {
+  const int64_t t = (int64_t)v * (int64_t)b2;
+  return (int32_t)(t >> 32) + (int32_t)((uint32_t)t >> 31);
+}
 
 // The upper-word requantization for multipliers of 1/2 and more: b 2^(32-c) no longer fits 32 bits,
 // so it is split into w 2^32 + r with r in [-2^31, 2^31) and the product into v w + (v r >> 32).
@@ -148,7 +154,9 @@ __device__ __forceinline__ int32_t epilogue_value(int32_t a, int32_t bias, int32
     if constexpr (FAST) return clamp_sym(requant_upper(a + bias, pb), 127);
     else return requant_add(a, pb, padd, pc, 127);
   } else if constexpr (KIND == EPI_HGELU) {
-    if constexpr (FAST) return clamp_sym(ihgelu_upper(requant_upper(a + bias, pb), gk), 127);
+    // (a register more, 33, would leave a short reduction three CTAs of the one-wave kernel per SM instead of four:
+    // 900 x 1024 x 256 4.0 -> 4.4 us; from K = 384 on the multiply-adds would gain 1 to 2 %)
+    if constexpr (FAST) return clamp_sym(ihgelu_upper(requant_upper_product(a + bias, pb), gk), 127);
     else return ihgelu_to_int8(requant_add(a, pb, padd, pc, 32767), gk, gelu_half);
   } else {
     if constexpr (FAST) return clamp_sym(igelu_magnitude_upper(requant_upper(a + bias, pb), gk, gelu_rnd), 127);
