@@ -75,8 +75,8 @@ int operator_consts(ibert_ctx* ctx, uint64_t tag, const double (&scalars)[5], co
   std::memcpy(c.from.data(), scalars, sizeof(scalars));
   std::memcpy(c.from.data() + sizeof(scalars), arrays[0].p, arrays[0].n);
   if (arrays[1].n) std::memcpy(c.from.data() + sizeof(scalars) + arrays[0].n, arrays[1].p, arrays[1].n);
-  ctx->consts_bytes += total;
   *out = &(ctx->consts[key] = std::move(c));
+  ctx->consts_bytes += total;
   return IBERT_OK;
 }
 

@@ -151,9 +151,11 @@ def test_linear_layernorm_residual_forms(res_ratio):
     assert_same(host(out), _oracle(*p), f"residual at {S_res / S_mid:.3g} times the scale of the sum")
 
 
-@pytest.mark.parametrize("M,N,K", [(1, 256, 64), (129, 256, 128), (300, 512, 144), (515, 768, 272), (260, 1024, 128)])
+@pytest.mark.parametrize("M,N,K", [(1, 256, 64), (129, 256, 128), (300, 512, 144), (515, 768, 272), (260, 1024, 128),
+                                   (20000, 256, 64), (9000, 768, 256), (7000, 1024, 64)])
 def test_linear_layernorm_residual_below_the_sums_scale(M, N, K):
-    """No multiply-high form: the epilogue in 16 columns at a time for pairs of tiles (and single ones of 256 channels)."""
+    """No multiply-high form: the epilogue in 16 columns at a time for pairs of tiles (and single ones of 256 channels);
+    the last three have several tiles per cluster."""
     p = _problem(M, N, K, M, 0.002)
     x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
     assert S_res < 0.5 * S_mid
