@@ -65,6 +65,7 @@ struct GemmLnArgs {
   const int64_t* B_i;      // per channel: LayerNorm output addend
   LnConsts ln;
   int32_t* status;
+  int w_static;            // the bias belongs to a layer (complete before the call)
 };
 
 // PAIR: two CTAs (same 256 channels, adjacent 128-token tiles) share every MMA through
@@ -154,8 +155,8 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if constexpr (PAIR) { ptx::tmem_alloc_pair(ptx::smem_addr(s_tmem), 2 * kCh); ptx::tmem_relinquish_pair(); }
     else { ptx::tmem_alloc(ptx::smem_addr(s_tmem), 2 * kCh); ptx::tmem_relinquish(); }
   }
-  // Statistics start at zero; the per-channel constants are weights, not outputs of the previous kernel, so they may be
-  // read before the grid dependency is resolved.  In CTA pairs the epilogue warps do it behind the first tile's main loop:
+  // Statistics start at zero; the per-channel constants, but for a caller's bias, are no outputs of the previous kernel, so
+  // they may be read before the grid dependency is resolved.  In CTA pairs the epilogue warps do it behind the first tile's main loop:
   // 8192 x 256, K = 256 11.0 -> 10.4 us, 8192 x 512, K = 512 13.2 -> 11.9, 16384 x 768, K = 768 27.9 -> 26.5, K = 3072 35.0
   // -> 34.0.  So do CTAs of 192 channels: a Base model of 32 x 128 778.4 -> 773.8 us, where each layer's constants come from
   // beyond the SM's caches (on the same layer over and over the spills it brings show, 8192 x 768, K = 3072 24.4 -> 24.7).
@@ -164,12 +165,18 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   auto load_constants = [&](int tid, int step) {
     for (int i = tid; i < 3 * kStatBytes / 4; i += step) reinterpret_cast<uint32_t*>(s_loc)[i] = 0;
     for (int i = tid; i < CH; i += step) {
-      s_cb[i] = make_int2(__ldg(args.pb + n0 + i), args.bias ? __ldg(args.bias + n0 + i) : 0);
+      s_cb[i].x = __ldg(args.pb + n0 + i);
       const int64_t B = __ldg(args.B_i + n0 + i);
       s_ln[i] = make_int4(__ldg(args.b_i + n0 + i), 0, (int32_t)(uint32_t)B, (int32_t)(B >> 32));
     }
   };
-  if constexpr (!kLateConstants) load_constants(threadIdx.x, kThreads);
+  auto load_bias = [&](int tid, int step) {
+    for (int i = tid; i < CH; i += step) s_cb[i].y = args.bias ? __ldg(args.bias + n0 + i) : 0;
+  };
+  if constexpr (!kLateConstants) {
+    load_constants(threadIdx.x, kThreads);
+    if (args.w_static) load_bias(threadIdx.x, kThreads);
+  }
   ptx::tc_fence_before_sync();
   ptx::cluster_sync();                 // barriers of every CTA are initialised
   ptx::tc_fence_after_sync();
@@ -261,6 +268,9 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if constexpr (kLateConstants) {
       load_constants(e_tid, kEpiThreads);
       ptx::grid_dep_wait();
+    }
+    if (kLateConstants || !args.w_static) {
+      load_bias(e_tid, kEpiThreads);
       ptx::named_bar_sync(1, kEpiThreads);
     }
 
@@ -593,6 +603,7 @@ int launch_gemm_ln_i8(ibert_ctx* ctx, const int8_t* x, const int8_t* w, int64_t 
   a.pb = epi.d_b; a.bias = epi.d_bias; a.b_i = d_b_i; a.B_i = d_B_i;
   a.ln = ln;
   a.status = ctx->d_status;
+  a.w_static = epi.w_static ? 1 : 0;
   const int64_t t_tiles = (T + kTok - 1) / kTok;
   const Shape shape = choose_shape(ctx, T, H, K).shape;
   const int width = cluster_width(shape, H), n_resident = resident_clusters(ctx, shape, H);

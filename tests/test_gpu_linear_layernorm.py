@@ -4,6 +4,7 @@ multiple of 256 run the 128-row cluster kernel and the others the two kernels ba
 the small-row cluster kernel."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from gpu_util import assert_same, ctx, dev, host
@@ -190,3 +191,22 @@ def test_variances_at_perfect_squares(M, N, mode, K, ratio):
     ctx().check()
     want, _ = oracle.layernorm(oracle.linear(x, 0.03, w, S_w, bias, 1, S_mid), S_mid, res, ratio * S_mid, gamma, beta, 4.5 / 127)
     assert_same(host(out), want, "linear + LayerNorm at perfect squares")
+
+
+@pytest.mark.parametrize("M,N,K", [(700, 512, 64), (600, 768, 64), (600, 1024, 64)])       # pairs, 192 channels per CTA, single CTAs
+def test_linear_layernorm_bias_of_the_kernel_before(M, N, K):
+    """A bias written on the stream directly in front of the call, another one every time."""
+    p = _problem(M, N, K, 31)
+    x, w, bias, res, S_w, S_x, S_mid, S_res, gamma, beta, S_out = p
+    c = ctx()
+    c.ibert_set_fusion(1)
+    xd, wd, rd, bd = dev(x), dev(w), dev(res), dev(bias)
+    own = torch.empty_like(bd)
+    for i in range(12):
+        torch.add(bd, 50000 * i, out=own)
+        out, _ = c.ibert_linear_layernorm_i8(xd, S_x, wd, S_w, own, S_mid, rd, S_res, gamma, beta, S_out)
+        torch.add(bd, -7, out=own)
+        if i % 4 == 3:
+            want = _oracle(x, w, (bias + 50000 * i).astype(np.int32), res, S_w, S_x, S_mid, S_res, gamma, beta, S_out)
+            assert_same(host(out), want, f"bias {i}")
+    c.check()

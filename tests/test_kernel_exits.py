@@ -80,3 +80,20 @@ def test_no_warp_vote_that_an_elected_lane_may_miss(name):
             at = end + cond.end()
             stop = _end_of_block(body, at) if cond.group(2) else body.index(";", at)
             assert stop < end + vote.start(), f"{name}: a vote inside `if ({cond.group(1)})`"
+
+
+def test_a_callers_bias_is_read_behind_the_dependency_wait():
+    """The fused GEMM + LayerNorm kernel starts before its predecessor has finished: constants of the context may be read at
+    once, a bias that comes with the call only where the predecessor's results are visible (layers: w_static)."""
+    lambdas, rest = _lambdas(KERNELS["gemm_ln_kernel"])
+    assert "args.bias" in lambdas["load_bias"] and "args.bias" not in rest
+    assert not any("args.bias" in text for name, text in lambdas.items() if name != "load_bias")
+    calls = [m.start() for m in re.finditer(r"load_bias\(", rest)]
+    assert len(calls) == 2
+    early, late = calls
+    assert rest[:early].rstrip().endswith("if (args.w_static)")
+    epilogue = rest[:late]
+    assert epilogue.count("ptx::grid_dep_wait();") == 3          # every thread (constants in front), producer, epilogue
+    assert re.search(r"if constexpr \(!kLateConstants\) ptx::grid_dep_wait\(\);", epilogue)
+    assert re.search(r"if constexpr \(kLateConstants\) \{\s*load_constants\([^)]*\);\s*ptx::grid_dep_wait\(\);\s*\}\s*if \(kLateConstants "
+                     r"\|\| !args\.w_static\) \{\s*$", epilogue)
